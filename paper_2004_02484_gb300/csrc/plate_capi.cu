@@ -3,26 +3,21 @@
 // points have their temperatures set directly, with input bounds, the log
 // barrier (eq. 8) and the fraction-to-the-boundary step (eq. 11).
 //
-// One iteration is two kernels (three with the red-black upper layer):
-//   k_plate_dir  one CTA per (instance, stage) loads the stage's grid into
-//     shared memory (w = x at the state points, u at the actuator points;
-//     lambda at the state points, zero at the actuators), evaluates K_i
-//     (eq. 9) and its norms, the stage's coefficients, and the lower layer
-//     (eqs. 21-24 with the u-iteration of Sec. 5.2): n_lo pointwise Jacobi
-//     sweeps on F_x and F_x^T over the state points.  It stores the
-//     direction Delta s_i and the stage's largest admissible step under
-//     eq. 11 (a per-instance atomic minimum).  Red-black: half 0 runs the
-//     even stages; half 1 the odd ones, its right-hand side lowered by the
-//     even neighbours' directions (M_L Delta x_{i-1}, M_U Delta lambda_{i+1};
-//     the form of eq. 18).
-//   k_update (stage_driver.cuh)  per (instance, stage): the convergence
-//     decision from ||K(S^k)||_inf (the whole instance's maximum, complete
-//     once every stage's k_plate_dir has run) and otherwise S^{k+1} = S^k -
-//     alpha_max Delta S.
-// The Laplacian of the grid, with the mirrored fictitious points of the
-// zero-Neumann condition (eqs. 2-3) or the zero Dirichlet ring, and its
-// transpose are host-built tables of five (column, weight) entries per
-// point.  Everything is float64.
+// One launch of k_plate_dir is one iteration k (two with the red-black upper
+// layer: half 0 the even stages; half 1 the odd ones, its right-hand side
+// lowered by the even neighbours' directions, M_L Delta x_{i-1} and M_U Delta
+// lambda_{i+1}, the form of eq. 18).  A group of threads per (instance,
+// stage), one or two grid points a thread (w = x at the state points, u at
+// the actuator points; lambda at the state points, zero at the actuators):
+// it forms S^k = S^{k-1} - alpha Delta S^{k-1} (the whole instance's step
+// alpha_max of eq. 11 is known then) for its own stage, and x_{i-1},
+// lambda_{i+1} of the neighbours for itself; evaluates K_i (eq. 9) and its
+// norms, the stage's coefficients, and the lower layer (eqs. 21-24 with the
+// u-iteration of Sec. 5.2): n_lo pointwise Jacobi sweeps on F_x and F_x^T
+// over the state points; stores Delta s_i and the stage's largest admissible
+// step (a per-instance atomic minimum).
+// The Laplacian of the grid has the mirrored fictitious points of the
+// zero-Neumann condition (eqs. 2-3) or the zero Dirichlet ring.
 #include <new>
 
 #include "../../include/nmpc_plate.h"
@@ -30,7 +25,6 @@
 
 namespace plate_dev {
 
-using stage_drv::ELL;
 using stage_drv::Ctl;
 using stage_drv::Iter;
 using stage_drv::Layout;
@@ -40,37 +34,23 @@ constexpr int MAX_NU = 64;
 // Per instance: the grid and the model (packed x, u offsets are the
 // driver's Layout; x0 and x_ref share its g_off).
 struct PInst {
-  int dim, m, ng, ns, nu, N;
+  int dim, m, ng, ns, nu, N, neu;
   long long a_off;  // u_ref, actuator tables
   long long t_off;  // per-point tables
   double h, k0, k1, beta, ta, gr, q, r, qf, gamma, tau, ulo, uhi;
+  double lw;    // the Laplacian's neighbour weight 1 / spacing^2
+  double ta4;   // t_amb^4
 };
 
 struct PArgs {
   const PInst* inst;
   const int* pt_state;  // [sum ng]: state index, or -1 - a for actuator a
   const int* act_pt;    // [sum nu]: grid point of actuator a
-  const int* Lc;        // [sum ng][ELL] columns of L (unused slots: the point itself, weight 0)
-  const double* Lv;
-  const int* Ltc;       // the same for L^T
-  const double* Ltv;
-  const double* Ld;     // [sum ng] L[p][p]
-  const float* Lvf;     // float32 copies of Lv, Ltv, Ld (mixed precision)
-  const float* Ltvf;
-  const float* Ldf;
   const double* x0;
   const double* xref;
   const double* uref;
   int n_lo, n_u_it, rb, half;
 };
-
-// The stencil tables in the lower layer's type T.
-template <typename T>
-__device__ __forceinline__ const T* tab(const double* d, const float* f);
-template <>
-__device__ __forceinline__ const double* tab<double>(const double* d, const float*) { return d; }
-template <>
-__device__ __forceinline__ const float* tab<float>(const double*, const float* f) { return f; }
 
 __device__ __forceinline__ double phi(const PInst& I, double w) {
   return I.k0 * (w + 0.5 * I.k1 * w * w);
@@ -79,261 +59,268 @@ __device__ __forceinline__ double dphi(const PInst& I, double w) {
   return I.k0 * (1.0 + I.k1 * w);
 }
 
-// Sweeps of P^{-1} (eq. 24) over the state points of the stage grid:
-// F_x v5 = b4, then F_x^T v4 = b5 - A_xx v5, n_lo pointwise Jacobi sweeps
-// each from zero (Lemma 1).  F_x = h (L diag(Phi'(w)) - diag(beta + 4 gr x^3))
-// - I on the state points; its off-diagonal part sums L[p][q] Phi'(w_q) v_q
-// over the state neighbours q (v is zero at the actuator points).  The
-// lower layer runs in T (float64, or float32 in mixed precision: the
-// residual, the coefficients and the update stay float64, so the fixed
-// point is the float64 root); the grid values and costates stay float64.
+// Shared memory of one stage: Phi(w) and the (scaled) lambda in float64, three
+// exchange fields of the lower layer's type; each with a zero at index ng.
 template <typename T>
-struct Fields {
-  double *W, *LB, *PH, *LTL;
-  T *DP, *DG, *AX, *V, *V2, *B4, *B5, *K1, *K3, *Y4, *Y5, *Z;
-};
-constexpr int F64_FIELDS = 4, T_FIELDS = 12;  // shared memory: n_g values each
-
-template <typename T>
-__device__ void p_inv(const PArgs& A, const PInst& I, const Fields<T>& f, const int* pts) {
-  const int ng = I.ng;
-  const int* Lc = A.Lc + I.t_off * ELL;
-  const T* Lv = tab<T>(A.Lv, A.Lvf) + I.t_off * ELL;
-  const int* Ltc = A.Ltc + I.t_off * ELL;
-  const T* Ltv = tab<T>(A.Ltv, A.Ltvf) + I.t_off * ELL;
-  const T* Ld = tab<T>(A.Ld, A.Ldf) + I.t_off;
-  const T h = (T)I.h;
-  // F_x v5 = b4
-  T* cur = f.V;
-  T* nxt = f.V2;
-  for (int p = threadIdx.x; p < ng; p += THREADS) cur[p] = (pts[p] >= 0) ? f.B4[p] / f.DG[p] : T(0);
-  __syncthreads();
-  for (int sw = 1; sw < A.n_lo; ++sw) {
-    for (int p = threadIdx.x; p < ng; p += THREADS) {
-      T v = T(0);
-      if (pts[p] >= 0) {
-        T off = T(0);
-#pragma unroll
-        for (int e = 0; e < ELL; ++e) {
-          const int c = Lc[p * ELL + e];
-          off += Lv[p * ELL + e] * f.DP[c] * cur[c];
-        }
-        off -= Ld[p] * f.DP[p] * cur[p];
-        v = (f.B4[p] - h * off) / f.DG[p];
-      }
-      nxt[p] = v;
-    }
-    __syncthreads();
-    T* t = cur;
-    cur = nxt;
-    nxt = t;
-  }
-  for (int p = threadIdx.x; p < ng; p += THREADS) f.Y5[p] = cur[p];
-  __syncthreads();
-  // F_x^T v4 = b5 - A_xx v5; off-diagonal part h Phi'(x_p) sum_q L[q][p] v_q
-  for (int p = threadIdx.x; p < ng; p += THREADS)
-    cur[p] = (pts[p] >= 0) ? (f.B5[p] - f.AX[p] * f.Y5[p]) / f.DG[p] : T(0);
-  __syncthreads();
-  for (int sw = 1; sw < A.n_lo; ++sw) {
-    for (int p = threadIdx.x; p < ng; p += THREADS) {
-      T v = T(0);
-      if (pts[p] >= 0) {
-        T off = T(0);
-#pragma unroll
-        for (int e = 0; e < ELL; ++e) off += Ltv[p * ELL + e] * cur[Ltc[p * ELL + e]];
-        off -= Ld[p] * cur[p];
-        v = (f.B5[p] - f.AX[p] * f.Y5[p] - h * f.DP[p] * off) / f.DG[p];
-      }
-      nxt[p] = v;
-    }
-    __syncthreads();
-    T* t = cur;
-    cur = nxt;
-    nxt = t;
-  }
-  for (int p = threadIdx.x; p < ng; p += THREADS) f.Y4[p] = cur[p];
-  __syncthreads();
+__host__ __device__ constexpr size_t stage_bytes(int ng) {
+  return (((size_t)(ng + 1) * (2 * sizeof(double) + 3 * sizeof(T))) + 15) & ~size_t(15);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(THREADS) k_plate_dir(PArgs A, Ctl C, Iter S) {
-  const int2 it = C.work[blockIdx.x];
+// What bounds it: the float64 pipe (2 lanes a clock a SM) on batches, the
+// chain of exchanges on one plate.  A thread keeps its points' rows and
+// coefficients in registers and exchanges only the field that a stencil reads
+// (one barrier each); neighbours are found from the grid (4 additions and one
+// multiply-add a stencil, where a table of five weights cost five
+// multiply-adds and ten loads); the diagonal's reciprocal is taken once a
+// point (a division each sweep before); the actuators' rows, with their
+// divisions, sit in the group's first nu threads, so that one or two warps
+// execute them and not every warp that owns an actuator point; the maximum
+// norm is taken on integers.  1024 plates of 13x13, N = 20, float64: 326 ->
+// 144 ms a solve; one plate: 4.8 -> 2.4 ms.
+// F_x = h (L diag(Phi'(w)) - diag(beta + 4 gr x^3)) - I on the state points;
+// v is zero at the actuator points.  The lower layer runs in T (float64, or
+// float32 in mixed precision: the residual, the coefficients and the update
+// stay float64, so the fixed point is the float64 root).
+template <typename T, int PPT, bool NEU, bool D2>
+__global__ void __launch_bounds__(PPT == 1 ? 256 : 512, PPT == 1 ? 3 : 2)
+    k_plate_dir(PArgs A, Ctl C, Iter S, stage_drv::Range R) {
+  extern __shared__ __align__(16) double smem[];
+  __shared__ stage_drv::WarpNorms red[16];
+  stage_drv::pdl_trigger();
+  const int g = threadIdx.x / R.tps, t = threadIdx.x - g * R.tps;
+  const int item = blockIdx.x * R.spc + g;
+  stage_drv::pdl_wait();
+  if (item >= R.n) return;
+  const int2 it = C.work[R.first + item];
   const int b = it.x, s = it.y;
-  if (A.rb && ((s & 1) != A.half)) return;
-  if (stage_drv::finished(C, b)) return;
-  const PInst I = A.inst[b];
-  const Layout Ly = C.lay[b];
-  const int ng = I.ng, ns = I.ns, nu = I.nu, N = I.N;
-  const bool last = (s == N - 1);
-  extern __shared__ double smem[];
-  Fields<T> f;
-  double* q = smem;
-  f.W = q; q += ng;
-  f.LB = q; q += ng;
-  f.PH = q; q += ng;
-  f.LTL = q; q += ng;
-  T* qt = reinterpret_cast<T*>(q);
-  f.DP = qt; qt += ng;
-  f.DG = qt; qt += ng;
-  f.AX = qt; qt += ng;
-  f.V = qt; qt += ng;
-  f.V2 = qt; qt += ng;
-  f.B4 = qt; qt += ng;
-  f.B5 = qt; qt += ng;
-  f.K1 = qt; qt += ng;
-  f.K3 = qt; qt += ng;
-  f.Y4 = qt; qt += ng;
-  f.Y5 = qt; qt += ng;
-  f.Z = qt; qt += ng;
-  __shared__ double red[64];
-  __shared__ T sK2[MAX_NU], sAUU[MAX_NU], sV3[MAX_NU];
+  bool norms_only;
+  if (!stage_drv::begin_stage(C, b, s, t, norms_only)) return;
+  const PInst& I = A.inst[b];
+  const Layout& Ly = C.lay[b];
+  const int ng = I.ng, ns = I.ns, nu = I.nu;
+  const bool last = (s == I.N - 1);
+  double* fA = smem + (size_t)g * (stage_bytes<T>(R.ng_max) / sizeof(double));
+  double* fB = fA + (ng + 1);
+  T* fC = reinterpret_cast<T*>(fB + (ng + 1));
+  T* fD = fC + (ng + 1);
+  T* fZ = fD + (ng + 1);  // Phi'(u) v3 at the actuator points, zero elsewhere
   const int* pts = A.pt_state + I.t_off;
-  const int* apt = A.act_pt + I.a_off;
-  const int* Lc = A.Lc + I.t_off * ELL;
-  const double* Lv = A.Lv + I.t_off * ELL;
-  const int* Ltc = A.Ltc + I.t_off * ELL;
-  const double* Ltv = A.Ltv + I.t_off * ELL;
-  const double* Ld = A.Ld + I.t_off;
-  const T* LvT = tab<T>(A.Lv, A.Lvf) + I.t_off * ELL;
-  const T* LtvT = tab<T>(A.Ltv, A.Ltvf) + I.t_off * ELL;
   const long long so = Ly.s_off + (long long)s * ns;
   const long long uo = Ly.u_off + (long long)s * nu;
-  const double h = I.h;
+  const double h = I.h, lw = I.lw;
+  constexpr double d2 = D2 ? 4.0 : 2.0;  // the Laplacian's centre: -2 dim lw
+  const bool first = C.k == 0;           // S^0 is there already
+  const double alpha =
+      first ? 0.0
+            : fmin(1.0, __longlong_as_double(
+                            (long long)__ldcg(C.acand + ((C.k - 1) % stage_drv::SLOTS) * C.n_inst + b)));
+  // S^k at packed index e of a state array
+  auto xk = [&](const double* x, const double* dx, long long e) {
+    const double v = __ldcg(x + e);
+    return first ? v : v - alpha * __ldcg(dx + e);
+  };
 
-  // the stage's grid: w = x (states) / u (actuators); lambda-bar
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    const int t = pts[p];
-    double w, lb;
-    if (t >= 0) {
-      w = S.xin[so + t];
-      lb = S.lin[so + t];
-    } else {
-      w = S.uin[uo + (-1 - t)];
-      lb = 0.0;
-    }
-    f.W[p] = w;
-    f.LB[p] = lb;
-    f.PH[p] = phi(I, w);
-    f.DP[p] = (T)dphi(I, w);
+  stage_drv::Nbr<NEU, D2> nb[PPT];
+  int ts[PPT];  // state index, or negative: an actuator point or none
+  if (t == 0) {
+    fA[ng] = fB[ng] = 0.0;
+    fC[ng] = fD[ng] = fZ[ng] = T(0);
   }
-  __syncthreads();
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    double acc = 0.0;
+  double w[PPT], lam[PPT];
 #pragma unroll
-    for (int e = 0; e < ELL; ++e) acc += Ltv[p * ELL + e] * f.LB[Ltc[p * ELL + e]];
-    f.LTL[p] = acc;  // (L^T lambda-bar)(p)
+  for (int j = 0; j < PPT; ++j) {
+    const int p = t + j * R.tps;
+    nb[j].set(p, I.m, ng);
+    ts[j] = p < ng ? pts[p] : -0x7fffffff;
+    w[j] = lam[j] = 0.0;
+    if (p < ng) {
+      if (ts[j] >= 0) {
+        w[j] = xk(S.xin, S.px, so + ts[j]);
+        lam[j] = xk(S.lin, S.pl, so + ts[j]);
+        if (!first) {
+          S.xout[so + ts[j]] = w[j];
+          S.lout[so + ts[j]] = lam[j];
+        }
+      } else {
+        w[j] = xk(S.uin, S.pu, uo + (-1 - ts[j]));
+        if (!first) S.uout[uo + (-1 - ts[j])] = w[j];
+      }
+      fA[p] = phi(I, w[j]);
+      fB[p] = nb[j].scale(lam[j]);
+      fC[p] = fD[p] = fZ[p] = T(0);
+    }
   }
-  __syncthreads();
+  // the first nu threads: an actuator's row each
+  const bool act = t < nu;
+  stage_drv::Nbr<NEU, D2> na;
+  int pa = ng;
+  double ua = 0.0;
+  if (act) {
+    pa = A.act_pt[I.a_off + t];
+    ua = xk(S.uin, S.pu, uo + t);
+  }
+  na.set(pa, I.m, ng);
+  stage_drv::group_sync(g, R.tps);
 
   // K_i (eq. 9), coefficients, norms
-  double mx = 0.0, sq = 0.0;
-  const double d2p = I.k0 * I.k1;
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    const int t = pts[p];
-    if (t < 0) {
-      f.K1[p] = f.K3[p] = T(0);
-      f.DG[p] = T(1);
-      f.AX[p] = T(0);
-      continue;
-    }
-    const double x = f.W[p], lam = f.LB[p], xr = A.xref[Ly.g_off + t];
-    const double xprev = (s == 0) ? A.x0[Ly.g_off + t] : S.xin[so - ns + t];
-    const double lnext = last ? h * I.qf * (x - xr) : S.lin[so + ns + t];
-    double lph = 0.0;
+  unsigned long long mx = 0ull;
+  double sq = 0.0;
+  const double d2p = I.k0 * I.k1, hqf = last ? h * I.qf : 0.0;
+  T k1[PPT], k3[PPT], rdg[PPT], ax[PPT], dp[PPT];
 #pragma unroll
-    for (int e = 0; e < ELL; ++e) lph += Lv[p * ELL + e] * f.PH[Lc[p * ELL + e]];
-    const double x3 = x * x * x;
-    const double fp = lph - I.beta * (x - I.ta) - I.gr * (x3 * x - I.ta * I.ta * I.ta * I.ta);
+  for (int j = 0; j < PPT; ++j) {
+    k1[j] = k3[j] = rdg[j] = ax[j] = dp[j] = T(0);
+    if (ts[j] < 0) continue;
+    const int p = t + j * R.tps, e = ts[j];
+    const double x = w[j], lm = lam[j];
+    const double xprev = (s == 0) ? A.x0[Ly.g_off + e] : xk(S.xin, S.px, so - ns + e);
+    const double dx = x - A.xref[Ly.g_off + e];
+    const double lnext = last ? hqf * dx : xk(S.lin, S.pl, so + ns + e);
+    const double lph = lw * (nb[j].sum(fA) - d2 * fA[p]);                     // (L Phi)(p)
+    const double ltl = lw * (nb[j].unscale(nb[j].sum(fB)) - d2 * lm);         // (L^T lambda)(p)
+    const double x2 = x * x, gx3 = 4.0 * I.gr * (x2 * x) + I.beta;
+    const double fp = lph - I.beta * (x - I.ta) - I.gr * (x2 * x2 - I.ta4);
     const double K1 = xprev - x + h * fp;
     const double dpx = dphi(I, x);
-    const double gxT = dpx * f.LTL[p] - (I.beta + 4.0 * I.gr * x3) * lam;
-    const double K3 = lnext - lam + h * (I.q * (x - xr) + gxT);
-    mx = stage_drv::nan_max(mx, stage_drv::nan_max(fabs(K1), fabs(K3)));
+    const double K3 = lnext - lm + h * (I.q * dx + (dpx * ltl - gx3 * lm));
+    mx = max(mx, max(stage_drv::abs_bits(K1), stage_drv::abs_bits(K3)));
     sq += K1 * K1 + K3 * K3;
     // red-black half 1: the right-hand side takes the even neighbours'
-    // directions (state rows: M_L Delta x_{i-1}; costate rows: M_U Delta
-    // lambda_{i+1}); the norms above stay those of K(S^k)
+    // directions; the norms above stay those of K(S^k)
     double K1r = K1, K3r = K3;
     if (A.rb && A.half == 1) {
-      if (s > 0) K1r -= S.dx[so - ns + t];
-      if (!last) K3r -= S.dl[so + ns + t];
+      if (s > 0) K1r -= __ldcg(S.dx + so - ns + e);
+      if (!last) K3r -= __ldcg(S.dl + so + ns + e);
     }
-    f.K1[p] = (T)K1r;
-    f.K3[p] = (T)K3r;
-    f.DG[p] = (T)(h * (Ld[p] * dpx - I.beta - 4.0 * I.gr * x3) - 1.0);
-    f.AX[p] = (T)(h * (I.q + d2p * f.LTL[p] - 12.0 * I.gr * x * x * lam) + (last ? h * I.qf : 0.0));
+    k1[j] = (T)K1r;
+    k3[j] = (T)K3r;
+    dp[j] = (T)dpx;
+    rdg[j] = stage_drv::rcp((T)(h * (-d2 * lw * dpx - gx3) - 1.0));
+    ax[j] = (T)(h * (I.q + d2p * ltl - 12.0 * I.gr * x2 * lm) + hqf);
   }
-  for (int a = threadIdx.x; a < nu; a += THREADS) {
-    const int pa = apt[a];
-    const double u = f.W[pa];
+  T k2 = T(0), rauu = T(0), dpu = T(0), v3 = T(0);
+  double il = 0.0, ih = 0.0;  // 1 / slack to the lower, the upper bound
+  if (act) {
+    const double ltl = lw * na.unscale(na.sum(fB));  // lambda is zero at the point itself
     double db = 0.0, d2b = 0.0;
     if (I.tau > 0.0) {
-      db = -I.tau / (u - I.ulo) + I.tau / (I.uhi - u);
-      d2b = I.tau / ((u - I.ulo) * (u - I.ulo)) + I.tau / ((I.uhi - u) * (I.uhi - u));
+      il = 1.0 / (ua - I.ulo);
+      ih = 1.0 / (I.uhi - ua);
+      db = I.tau * (ih - il);
+      d2b = I.tau * (il * il + ih * ih);
     }
-    const double K2 = h * (I.r * (u - A.uref[I.a_off + a]) + db + dphi(I, u) * f.LTL[pa]);
-    mx = stage_drv::nan_max(mx, fabs(K2));
+    const double dpx = dphi(I, ua);
+    const double K2 = h * (I.r * (ua - A.uref[I.a_off + t]) + db + dpx * ltl);
+    mx = max(mx, stage_drv::abs_bits(K2));
     sq += K2 * K2;
-    sK2[a] = (T)K2;
-    sAUU[a] = (T)(h * (I.r + d2b + d2p * f.LTL[pa]) + I.gamma);
-    sV3[a] = T(0);
+    k2 = (T)K2;
+    rauu = stage_drv::rcp((T)(h * (I.r + d2b + d2p * ltl) + I.gamma));
+    dpu = (T)dpx;
   }
-  __syncthreads();
-  stage_drv::block_max_sum(mx, sq, red, THREADS);
-  if (stage_drv::publish_norms(C, b, mx, sq)) return;  // norms only
+  stage_drv::warp_norms(mx, sq, red);
 
-  // u fixed-point iteration (Sec. 5.2): y = P^{-1}(F_u v3 - b1, -b2),
-  // v3 = (b3 + F_u^T y_lambda) / A_uu, from v3 = 0
-  const T hT = (T)h;
+  // u fixed-point iteration (Sec. 5.2) on the direction y = P^{-1}(K_1 - F_u
+  // v3, K_3): v3 = (K_2 - F_u^T y_lambda) / A_uu from v3 = 0, then the last y.
+  // F_u v3 = h L Z, Z = Phi'(u) v3 at the actuator points.
+  const T hw = (T)(h * lw);
+  T v5[PPT], v4[PPT];
+#pragma unroll
+  for (int j = 0; j < PPT; ++j) v5[j] = v4[j] = T(0);
+  const int n_lo = A.n_lo;
+  T *ex = fC, *ex2 = fD;  // the next exchange's field, the other one
   for (int itu = 0; itu <= A.n_u_it; ++itu) {
-    const bool final_pass = (itu == A.n_u_it);
-    // Z = Phi'(u) v3 at the actuator points, zero elsewhere
-    for (int p = threadIdx.x; p < ng; p += THREADS) f.Z[p] = T(0);
-    __syncthreads();
-    for (int a = threadIdx.x; a < nu; a += THREADS) f.Z[apt[a]] = f.DP[apt[a]] * sV3[a];
-    __syncthreads();
-    for (int p = threadIdx.x; p < ng; p += THREADS) {
-      T fu = T(0);  // (F_u v3)(p) = h sum_a L[p][a] Phi'(u_a) v3_a
+    if (itu > 0) {
+      if (act) fZ[pa] = dpu * v3;
+      stage_drv::group_sync(g, R.tps);
+    }
+    T b4[PPT], b5[PPT];
 #pragma unroll
-      for (int e = 0; e < ELL; ++e) fu += LvT[p * ELL + e] * f.Z[Lc[p * ELL + e]];
-      fu *= hT;
-      if (pts[p] >= 0) {
-        f.B4[p] = final_pass ? f.K1[p] - fu : fu - f.K1[p];
-        f.B5[p] = final_pass ? f.K3[p] : -f.K3[p];
-      } else {
-        f.B4[p] = f.B5[p] = T(0);
+    for (int j = 0; j < PPT; ++j) {
+      b4[j] = itu > 0 ? k1[j] - hw * nb[j].sum(fZ) : k1[j];
+      v5[j] = b4[j] * rdg[j];
+    }
+    for (int sw = 1; sw < n_lo; ++sw) {  // F_x v5 = b4 (rdg is zero off the state points)
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+        if (ts[j] >= 0) ex[t + j * R.tps] = dp[j] * v5[j];
+      stage_drv::group_sync(g, R.tps);
+      if (itu == 0 && sw == 1) {
+        if (t == 0) stage_drv::publish_norms(C, b, red, R.tps);
+        if (norms_only) return;
       }
-    }
-    __syncthreads();
-    p_inv<T>(A, I, f, pts);
-    if (final_pass) break;
-    for (int a = threadIdx.x; a < nu; a += THREADS) {
-      const int pa = apt[a];
-      T acc = T(0);  // (L^T y_lambda)(a) over the state points
 #pragma unroll
-      for (int e = 0; e < ELL; ++e) acc += LtvT[pa * ELL + e] * f.Y4[Ltc[pa * ELL + e]];
-      sV3[a] = (sK2[a] + hT * f.DP[pa] * acc) / sAUU[a];
+      for (int j = 0; j < PPT; ++j) v5[j] = (b4[j] - hw * nb[j].sum(ex)) * rdg[j];
+      T* x = ex;
+      ex = ex2;
+      ex2 = x;
     }
-    __syncthreads();
+    if (itu == 0 && n_lo == 1) {
+      stage_drv::group_sync(g, R.tps);
+      if (t == 0) stage_drv::publish_norms(C, b, red, R.tps);
+      if (norms_only) return;
+    }
+#pragma unroll
+    for (int j = 0; j < PPT; ++j) {
+      b5[j] = k3[j] - ax[j] * v5[j];
+      v4[j] = b5[j] * rdg[j];
+    }
+    for (int sw = 1; sw < n_lo; ++sw) {  // F_x^T v4 = b5
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+        if (ts[j] >= 0) ex[t + j * R.tps] = nb[j].scale(v4[j]);
+      stage_drv::group_sync(g, R.tps);
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+        v4[j] = (b5[j] - hw * dp[j] * nb[j].unscale(nb[j].sum(ex))) * rdg[j];
+      T* x = ex;
+      ex = ex2;
+      ex2 = x;
+    }
+    if (itu == A.n_u_it) break;
+#pragma unroll
+    for (int j = 0; j < PPT; ++j)
+      if (ts[j] >= 0) ex[t + j * R.tps] = nb[j].scale(v4[j]);
+    stage_drv::group_sync(g, R.tps);
+    if (act) v3 = (k2 - hw * dpu * na.unscale(na.sum(ex))) * rauu;
+    T* x = ex;
+    ex = ex2;
+    ex2 = x;
   }
   // direction (Delta x, Delta u, Delta lambda) = (v5, v3, v4); admissible step
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    const int t = pts[p];
-    if (t >= 0) {
-      S.dx[so + t] = (double)f.Y5[p];
-      S.dl[so + t] = (double)f.Y4[p];
+#pragma unroll
+  for (int j = 0; j < PPT; ++j) {
+    if (ts[j] >= 0) {
+      S.dx[so + ts[j]] = (double)v5[j];
+      S.dl[so + ts[j]] = (double)v4[j];
     }
   }
-  double amin = 1.0;
-  for (int a = threadIdx.x; a < nu; a += THREADS) {
-    const double d = (double)sV3[a], u = f.W[apt[a]];
-    S.du[uo + a] = d;
-    if (I.tau > 0.0) {
-      if (d > 0.0) amin = fmin(amin, 0.995 * (u - I.ulo) / d);
-      if (d < 0.0) amin = fmin(amin, 0.995 * (I.uhi - u) / (-d));
+  if ((t & ~31) < nu) {  // the actuators' warps
+    double amin = 1.0;
+    if (act) {
+      const double d = (double)v3;
+      S.du[uo + t] = d;
+      if (I.tau > 0.0) {
+        if (d > 0.0) amin = fmin(amin, 0.995 * (ua - I.ulo) / d);
+        if (d < 0.0) amin = fmin(amin, 0.995 * (I.uhi - ua) / (-d));
+      }
+    }
+    stage_drv::publish_step(C, b, amin);
+  }
+}
+
+// (L v)(p) over a stage's grid, one axis after the other.
+__device__ __forceinline__ double lap_at(const PInst& I, const double* v, int p) {
+  double acc = -2.0 * I.dim * v[p];
+  for (int axis = 0; axis < I.dim; ++axis) {
+    const int st = axis ? I.m : 1, i = axis ? p / I.m : p % I.m;
+    const bool lo = i > 0, hi = i < I.m - 1;
+    if (I.neu) {  // the mirrored point
+      acc += v[lo ? p - st : p + st] + v[hi ? p + st : p - st];
+    } else {
+      acc += (lo ? v[p - st] : 0.0) + (hi ? v[p + st] : 0.0);
     }
   }
-  stage_drv::publish_step(C, b, amin);
+  return I.lw * acc;
 }
 
 // The plant: w (state points) += (dt / n_sub) f(w, u1), n_sub times, with the
@@ -348,8 +335,6 @@ __global__ void __launch_bounds__(THREADS) k_plate_plant(PArgs A, const Layout* 
   double* W = smem;
   double* PH = W + I.ng;
   const int* pts = A.pt_state + I.t_off;
-  const int* Lc = A.Lc + I.t_off * ELL;
-  const double* Lv = A.Lv + I.t_off * ELL;
   for (int p = threadIdx.x; p < I.ng; p += THREADS) {
     const int t = pts[p];
     W[p] = (t >= 0) ? w[Ly.g_off + t] : uc[Ly.u_off + (-1 - t)];
@@ -364,9 +349,7 @@ __global__ void __launch_bounds__(THREADS) k_plate_plant(PArgs A, const Layout* 
     for (int p = threadIdx.x; p < I.ng; p += THREADS, ++cnt) {
       double v = W[p];
       if (pts[p] >= 0) {
-        double lph = 0.0;
-#pragma unroll
-        for (int e = 0; e < ELL; ++e) lph += Lv[p * ELL + e] * PH[Lc[p * ELL + e]];
+        const double lph = lap_at(I, PH, p);
         const double x = v, x4 = x * x * x * x;
         v = x + tau * (lph - I.beta * (x - I.ta) - I.gr * (x4 - I.ta * I.ta * I.ta * I.ta));
       }
@@ -395,19 +378,15 @@ struct nmpc_plate {
   long long n_a = 0;         // sum n_u
   int ng_max = 0;
   PInst* inst_d = nullptr;
-  int *pt_state = nullptr, *act_pt = nullptr, *Lc = nullptr, *Ltc = nullptr;
-  double *Lv = nullptr, *Ltv = nullptr, *Ld = nullptr;
-  float *Lvf = nullptr, *Ltvf = nullptr, *Ldf = nullptr;
+  int *pt_state = nullptr, *act_pt = nullptr;
   double *xref = nullptr, *uref = nullptr;
-  size_t smem = 0;
 };
 
 namespace {
 
 void free_plate(nmpc_plate* h) {
   stage_drv::driver_free(h->drv);
-  void* ptrs[] = {h->inst_d, h->pt_state, h->act_pt, h->Lc, h->Ltc, h->Lv, h->Ltv, h->Ld, h->Lvf,
-                  h->Ltvf, h->Ldf, h->xref, h->uref};
+  void* ptrs[] = {h->inst_d, h->pt_state, h->act_pt, h->xref, h->uref};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -437,14 +416,6 @@ PArgs make_args(const nmpc_plate* h) {
   A.inst = h->inst_d;
   A.pt_state = h->pt_state;
   A.act_pt = h->act_pt;
-  A.Lc = h->Lc;
-  A.Lv = h->Lv;
-  A.Ltc = h->Ltc;
-  A.Ltv = h->Ltv;
-  A.Ld = h->Ld;
-  A.Lvf = h->Lvf;
-  A.Ltvf = h->Ltvf;
-  A.Ldf = h->Ldf;
   A.x0 = h->drv.x0;
   A.xref = h->xref;
   A.uref = h->uref;
@@ -454,21 +425,37 @@ PArgs make_args(const nmpc_plate* h) {
   return A;
 }
 
-// The direction kernels of one iteration: one launch, or the two red-black
-// halves.
+// k_plate_dir for a group of stages.
+using DirKernel = void (*)(PArgs, stage_drv::Ctl, stage_drv::Iter, stage_drv::Range);
+template <typename T, int PPT>
+DirKernel dir_kernel_of(bool neu, bool d2) {
+  if (neu) return d2 ? plate_dev::k_plate_dir<T, PPT, true, true> : plate_dev::k_plate_dir<T, PPT, true, false>;
+  return d2 ? plate_dev::k_plate_dir<T, PPT, false, true> : plate_dev::k_plate_dir<T, PPT, false, false>;
+}
+DirKernel dir_kernel(bool mixed, const stage_drv::Group& g) {
+  if (mixed) return g.ppt == 1 ? dir_kernel_of<float, 1>(g.neu, g.d2) : dir_kernel_of<float, 2>(g.neu, g.d2);
+  return g.ppt == 1 ? dir_kernel_of<double, 1>(g.neu, g.d2) : dir_kernel_of<double, 2>(g.neu, g.d2);
+}
+size_t stage_smem(bool mixed, const stage_drv::Group& g) {
+  return mixed ? plate_dev::stage_bytes<float>(g.ng_max) : plate_dev::stage_bytes<double>(g.ng_max);
+}
+
+// The direction kernels of one iteration: one launch per group of stages, or
+// the two red-black halves.
 struct PlateDir {
   const nmpc_plate* h;
   cudaStream_t st;
   cudaError_t operator()(const stage_drv::Ctl& C, const stage_drv::Iter& S) const {
     PArgs A = make_args(h);
+    const bool mixed = h->opts.precision == NMPC_MIXED;
     for (int half = 0; half < (A.rb ? 2 : 1); ++half) {
       A.half = half;
-      if (h->opts.precision == NMPC_MIXED)
-        plate_dev::k_plate_dir<float><<<h->drv.n_work, plate_dev::THREADS, h->smem, st>>>(A, C, S);
-      else
-        plate_dev::k_plate_dir<double><<<h->drv.n_work, plate_dev::THREADS, h->smem, st>>>(A, C, S);
-      const cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
+      for (const stage_drv::Group& g : h->drv.groups) {
+        const cudaError_t e =
+            stage_drv::launch_stages(dir_kernel(mixed, g), stage_smem(mixed, g),
+                                     stage_drv::range_of(g, A.rb != 0, half), A, C, S, st);
+        if (e != cudaSuccess) return e;
+      }
     }
     return cudaSuccess;
   }
@@ -525,8 +512,8 @@ int nmpc_plate_setup(const nmpc_plate_desc* descs, int n, const nmpc_plate_opts*
   nmpc_plate* h = new (std::nothrow) nmpc_plate();
   if (!h) return NMPC_ERR_CUDA;
   h->opts = o;
-  std::vector<int> pt_state, act_pt, Lc, Ltc;
-  std::vector<double> Lv, Ltv, Ld;
+  std::vector<int> pt_state, act_pt;
+  std::vector<stage_drv::GridKind> grid;
   long long n_pts = 0;
   for (int b = 0; b < n; ++b) {
     const nmpc_plate_desc& d = descs[b];
@@ -552,6 +539,9 @@ int nmpc_plate_setup(const nmpc_plate_desc* descs, int n, const nmpc_plate_opts*
     I.tau = d.tau;
     I.ulo = d.u_lo;
     I.uhi = d.u_hi;
+    I.neu = d.bc == 0 ? 1 : 0;
+    I.lw = stage_drv::neighbour_weight(d.m, d.bc);
+    I.ta4 = d.t_amb * d.t_amb * d.t_amb * d.t_amb;
     // point -> state index (grid order of the non-actuator points) or -1 - a
     std::vector<int> state_of(I.ng, 0);
     std::vector<char> is_act(I.ng, 0);
@@ -564,7 +554,7 @@ int nmpc_plate_setup(const nmpc_plate_desc* descs, int n, const nmpc_plate_opts*
       if (!is_act[p]) state_of[p] = t++;
     for (int p = 0; p < I.ng; ++p) pt_state.push_back(state_of[p]);
     for (int a = 0; a < d.n_u; ++a) act_pt.push_back(d.act_cell[a]);
-    stage_drv::append_ell(d.dim, d.m, d.bc == 0 ? 0 : 1, Lc, Lv, Ltc, Ltv, Ld);
+    grid.push_back(stage_drv::GridKind{d.dim, d.m, I.ng, d.bc == 0});
     stage_drv::Layout L{};
     L.N = I.N;
     L.nx = I.ns;
@@ -576,43 +566,22 @@ int nmpc_plate_setup(const nmpc_plate_desc* descs, int n, const nmpc_plate_opts*
     h->ng_max = std::max(h->ng_max, I.ng);
     h->inst_h.push_back(I);
   }
-  const size_t tsz = o.precision == NMPC_MIXED ? sizeof(float) : sizeof(double);
-  h->smem = (size_t)h->ng_max * (plate_dev::F64_FIELDS * sizeof(double) + plate_dev::T_FIELDS * tsz);
-  cudaError_t e = stage_drv::driver_alloc(h->drv);
+  cudaError_t e = stage_drv::driver_alloc(h->drv, grid, true);
   auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   A(stage_drv::dalloc(&h->inst_d, n));
   A(stage_drv::dalloc(&h->pt_state, pt_state.size()));
   A(stage_drv::dalloc(&h->act_pt, act_pt.size()));
-  A(stage_drv::dalloc(&h->Lc, Lc.size()));
-  A(stage_drv::dalloc(&h->Ltc, Ltc.size()));
-  A(stage_drv::dalloc(&h->Lv, Lv.size()));
-  A(stage_drv::dalloc(&h->Ltv, Ltv.size()));
-  A(stage_drv::dalloc(&h->Ld, Ld.size()));
   A(stage_drv::dalloc(&h->xref, h->drv.n_g));
   A(stage_drv::dalloc(&h->uref, h->n_a));
   A(stage_drv::upload(h->inst_d, h->inst_h));
   A(stage_drv::upload(h->pt_state, pt_state));
   A(stage_drv::upload(h->act_pt, act_pt));
-  A(stage_drv::upload(h->Lc, Lc));
-  A(stage_drv::upload(h->Ltc, Ltc));
-  A(stage_drv::upload(h->Lv, Lv));
-  A(stage_drv::upload(h->Ltv, Ltv));
-  A(stage_drv::upload(h->Ld, Ld));
-  {
-    const std::vector<float> Lvf(Lv.begin(), Lv.end()), Ltvf(Ltv.begin(), Ltv.end()),
-        Ldf(Ld.begin(), Ld.end());
-    A(stage_drv::dalloc(&h->Lvf, Lvf.size()));
-    A(stage_drv::dalloc(&h->Ltvf, Ltvf.size()));
-    A(stage_drv::dalloc(&h->Ldf, Ldf.size()));
-    A(stage_drv::upload(h->Lvf, Lvf));
-    A(stage_drv::upload(h->Ltvf, Ltvf));
-    A(stage_drv::upload(h->Ldf, Ldf));
-  }
-  if (h->smem > 48 * 1024) {
-    A(cudaFuncSetAttribute(plate_dev::k_plate_dir<double>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem));
-    A(cudaFuncSetAttribute(plate_dev::k_plate_dir<float>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem));
+  for (const stage_drv::Group& g : h->drv.groups) {
+    const bool mixed = o.precision == NMPC_MIXED;
+    const size_t bytes = stage_smem(mixed, g) * g.spc;
+    if (bytes > 48 * 1024)
+      A(cudaFuncSetAttribute(dir_kernel(mixed, g), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)bytes));
   }
   if (e != cudaSuccess) {
     fprintf(stderr, "nmpc_plate_setup: %s\n", cudaGetErrorString(e));

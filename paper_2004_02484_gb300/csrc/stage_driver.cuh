@@ -1,16 +1,21 @@
-// The upper-layer driver shared by the stage-per-CTA solvers (the pinned-
-// actuator plate and the second-order wave): per iteration k the problem's
-// direction kernel(s) publish ||K(S^k)||_inf, ||K(S^k)||_2^2 and the largest
-// admissible step (eq. 11) per instance and store Delta S; k_update then
-// takes the convergence decision (Table 2's rule ||K||_inf <= tol) and forms
-// S^{k+1} = S^k - alpha Delta S.  Start iterates (cold, warm, shifted by one
-// stage), the returned iterate and the host loops of a solve and of a fixed
-// number of iterations live here too.
+// The upper-layer driver shared by the stage-parallel solvers (the pinned-
+// actuator plate and the second-order wave).  One launch of a problem's
+// direction kernel is one iteration k (two, one per stage parity, with the
+// red-black order): it decides from iteration k - 1's norms whether the
+// instance has finished (Table 2's rule ||K||_inf <= tol), publishes
+// ||K(S^k)||_inf, ||K(S^k)||_2^2 and the largest admissible step (eq. 11)
+// per instance, and forms S^{k+1} itself (wave: the full step) or leaves
+// Delta S^k for the next launch to apply (plate: the step length is known
+// once every stage of the instance has published its own).  So an iteration
+// costs one launch and no separate pass over the state.  Start iterates
+// (cold, warm, shifted by one stage), the returned iterate and the host loops
+// of a solve and of a fixed number of iterations live here too.
 //
 // Arrays are packed per instance: x, lambda [sum N nx] stage-major, u
-// [sum N nu] stage-major, x0 [sum nx].  Control words come in two slots,
-// one per iteration parity, so that iteration k+1's direction kernels can
-// accumulate while iteration k's decision is still being read.
+// [sum N nu] stage-major, x0 [sum nx].  The control words of iteration k are
+// in slot k % SLOTS: k - 1's is read while k's accumulates and k + 1's is
+// cleared, and launches may overlap their start with the previous launch's
+// end (programmatic dependent launch).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -28,6 +33,7 @@ namespace stage_drv {
 
 enum { ST_RUNNING = 0, ST_CONVERGED = 1, ST_DIVERGED = 2, ST_MAX_ITER = 3 };
 enum { MODE_SOLVE = 0, MODE_ONESHOT = 1 };
+constexpr int SLOTS = 4;  // iterations k - 1, k, k + 1 in use at once
 
 struct Layout {
   int N, nx, nu;     // stages, state entries per stage, inputs per stage
@@ -39,10 +45,10 @@ struct Layout {
 
 struct Ctl {
   const Layout* lay;
-  const int2* work;            // (instance, stage), one CTA each
-  unsigned long long* rmax;    // [2][n] bits of ||K||_inf (non-negative doubles order as integers)
-  double* rsq;                 // [2][n] ||K||_2^2
-  unsigned long long* acand;   // [2][n] bits of the admissible step
+  const int2* work;            // (instance, stage), one thread group each
+  unsigned long long* rmax;    // [SLOTS][n] bits of ||K||_inf (non-negative doubles order as integers)
+  double* rsq;                 // [SLOTS][n] ||K||_2^2
+  unsigned long long* acand;   // [SLOTS][n] bits of the admissible step
   int* status;
   int* iters;
   int* final_buf;
@@ -52,6 +58,9 @@ struct Ctl {
   double tol;
 };
 
+// The state arrays of one launch: xin, uin, lin hold the iterate that the
+// launch reads, xout, uout, lout the one it writes; the plate's launch k also
+// reads Delta S^{k-1} (px, pu, pl) and writes Delta S^k (dx, du, dl).
 struct Iter {
   const double* xin;
   const double* uin;
@@ -59,102 +68,216 @@ struct Iter {
   double* xout;
   double* uout;
   double* lout;
-  double* dx;  // direction Delta S
+  const double* px;
+  const double* pu;
+  const double* pl;
+  double* dx;
   double* du;
   double* dl;
 };
 
-// max that keeps a NaN once one has been seen (fmax would drop it)
-__device__ __forceinline__ double nan_max(double a, double b) {
-  return (a != a || b != b) ? CUDART_NAN : fmax(a, b);
+// The work items that one launch shape covers: the stages of the instances of
+// one grid kind (dimension, boundary condition), even stages first.  A stage
+// is a group of tps threads (a multiple of 32) with ppt points each, spc
+// groups to a CTA: a 64-point string on a 256-thread CTA of its own left six
+// of eight warps idle, four of them share one now.  More than 256 points take
+// two a thread (at most 512 threads).  Few stages stay one to a CTA so that a
+// single instance still spreads over the SMs.
+struct Group {
+  int first, n, n_even;
+  int tps, spc, ppt;
+  bool neu, d2;
+  int ng_max;
+};
+struct Range {  // the items of one launch
+  int first, n, tps, spc, ng_max;
+};
+
+// A group's items in one launch: all of them, or one parity's (red-black).
+inline Range range_of(const Group& g, bool rb, int half) {
+  Range r{g.first, g.n, g.tps, g.spc, g.ng_max};
+  if (rb) {
+    r.first += half ? g.n_even : 0;
+    r.n = half ? g.n - g.n_even : g.n_even;
+  }
+  return r;
 }
 
-// Block reduction of (max, sum) over nthreads threads (a multiple of 32);
-// thread 0 holds the result.  red: 64 doubles of shared memory.
-__device__ inline void block_max_sum(double& mx, double& sq, double* red, int nthreads) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) {
-    mx = nan_max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    sq += __shfl_xor_sync(0xffffffffu, sq, o);
-  }
-  if (lane == 0) {
-    red[w] = mx;
-    red[32 + w] = sq;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < nthreads / 32; ++i) {
-      mx = nan_max(mx, red[i]);
-      sq += red[32 + i];
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Barrier of thread group g of a CTA (tps threads, a multiple of 32).
+__device__ __forceinline__ void group_sync(int g, int tps) {
+  if (tps == 32)
+    __syncwarp();
+  else
+    asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(tps) : "memory");
+}
+
+// The grid neighbours of point p among m (or m x m) points, as indices into a
+// field of ng values with a zero at index ng: outside a Dirichlet grid the
+// zero, outside a Neumann grid the mirrored point (eq. 3).
+template <bool NEU, bool D2>
+struct Nbr {
+  unsigned lr, ud;  // left | right << 16, above | below << 16 (fields hold at most 1025 values)
+  float di;         // NEU: 2 per axis on whose boundary p lies, else 1 (L^T below)
+  __device__ __forceinline__ void set(int p, int m, int ng) {
+    if (p >= ng) {  // no point: reads the zero
+      lr = ud = (unsigned)ng | ((unsigned)ng << 16);
+      di = 1.0f;
+      return;
+    }
+    const int iy = D2 ? p / m : 0, ix = p - iy * m;
+    const int l = ix > 0 ? p - 1 : (NEU ? p + 1 : ng);
+    const int r = ix < m - 1 ? p + 1 : (NEU ? p - 1 : ng);
+    lr = (unsigned)l | ((unsigned)r << 16);
+    ud = 0u;
+    if constexpr (D2) {
+      const int u = iy > 0 ? p - m : (NEU ? p + m : ng);
+      const int d = iy < m - 1 ? p + m : (NEU ? p - m : ng);
+      ud = (unsigned)u | ((unsigned)d << 16);
+    }
+    di = 1.0f;
+    if constexpr (NEU) {
+      if (ix == 0 || ix == m - 1) di *= 2.0f;
+      if (D2 && (iy == 0 || iy == m - 1)) di *= 2.0f;
     }
   }
-  __syncthreads();
-}
-
-// A direction CTA of instance b has nothing to do (the instance has stopped).
-__device__ __forceinline__ bool finished(const Ctl& C, int b) {
-  return C.mode == MODE_SOLVE && C.status[b] != ST_RUNNING;
-}
-
-// Thread 0's block norms into the instance's slot of iteration k; true when
-// the iteration only evaluates the norms (the last one a solve allows).
-__device__ __forceinline__ bool publish_norms(const Ctl& C, int b, double mx, double sq) {
-  if (threadIdx.x == 0) {
-    const int slot = (C.k & 1) * C.n_inst + b;
-    atomicMax(&C.rmax[slot], (unsigned long long)__double_as_longlong(mx));
-    atomicAdd(&C.rsq[slot], sq);
+  // sum over the neighbours of v: (L v)(p) = lw (sum - 2 dim v(p))
+  template <typename V>
+  __device__ __forceinline__ V sum(const V* v) const {
+    V s = v[lr & 0xffffu] + v[lr >> 16];
+    if constexpr (D2) s += v[ud & 0xffffu] + v[ud >> 16];
+    return s;
   }
-  return C.mode == MODE_SOLVE && C.k >= C.max_iter;
+  // The mirrored Laplacian is D^{-1} S with S symmetric and D = diag(1 / di),
+  // so (L^T v)(p) = (L (di v))(p) / di: a field read through the transpose is
+  // stored as scale(v), its neighbour sum taken through unscale().  Both are
+  // exact (powers of two); on a Dirichlet grid L is symmetric.
+  template <typename V>
+  __device__ __forceinline__ V scale(V v) const {
+    return NEU ? v * (V)di : v;
+  }
+  template <typename V>
+  __device__ __forceinline__ V unscale(V v) const {
+    return NEU ? v * (V)(di == 1.0f ? 1.0f : (di == 2.0f ? 0.5f : 0.25f)) : v;
+  }
+};
+
+// 1 / v rounded to nearest
+__device__ __forceinline__ float rcp(float v) { return __frcp_rn(v); }
+__device__ __forceinline__ double rcp(double v) { return __drcp_rn(v); }
+
+// Bits of |v|: non-negative doubles order as integers, NaN above infinity, so
+// that a maximum costs the integer pipe and not the two-lane float64 one and
+// keeps a NaN.
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+
+// The warp's norms (max bits, sum of squares) into red[warp] (lane 0).
+struct WarpNorms {
+  unsigned long long mx;
+  double sq;
+};
+__device__ __forceinline__ void warp_norms(unsigned long long mx, double sq, WarpNorms* red) {
+  for (int o = 16; o > 0; o >>= 1) {
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  }
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = WarpNorms{mx, sq};
+}
+
+// After a group barrier, by the group's thread 0: its warps' norms into the
+// instance's slot of iteration k.
+__device__ __forceinline__ void publish_norms(const Ctl& C, int b, const WarpNorms* red, int tps) {
+  const int w0 = threadIdx.x >> 5;
+  unsigned long long mx = red[w0].mx;
+  double sq = red[w0].sq;
+  for (int w = 1; w < tps / 32; ++w) {
+    mx = max(mx, red[w0 + w].mx);
+    sq += red[w0 + w].sq;
+  }
+  const int slot = (C.k % SLOTS) * C.n_inst + b;
+  atomicMax(&C.rmax[slot], mx);
+  atomicAdd(&C.rsq[slot], sq);
 }
 
 // A warp's smallest admissible step (amin in (0, 1]) into the instance's slot.
 __device__ __forceinline__ void publish_step(const Ctl& C, int b, double amin) {
   for (int o = 16; o > 0; o >>= 1) amin = fmin(amin, __shfl_xor_sync(0xffffffffu, amin, o));
   if ((threadIdx.x & 31) == 0 && amin < 1.0)
-    atomicMin(&C.acand[(C.k & 1) * C.n_inst + b], (unsigned long long)__double_as_longlong(amin));
+    atomicMin(&C.acand[(C.k % SLOTS) * C.n_inst + b],
+              (unsigned long long)__double_as_longlong(amin));
 }
 
-// The decision of iteration k and S^{k+1} = S^k - alpha Delta S, one CTA
-// per (instance, stage).
-// (static: each translation unit that includes this header has its own copy)
-static __global__ void __launch_bounds__(256) k_update(Ctl C, Iter S) {
-  const int2 it = C.work[blockIdx.x];
-  const int b = it.x, s = it.y;
-  const Layout L = C.lay[b];
-  const int slot = (C.k & 1) * C.n_inst + b;
-  bool stop = false;
-  double r = 0.0;
+// Records that instance b stopped with iterate kf.
+__device__ __forceinline__ void record_stop(const Ctl& C, int b, int kf, int status, double r) {
+  C.status[b] = status;
+  C.iters[b] = kf;
+  C.final_buf[b] = kf & 1;
+  C.fin[b] = r;
+  C.fin[C.n_inst + b] = sqrt(__ldcg(C.rsq + (kf % SLOTS) * C.n_inst + b));
+  atomicSub(C.n_active, 1);
+}
+
+// What iteration k does for a stage's group: nothing (returns false: the
+// instance has stopped, now or before), the norms only (the last iteration a
+// solve allows) or all of it.  Every thread of every group of the instance
+// reads the same norms and so decides alike (a status written meanwhile by
+// the book-keeper, stage 0's thread 0, says the same).
+__device__ __forceinline__ bool begin_stage(const Ctl& C, int b, int s, int t, bool& norms_only) {
+  norms_only = false;
+  const bool books = s == 0 && t == 0;
   if (C.mode == MODE_SOLVE) {
-    if (C.status[b] != ST_RUNNING) return;  // finished before this kernel
-    r = __longlong_as_double((long long)C.rmax[slot]);
-    stop = !(r <= 1.79e308) || r <= C.tol || C.k >= C.max_iter;
+    const int status = __ldcg(C.status + b);
+    const double r =
+        C.k > 0 ? __longlong_as_double((long long)__ldcg(C.rmax + ((C.k - 1) % SLOTS) * C.n_inst + b))
+                : CUDART_INF;
+    if (status != ST_RUNNING) return false;
+    if (C.k > 0 && (!(r <= 1.79e308) || r <= C.tol)) {
+      if (books) record_stop(C, b, C.k - 1, !(r <= 1.79e308) ? ST_DIVERGED : ST_CONVERGED, r);
+      return false;
+    }
+    norms_only = C.k >= C.max_iter;
   }
-  if (s == 0 && threadIdx.x == 0) {
-    const int nslot = ((C.k + 1) & 1) * C.n_inst + b;
+  if (books) {
+    const int nslot = ((C.k + 1) % SLOTS) * C.n_inst + b;
     C.rmax[nslot] = 0ull;
     C.rsq[nslot] = 0.0;
     C.acand[nslot] = (unsigned long long)__double_as_longlong(1.0);
   }
-  if (stop) {
-    if (s == 0 && threadIdx.x == 0) {
-      C.status[b] = !(r <= 1.79e308) ? ST_DIVERGED : (r <= C.tol ? ST_CONVERGED : ST_MAX_ITER);
-      C.iters[b] = C.k;
-      C.final_buf[b] = C.k & 1;
-      C.fin[b] = r;
-      C.fin[C.n_inst + b] = sqrt(C.rsq[slot]);
-      atomicSub(C.n_active, 1);
-    }
-    return;
-  }
-  const double alpha = fmin(1.0, __longlong_as_double((long long)C.acand[slot]));
+  return true;
+}
+
+// The decision of iteration C.k for the instances still running, once its
+// launches are done (the host polls the running count after it).
+static __global__ void k_settle(Ctl C) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= C.n_inst || C.status[b] != ST_RUNNING) return;
+  const double r = __longlong_as_double((long long)C.rmax[(C.k % SLOTS) * C.n_inst + b]);
+  if (!(r <= 1.79e308) || r <= C.tol || C.k >= C.max_iter)
+    record_stop(C, b, C.k, !(r <= 1.79e308) ? ST_DIVERGED : (r <= C.tol ? ST_CONVERGED : ST_MAX_ITER),
+                r);
+}
+
+// S_out = S_in - alpha Delta S with iteration C.k's step, one CTA per
+// (instance, stage): the last iterate of a fixed number of iterations whose
+// directions wait for the step (plate).
+static __global__ void __launch_bounds__(256) k_apply(Ctl C, Iter S) {
+  const int2 it = C.work[blockIdx.x];
+  const int b = it.x, s = it.y;
+  const Layout L = C.lay[b];
+  const double alpha =
+      fmin(1.0, __longlong_as_double((long long)C.acand[(C.k % SLOTS) * C.n_inst + b]));
   const long long so = L.s_off + (long long)s * L.nx;
   const long long uo = L.u_off + (long long)s * L.nu;
   for (int t = threadIdx.x; t < L.nx; t += blockDim.x) {
-    S.xout[so + t] = S.xin[so + t] - alpha * S.dx[so + t];
-    S.lout[so + t] = S.lin[so + t] - alpha * S.dl[so + t];
+    S.xout[so + t] = S.xin[so + t] - alpha * S.px[so + t];
+    S.lout[so + t] = S.lin[so + t] - alpha * S.pl[so + t];
   }
   for (int a = threadIdx.x; a < L.nu; a += blockDim.x)
-    S.uout[uo + a] = S.uin[uo + a] - alpha * S.du[uo + a];
+    S.uout[uo + a] = S.uin[uo + a] - alpha * S.pu[uo + a];
 }
 
 // Start iterate into buffer 0 (mode 0 cold, 1 a copy of the current state,
@@ -182,7 +305,7 @@ static __global__ void k_init(const Layout* lay, int n_inst, int mode, const dou
     u[L.u_off + e] = (mode == 0) ? L.u_cold : uc[L.u_off + (long long)ss * L.nu + a];
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < SLOTS; ++q) {
       rmax[q * n_inst + b] = 0ull;
       rsq[q * n_inst + b] = 0.0;
       acand[q * n_inst + b] = (unsigned long long)__double_as_longlong(1.0);
@@ -190,6 +313,16 @@ static __global__ void k_init(const Layout* lay, int n_inst, int mode, const dou
     status[b] = ST_RUNNING;
     if (b == 0) *n_active = n_inst;
   }
+}
+
+// The control words of every slot, cleared.
+static __global__ void k_reset(int n, unsigned long long* rmax, double* rsq,
+                               unsigned long long* acand) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  rmax[i] = 0ull;
+  rsq[i] = 0.0;
+  acand[i] = (unsigned long long)__double_as_longlong(1.0);
 }
 
 // The returned iterate (buffer final_buf[b]) into the current state.
@@ -237,27 +370,45 @@ cudaError_t upload(T* d, const std::vector<T>& v) {
 }
 
 // Device state of the driver: three iterate buffers (two ping-pong, one
-// current state), the direction, the control words and the instance layout.
+// current state), two directions (where the problem asks for them), the
+// control words and the instance layout.
 struct Driver {
   int n = 0;
   std::vector<Layout> lay_h;
   long long n_g = 0, n_x = 0, n_u = 0;  // sum nx (x0), sum N nx, sum N nu
   Layout* lay = nullptr;
+  std::vector<Group> groups;
   int2* work = nullptr;
   int n_work = 0;
   double* x0 = nullptr;  // the solve's start state [n_g]
   double* xb[3] = {nullptr, nullptr, nullptr};
   double* ub[3] = {nullptr, nullptr, nullptr};
   double* lb[3] = {nullptr, nullptr, nullptr};
-  double *dx = nullptr, *du = nullptr, *dl = nullptr;
+  double *dx[2] = {nullptr, nullptr}, *du[2] = {nullptr, nullptr}, *dl[2] = {nullptr, nullptr};
   unsigned long long *rmax = nullptr, *acand = nullptr;
   double *rsq = nullptr, *fin = nullptr;
   int *status = nullptr, *iters = nullptr, *final_buf = nullptr, *n_active = nullptr;
   bool has_state = false;
 };
 
-// Offsets from lay_h[b].{N, nx, nu}; one work item per (instance, stage).
-inline cudaError_t driver_alloc(Driver& d) {
+// An instance's grid: dimension, points per axis and in all, Neumann or not.
+struct GridKind {
+  int dim, m, ng;
+  bool neu;
+};
+
+// The thread groups' shape for stages of ng points, n of them in all.
+inline void shape_group(Group& g) {
+  g.ppt = g.ng_max > 256 ? 2 : 1;
+  g.tps = 32 * ((g.ng_max + 32 * g.ppt - 1) / (32 * g.ppt));
+  // at most 256 threads a CTA (8 named barriers); two CTAs' worth of stages
+  // for each of the 152 SMs before stages share a CTA
+  g.spc = std::max(1, std::min(256 / g.tps, g.n / 304));
+}
+
+// Offsets from lay_h[b].{N, nx, nu}; the work items (instance, stage) by grid
+// kind, even stages first.
+inline cudaError_t driver_alloc(Driver& d, const std::vector<GridKind>& grid, bool directions) {
   d.n = (int)d.lay_h.size();
   d.n_g = d.n_x = d.n_u = 0;
   std::vector<int2> work;
@@ -269,7 +420,24 @@ inline cudaError_t driver_alloc(Driver& d) {
     d.n_x += (long long)L.N * L.nx;
     d.n_u += (long long)L.N * L.nu;
     d.n_g += L.nx;
-    for (int s = 0; s < L.N; ++s) work.push_back(make_int2(b, s));
+  }
+  for (int kind = 0; kind < 4; ++kind) {
+    Group g{};
+    g.neu = kind & 1;
+    g.d2 = kind & 2;
+    g.first = (int)work.size();
+    for (int par = 0; par < 2; ++par) {
+      for (int b = 0; b < d.n; ++b) {
+        if (grid[b].neu != g.neu || (grid[b].dim == 2) != g.d2) continue;
+        g.ng_max = std::max(g.ng_max, grid[b].ng);
+        for (int s = par; s < d.lay_h[b].N; s += 2) work.push_back(make_int2(b, s));
+      }
+      if (par == 0) g.n_even = (int)work.size() - g.first;
+    }
+    g.n = (int)work.size() - g.first;
+    if (g.n == 0) continue;
+    shape_group(g);
+    d.groups.push_back(g);
   }
   d.n_work = (int)work.size();
   cudaError_t e = cudaSuccess;
@@ -282,12 +450,14 @@ inline cudaError_t driver_alloc(Driver& d) {
     A(dalloc(&d.ub[q], d.n_u));
     A(dalloc(&d.lb[q], d.n_x));
   }
-  A(dalloc(&d.dx, d.n_x));
-  A(dalloc(&d.du, d.n_u));
-  A(dalloc(&d.dl, d.n_x));
-  A(dalloc(&d.rmax, 2 * d.n));
-  A(dalloc(&d.acand, 2 * d.n));
-  A(dalloc(&d.rsq, 2 * d.n));
+  for (int q = 0; directions && q < 2; ++q) {
+    A(dalloc(&d.dx[q], d.n_x));
+    A(dalloc(&d.du[q], d.n_u));
+    A(dalloc(&d.dl[q], d.n_x));
+  }
+  A(dalloc(&d.rmax, SLOTS * d.n));
+  A(dalloc(&d.acand, SLOTS * d.n));
+  A(dalloc(&d.rsq, SLOTS * d.n));
   A(dalloc(&d.fin, 2 * d.n));
   A(dalloc(&d.status, d.n));
   A(dalloc(&d.iters, d.n));
@@ -300,7 +470,7 @@ inline cudaError_t driver_alloc(Driver& d) {
 
 inline void driver_free(Driver& d) {
   void* ptrs[] = {d.lay, d.work, d.x0, d.xb[0], d.xb[1], d.xb[2], d.ub[0], d.ub[1], d.ub[2],
-                  d.lb[0], d.lb[1], d.lb[2], d.dx, d.du, d.dl, d.rmax, d.acand, d.rsq, d.fin,
+                  d.lb[0], d.lb[1], d.lb[2], d.dx[0], d.dx[1], d.du[0], d.du[1], d.dl[0], d.dl[1], d.rmax, d.acand, d.rsq, d.fin,
                   d.status, d.iters, d.final_buf, d.n_active};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -326,31 +496,47 @@ inline Ctl make_ctl(const Driver& d, int k, int mode, int max_iter, double tol) 
   return C;
 }
 
-inline Iter make_iter(const Driver& d, int rd) {
+// Launch k's arrays.  Without directions it reads S^k and writes S^{k+1};
+// with them it reads S^{k-1} and Delta S^{k-1} (k = 0: S^0), writes S^k and
+// Delta S^k.  Iterate k is in buffer k & 1 either way.
+inline Iter make_iter(const Driver& d, int k) {
+  const bool dir = d.dx[0] != nullptr;
+  const int rd = dir ? (k > 0 ? (k - 1) & 1 : 0) : k & 1, wr = dir ? k & 1 : (k + 1) & 1;
   Iter S{};
   S.xin = d.xb[rd];
   S.uin = d.ub[rd];
   S.lin = d.lb[rd];
-  S.xout = d.xb[rd ^ 1];
-  S.uout = d.ub[rd ^ 1];
-  S.lout = d.lb[rd ^ 1];
-  S.dx = d.dx;
-  S.du = d.du;
-  S.dl = d.dl;
+  S.xout = d.xb[wr];
+  S.uout = d.ub[wr];
+  S.lout = d.lb[wr];
+  S.px = d.dx[rd];
+  S.pu = d.du[rd];
+  S.pl = d.dl[rd];
+  S.dx = d.dx[k & 1];
+  S.du = d.du[k & 1];
+  S.dl = d.dl[k & 1];
   return S;
 }
 
 inline dim3 inst_grid(const Driver& d) { return dim3(8, (unsigned)d.n); }
 
-// One iteration: the problem's direction kernel(s), dir(C, S) -> cudaError_t,
-// then the update.
-template <class Dir>
-cudaError_t launch_iteration(const Driver& d, const Ctl& C, const Iter& S, Dir& dir,
-                             cudaStream_t st) {
-  cudaError_t e = dir(C, S);
-  if (e != cudaSuccess) return e;
-  k_update<<<d.n_work, 256, 0, st>>>(C, S);
-  return cudaGetLastError();
+// A direction kernel over one range of items, overlapping its start with the
+// previous launch's end.
+template <typename K, typename Args>
+cudaError_t launch_stages(K kernel, size_t smem_per_group, const Range& r, const Args& A,
+                          const Ctl& C, const Iter& S, cudaStream_t st) {
+  if (r.n == 0) return cudaSuccess;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((r.n + r.spc - 1) / r.spc));
+  cfg.blockDim = dim3((unsigned)(r.tps * r.spc));
+  cfg.dynamicSmemBytes = smem_per_group * r.spc;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, A, C, S, r);
 }
 
 // A solve from d.x0 (already on the device): init NMPC_INIT_*; host polls of
@@ -371,8 +557,9 @@ int solve(Driver& d, int init, int max_iter, double tol, int check_every, Dir& d
   int active = d.n;
   for (int k = 0; k <= max_iter;) {
     for (int c = 0; c < check_every && k <= max_iter; ++c, ++k)
-      SDRV_CHECK(launch_iteration(d, make_ctl(d, k, MODE_SOLVE, max_iter, tol), make_iter(d, k & 1),
-                                  dir, st));
+      SDRV_CHECK(dir(make_ctl(d, k, MODE_SOLVE, max_iter, tol), make_iter(d, k)));
+    k_settle<<<(d.n + 127) / 128, 128, 0, st>>>(make_ctl(d, k - 1, MODE_SOLVE, max_iter, tol));
+    SDRV_CHECK(cudaGetLastError());
     SDRV_CHECK(cudaMemcpyAsync(&active, d.n_active, sizeof(int), cudaMemcpyDeviceToHost, st));
     SDRV_CHECK(cudaStreamSynchronize(st));
     if (active == 0) break;
@@ -413,31 +600,26 @@ int iterate(Driver& d, const double* x_in, const double* u_in, const double* lam
   SDRV_CHECK(cudaMemcpyAsync(d.xb[0], x_in, d.n_x * sizeof(double), cudaMemcpyDeviceToDevice, st));
   SDRV_CHECK(cudaMemcpyAsync(d.ub[0], u_in, d.n_u * sizeof(double), cudaMemcpyDeviceToDevice, st));
   SDRV_CHECK(cudaMemcpyAsync(d.lb[0], lam_in, d.n_x * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  double one = 1.0;
-  unsigned long long one_bits;
-  std::memcpy(&one_bits, &one, sizeof(one_bits));
-  std::vector<unsigned long long> aone(2 * d.n, one_bits);
-  for (int it = 0; it < n_iter; ++it) {
-    // slot 0 of the control words serves every iteration
-    SDRV_CHECK(cudaMemsetAsync(d.rmax, 0, 2 * d.n * sizeof(unsigned long long), st));
-    SDRV_CHECK(cudaMemsetAsync(d.rsq, 0, 2 * d.n * sizeof(double), st));
-    SDRV_CHECK(cudaMemcpyAsync(d.acand, aone.data(), aone.size() * sizeof(unsigned long long),
-                               cudaMemcpyHostToDevice, st));
-    SDRV_CHECK(launch_iteration(d, make_ctl(d, 0, MODE_ONESHOT, 0, 0.0), make_iter(d, it & 1), dir,
-                                st));
-    SDRV_CHECK(cudaStreamSynchronize(st));  // aone outlives the copy
+  k_reset<<<(SLOTS * d.n + 127) / 128, 128, 0, st>>>(SLOTS * d.n, d.rmax, d.rsq, d.acand);
+  SDRV_CHECK(cudaGetLastError());
+  for (int k = 0; k < n_iter; ++k)
+    SDRV_CHECK(dir(make_ctl(d, k, MODE_ONESHOT, 0, 0.0), make_iter(d, k)));
+  if (d.dx[0]) {
+    k_apply<<<d.n_work, 256, 0, st>>>(make_ctl(d, n_iter - 1, MODE_ONESHOT, 0, 0.0),
+                                      make_iter(d, n_iter));
+    SDRV_CHECK(cudaGetLastError());
   }
-  const int fb = n_iter & 1;
+  const int fb = n_iter & 1, slot = (n_iter - 1) % SLOTS;
   SDRV_CHECK(cudaMemcpyAsync(x_out, d.xb[fb], d.n_x * sizeof(double), cudaMemcpyDeviceToDevice, st));
   SDRV_CHECK(cudaMemcpyAsync(u_out, d.ub[fb], d.n_u * sizeof(double), cudaMemcpyDeviceToDevice, st));
   SDRV_CHECK(cudaMemcpyAsync(lam_out, d.lb[fb], d.n_x * sizeof(double), cudaMemcpyDeviceToDevice, st));
   if (out) {
     std::vector<unsigned long long> rm(d.n), ac(d.n);
     std::vector<double> rs(d.n);
-    SDRV_CHECK(cudaMemcpyAsync(rm.data(), d.rmax, d.n * sizeof(unsigned long long),
+    SDRV_CHECK(cudaMemcpyAsync(rm.data(), d.rmax + (size_t)slot * d.n, d.n * sizeof(unsigned long long),
                                cudaMemcpyDeviceToHost, st));
-    SDRV_CHECK(cudaMemcpyAsync(rs.data(), d.rsq, d.n * sizeof(double), cudaMemcpyDeviceToHost, st));
-    SDRV_CHECK(cudaMemcpyAsync(ac.data(), d.acand, d.n * sizeof(unsigned long long),
+    SDRV_CHECK(cudaMemcpyAsync(rs.data(), d.rsq + (size_t)slot * d.n, d.n * sizeof(double), cudaMemcpyDeviceToHost, st));
+    SDRV_CHECK(cudaMemcpyAsync(ac.data(), d.acand + (size_t)slot * d.n, d.n * sizeof(unsigned long long),
                                cudaMemcpyDeviceToHost, st));
     SDRV_CHECK(cudaStreamSynchronize(st));
     for (int b = 0; b < d.n; ++b) {
@@ -459,66 +641,39 @@ inline int get_state(const Driver& d, double* x, double* u, double* lam, cudaStr
   return NMPC_OK;
 }
 
-// Row p of the grid Laplacian (dim 1 or 2, m points per axis) as (column,
-// weight) pairs: zero Neumann by mirrored fictitious points (a missing
-// neighbour is replaced by the inner one, so that neighbour's weight
-// doubles; the points include the boundary, spacing 1/(m-1)), zero Dirichlet
-// by dropping neighbours outside (interior points, spacing 1/(m+1)).
-inline void laplacian_rows(int dim, int m, int bc,
-                           std::vector<std::vector<std::pair<int, double>>>& rows) {
-  const int ng = dim == 2 ? m * m : m;
+// The grid Laplacian's neighbour weight, 1 / spacing^2: zero Neumann grids
+// (bc 0) include the boundary (spacing 1 / (m - 1)), zero Dirichlet ones hold
+// the interior points (spacing 1 / (m + 1)).
+inline double neighbour_weight(int m, int bc) {
   const double dp = bc == 0 ? 1.0 / (m - 1) : 1.0 / (m + 1);
-  const double w = 1.0 / (dp * dp);
-  rows.assign(ng, {});
-  auto add = [&](int p, int c, double v) {
-    for (auto& e : rows[p])
-      if (e.first == c) {
-        e.second += v;
-        return;
-      }
-    rows[p].push_back({c, v});
-  };
-  for (int p = 0; p < ng; ++p) {
-    const int ix = p % m, iy = p / m;
-    add(p, p, -2.0 * dim * w);
-    for (int axis = 0; axis < dim; ++axis) {
-      const int i = axis == 0 ? ix : iy;
-      for (int dir = -1; dir <= 1; dir += 2) {
-        int j = i + dir;
-        if (j < 0 || j >= m) {
-          if (bc == 1) continue;  // Dirichlet: zero outside
-          j = i - dir;            // Neumann: the mirrored point
-        }
-        add(p, axis == 0 ? iy * m + j : j * m + ix, w);
-      }
-    }
-  }
+  return 1.0 / (dp * dp);
 }
 
-// ELL tables (ELL entries per point; unused slots: the point itself with
-// weight 0) of L and L^T, and the diagonal of L, appended to the vectors.
-constexpr int ELL = 5;
-inline void append_ell(int dim, int m, int bc, std::vector<int>& Lc, std::vector<double>& Lv,
-                       std::vector<int>& Ltc, std::vector<double>& Ltv, std::vector<double>& Ld) {
-  std::vector<std::vector<std::pair<int, double>>> rows;
-  laplacian_rows(dim, m, bc, rows);
-  const int ng = (int)rows.size();
-  std::vector<std::vector<std::pair<int, double>>> trows(ng);
-  for (int p = 0; p < ng; ++p)
-    for (auto& e : rows[p]) trows[e.first].push_back({p, e.second});
-  for (int p = 0; p < ng; ++p) {
-    double diag = 0.0;
-    for (int e = 0; e < ELL; ++e) {
-      const bool on = e < (int)rows[p].size();
-      Lc.push_back(on ? rows[p][e].first : p);
-      Lv.push_back(on ? rows[p][e].second : 0.0);
-      if (on && rows[p][e].first == p) diag = rows[p][e].second;
-      const bool ton = e < (int)trows[p].size();
-      Ltc.push_back(ton ? trows[p][e].first : p);
-      Ltv.push_back(ton ? trows[p][e].second : 0.0);
+// Per grid point the actuator on it, or minus the number of grid steps to the
+// nearest one.
+inline std::vector<int> actuator_map(int dim, int m, int n_u, const int* act_cell) {
+  const int ng = dim == 2 ? m * m : m;
+  std::vector<int> of(ng, 0), front;
+  for (int a = 0; a < n_u; ++a) front.push_back(act_cell[a]);
+  std::vector<char> seen(ng, 0);
+  for (int p : front) seen[p] = 1;
+  for (int dist = 1; !front.empty(); ++dist) {
+    std::vector<int> next;
+    for (int p : front) {
+      const int ix = p % m, iy = p / m;
+      const int q[4] = {ix > 0 ? p - 1 : -1, ix < m - 1 ? p + 1 : -1,
+                        dim == 2 && iy > 0 ? p - m : -1, dim == 2 && iy < m - 1 ? p + m : -1};
+      for (int c : q)
+        if (c >= 0 && !seen[c]) {
+          seen[c] = 1;
+          of[c] = -dist;
+          next.push_back(c);
+        }
     }
-    Ld.push_back(diag);
+    front = next;
   }
+  for (int a = 0; a < n_u; ++a) of[act_cell[a]] = a;
+  return of;
 }
 
 }  // namespace stage_drv

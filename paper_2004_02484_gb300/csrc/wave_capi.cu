@@ -2,22 +2,17 @@
 // on a w_tt + b w_t = c Lap w - kappa w^3 + point forces (Sec. 2, eq. 1 with
 // a != 0), state x = (W, V = dW/dt) (eq. 5).
 //
-// One iteration is two kernels (three with the red-black upper layer):
-//   k_wave_dir  one CTA per (instance, stage) loads the stage's W, V,
-//     lambda_W, lambda_V into shared memory, evaluates K_i (eq. 9) and its
-//     norms, the stage's coefficients, and the lower layer (eqs. 21-24 with
-//     the u-iteration of Sec. 5.2) whose F_x and F_x^T solves eliminate v6
-//     (eq. 25): E v7 = b7 + h grad_W g b6 and E^T v9 = b9 + h b8 by n_lo
-//     pointwise Jacobi sweeps, v6 = h v7 - b6, v8 = h grad_W g^T v9 - b8.
-//     It stores the direction Delta s_i.  Red-black: half 0 runs the even
-//     stages, half 1 the odd ones with the even neighbours' directions in
-//     its right-hand side (eq. 18's form).
-//   k_update (stage_driver.cuh)  the convergence decision and S^{k+1} =
-//     S^k - Delta S (no bounds: the full step).
+// One launch of k_wave_dir is one iteration (two with the red-black upper
+// layer: half 0 the even stages, half 1 the odd ones with the even
+// neighbours' new x_{i-1}, lambda_{i+1} in the right-hand side, eq. 18's
+// form).  A group of threads per (instance, stage), one or two points a
+// thread: K_i (eq. 9) and its norms, the stage's coefficients, and the lower
+// layer (eqs. 21-24 with the u-iteration of Sec. 5.2) whose F_x and F_x^T
+// solves eliminate v6 (eq. 25): E v7 = b7 + h grad_W g b6 and E^T v9 = b9 +
+// h b8 by n_lo pointwise Jacobi sweeps, v6 = h v7 - b6, v8 = h grad_W g^T v9
+// - b8; then S^{k+1} = S^k - Delta S (no bounds: the full step).
 // grad_W g = (c L - 3 kappa diag(W^2)) / a and grad_V g = -(b / a) I, so E
-// has the stencil of L scaled by h^2 c / a off the diagonal.  The Laplacian
-// and its transpose are host-built tables of five (column, weight) entries
-// per point.  Everything is float64.
+// has the stencil of L scaled by h^2 c / a off the diagonal.
 #include <new>
 
 #include "../../include/nmpc_wave.h"
@@ -26,265 +21,295 @@
 namespace wave_dev {
 
 using stage_drv::Ctl;
-using stage_drv::ELL;
 using stage_drv::Iter;
 using stage_drv::Layout;
 constexpr int THREADS = 256;
 constexpr int MAX_NU = 64;
-// shared-memory fields of n_g values in k_wave_dir: float64 grid values and
-// costates, the lower layer's fields in its type T
-constexpr int F64_FIELDS = 4, T_FIELDS = 18;
 constexpr int NG_PER_THREAD = (NMPC_WAVE_MAX_POINTS + THREADS - 1) / THREADS;  // the plant's points
 
 struct WInst {
-  int dim, m, ng, nu, N;
+  int dim, m, ng, nu, N, neu;
   long long w_off;  // w_ref
   long long a_off;  // u_ref, actuator table
   long long t_off;  // per-point tables
   double h, a, b, c, kappa, gain, q, qv, r, qf, gamma;
+  double lw;        // the Laplacian's neighbour weight 1 / spacing^2
+  // derived (the float64 pipe is the scarce one): 1 / a; c lw / a; kappa / a;
+  // b / a; gain / a; h^2 c lw / a; E's diagonal at W = 0 and its 3 h^2;
+  // h gain / a; 1 / (h r + gamma)
+  double ia, cl, kia, bia, gia, se, ed0, hh3, fu, rauu;
 };
+
+// The derived fields.
+inline void derive(WInst& I) {
+  const double d2 = 2.0 * I.dim;
+  I.ia = 1.0 / I.a;
+  I.cl = I.c * I.ia * I.lw;
+  I.kia = I.kappa * I.ia;
+  I.bia = I.b * I.ia;
+  I.gia = I.gain * I.ia;
+  I.se = I.h * I.h * I.cl;
+  I.ed0 = -(1.0 + I.h * I.bia) - d2 * I.se;
+  I.hh3 = 3.0 * I.h * I.h;
+  I.fu = I.h * I.gia;
+  I.rauu = 1.0 / (I.h * I.r + I.gamma);
+}
 
 struct WArgs {
   const WInst* inst;
-  const int* act_of;  // [sum ng]: actuator index at the point, or -1
+  const int* act_of;  // [sum ng]: actuator index at the point, or -(grid steps to the nearest one)
   const int* act_pt;  // [sum nu]: grid point of actuator a
-  const int* Lc;      // [sum ng][ELL] columns of L (unused slots: the point itself, weight 0)
-  const double* Lv;
-  const int* Ltc;     // the same for L^T
-  const double* Ltv;
-  const double* Ld;   // [sum ng] L[p][p]
-  const float* Lvf;   // float32 copies of Lv, Ltv, Ld (mixed precision)
-  const float* Ltvf;
-  const float* Ldf;
   const double* x0;
   const double* wref;
   const double* uref;
   int n_lo, n_u_it, rb, half;
 };
 
+// Shared memory of one stage: W and the (scaled) lambda_V in float64, two
+// exchange fields of the lower layer's type; each with a zero at index ng.
+template <typename T>
+__host__ __device__ constexpr size_t stage_bytes(int ng) {
+  return (((size_t)(ng + 1) * (2 * sizeof(double) + 2 * sizeof(T))) + 15) & ~size_t(15);
+}
+
+// What bounds it: the float64 pipe (2 lanes a clock a SM; the residual, the
+// coefficients and, in NMPC_FP64, the lower layer run there), so the layout
+// saves float64 instructions first.  A thread keeps its points' rows and
+// coefficients in registers and exchanges only the field that a stencil reads
+// (one barrier each, two alternating buffers); neighbours are found from the
+// grid (4 additions and one multiply-add a stencil, where a table of five
+// weights cost five multiply-adds and ten loads); the diagonal's reciprocal is
+// taken once a point (a division each sweep before); h grad_W g b6 is common
+// to every u-iteration, v8 is needed by the last one only; the maximum norm
+// is taken on integers.  With n_lo = 2 the u-iterations after the first
+// recompute only the points that a control can reach (2 grid steps for v9):
+// all others keep the bits that they would get again.  256 membranes of
+// 32x32, N = 10, float64: 81.2 -> 25.9 ms a solve; 256 strings of 64 points,
+// N = 20, mixed, red-black: 21.3 -> 4.6 ms (with four stages a CTA).
 // The lower layer runs in T: float64, or float32 in mixed precision (the
 // residual, the coefficients and the update stay float64, so the fixed point
-// is the float64 root); WT holds W in T for the lower layer's products.
-template <typename T>
-struct Fields {
-  double *W, *V, *LW, *LV;
-  T *WT, *ED, *AXW, *K1W, *K1V, *K3W, *K3V;
-  T *B6, *B7, *B8, *B9, *T_, *C0, *C1, *Y6, *Y7, *Y8, *Y9;
-};
-
-template <typename V>
-struct Stencil {
-  const int *Lc, *Ltc;
-  const V *Lv, *Ltv, *Ld;
-  __device__ V lap(const V* v, int p) const {  // (L v)(p)
-    V acc = V(0);
-#pragma unroll
-    for (int e = 0; e < ELL; ++e) acc += Lv[p * ELL + e] * v[Lc[p * ELL + e]];
-    return acc;
-  }
-  __device__ V lapT(const V* v, int p) const {  // (L^T v)(p)
-    V acc = V(0);
-#pragma unroll
-    for (int e = 0; e < ELL; ++e) acc += Ltv[p * ELL + e] * v[Ltc[p * ELL + e]];
-    return acc;
-  }
-};
-
-// The stencil tables in type V.
-template <typename V>
-__device__ __forceinline__ const V* tab(const double* d, const float* f);
-template <>
-__device__ __forceinline__ const double* tab<double>(const double* d, const float*) { return d; }
-template <>
-__device__ __forceinline__ const float* tab<float>(const double*, const float* f) { return f; }
-
-// n_lo Jacobi sweeps from zero on E v = T (transposed: E^T), result in the
-// returned buffer (C0 or C1).  E = diag ED + (h^2 c / a)(L - diag L).
-template <typename T>
-__device__ T* jacobi_E(const WArgs& A, const WInst& I, const Stencil<T>& L, const Fields<T>& f,
-                       bool transposed) {
-  const int ng = I.ng;
-  const T s = (T)(I.h * I.h * I.c / I.a);
-  T* cur = f.C0;
-  T* nxt = f.C1;
-  for (int p = threadIdx.x; p < ng; p += THREADS) cur[p] = f.T_[p] / f.ED[p];
-  __syncthreads();
-  for (int sw = 1; sw < A.n_lo; ++sw) {
-    for (int p = threadIdx.x; p < ng; p += THREADS) {
-      const T lv = transposed ? L.lapT(cur, p) : L.lap(cur, p);
-      nxt[p] = (f.T_[p] - s * (lv - L.Ld[p] * cur[p])) / f.ED[p];
-    }
-    __syncthreads();
-    T* t = cur;
-    cur = nxt;
-    nxt = t;
-  }
-  return cur;
-}
-
-// P^{-1} (eq. 24): F_x (Y6, Y7) = (B6, B7), then F_x^T (Y8, Y9) = (B8, B9) -
-// A_xx (Y6, Y7), both by the v6 elimination (eq. 25).  B8 is overwritten.
-template <typename T>
-__device__ void p_inv(const WArgs& A, const WInst& I, const Stencil<T>& L, const Fields<T>& f) {
-  const int ng = I.ng;
-  const T h = (T)I.h, ia = (T)(1.0 / I.a), axv = (T)(I.h * I.qv), c = (T)I.c;
-  const T k3 = (T)(3.0 * I.kappa);
-  // E v7 = b7 + h grad_W g b6
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    const T gw = (c * L.lap(f.B6, p) - k3 * f.WT[p] * f.WT[p] * f.B6[p]) * ia;
-    f.T_[p] = f.B7[p] + h * gw;
-  }
-  __syncthreads();
-  const T* v7 = jacobi_E<T>(A, I, L, f, false);
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    f.Y7[p] = v7[p];
-    f.Y6[p] = h * v7[p] - f.B6[p];
-  }
-  __syncthreads();
-  // (b8, b9) = (B8, B9) - A_xx (Y6, Y7); E^T v9 = b9 + h b8
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    const T b8 = f.B8[p] - f.AXW[p] * f.Y6[p];
-    f.B8[p] = b8;
-    f.T_[p] = (f.B9[p] - axv * f.Y7[p]) + h * b8;
-  }
-  __syncthreads();
-  const T* v9 = jacobi_E<T>(A, I, L, f, true);
-  for (int p = threadIdx.x; p < ng; p += THREADS) f.Y9[p] = v9[p];
-  __syncthreads();
-  // v8 = h grad_W g^T v9 - b8
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    const T gwt = (c * L.lapT(f.Y9, p) - k3 * f.WT[p] * f.WT[p] * f.Y9[p]) * ia;
-    f.Y8[p] = h * gwt - f.B8[p];
-  }
-  __syncthreads();
-}
-
-template <typename T>
-__global__ void __launch_bounds__(THREADS) k_wave_dir(WArgs A, Ctl C, Iter S) {
-  const int2 it = C.work[blockIdx.x];
+// is the float64 root).
+template <typename T, int PPT, bool NEU, bool D2>
+__global__ void __launch_bounds__(PPT == 1 ? 256 : 512, PPT == 1 ? 3 : 2)
+    k_wave_dir(WArgs A, Ctl C, Iter S, stage_drv::Range R) {
+  extern __shared__ __align__(16) double smem[];
+  __shared__ stage_drv::WarpNorms red[16];
+  __shared__ T sK2[8 * MAX_NU], sV3[8 * MAX_NU];  // per control, by its point's thread only
+  stage_drv::pdl_trigger();
+  const int g = threadIdx.x / R.tps, t = threadIdx.x - g * R.tps;
+  const int item = blockIdx.x * R.spc + g;
+  stage_drv::pdl_wait();
+  if (item >= R.n) return;
+  const int2 it = C.work[R.first + item];
   const int b = it.x, s = it.y;
-  if (A.rb && ((s & 1) != A.half)) return;
-  if (stage_drv::finished(C, b)) return;
-  const WInst I = A.inst[b];
-  const Layout Ly = C.lay[b];
+  bool norms_only;
+  if (!stage_drv::begin_stage(C, b, s, t, norms_only)) return;
+  const WInst& I = A.inst[b];
+  const Layout& Ly = C.lay[b];
   const int ng = I.ng, nu = I.nu, nx = 2 * ng;
   const bool last = (s == I.N - 1);
-  extern __shared__ double smem[];
-  Fields<T> f;
-  {
-    double** fd[F64_FIELDS] = {&f.W, &f.V, &f.LW, &f.LV};
-    for (int q = 0; q < F64_FIELDS; ++q) *fd[q] = smem + (size_t)q * ng;
-    T* base = reinterpret_cast<T*>(smem + (size_t)F64_FIELDS * ng);
-    T** ft[T_FIELDS] = {&f.WT, &f.ED, &f.AXW, &f.K1W, &f.K1V, &f.K3W, &f.K3V, &f.B6, &f.B7,
-                        &f.B8, &f.B9, &f.T_,  &f.C0,  &f.C1,  &f.Y6,  &f.Y7,  &f.Y8, &f.Y9};
-    for (int q = 0; q < T_FIELDS; ++q) *ft[q] = base + (size_t)q * ng;
-  }
-  __shared__ double sU[MAX_NU], red[64];
-  __shared__ T sK2[MAX_NU], sV3[MAX_NU];
-  // the residual's stencil (float64) and the lower layer's (T)
-  Stencil<double> L{A.Lc + I.t_off * ELL, A.Ltc + I.t_off * ELL, A.Lv + I.t_off * ELL,
-                    A.Ltv + I.t_off * ELL, A.Ld + I.t_off};
-  Stencil<T> LT{A.Lc + I.t_off * ELL, A.Ltc + I.t_off * ELL,
-                tab<T>(A.Lv, A.Lvf) + I.t_off * ELL, tab<T>(A.Ltv, A.Ltvf) + I.t_off * ELL,
-                tab<T>(A.Ld, A.Ldf) + I.t_off};
+  // this launch's stage size sets the fields' distance (ng_max would do too)
+  double* fA = smem + (size_t)g * (stage_bytes<T>(R.ng_max) / sizeof(double));
+  double* fB = fA + (ng + 1);
+  T* fC = reinterpret_cast<T*>(fB + (ng + 1));
+  T* fD = fC + (ng + 1);
   const int* act_of = A.act_of + I.t_off;
-  const int* apt = A.act_pt + I.a_off;
   const long long so = Ly.s_off + (long long)s * nx;
   const long long uo = Ly.u_off + (long long)s * nu;
-  const double h = I.h, ia = 1.0 / I.a;
+  const double h = I.h;
+  constexpr double d2 = D2 ? 4.0 : 2.0;  // the Laplacian's centre: -2 dim lw
+  const bool gs = A.rb && A.half == 1;
 
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    f.W[p] = S.xin[so + p];
-    f.V[p] = S.xin[so + ng + p];
-    f.LW[p] = S.lin[so + p];
-    f.LV[p] = S.lin[so + ng + p];
+  stage_drv::Nbr<NEU, D2> nb[PPT];
+  int ap[PPT];
+  bool on[PPT];
+  if (t == 0) {
+    fA[ng] = fB[ng] = 0.0;
+    fC[ng] = fD[ng] = T(0);
   }
-  for (int a = threadIdx.x; a < nu; a += THREADS) sU[a] = S.uin[uo + a];
-  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < PPT; ++j) {
+    const int p = t + j * R.tps;
+    on[j] = p < ng;
+    nb[j].set(p, I.m, ng);
+    ap[j] = on[j] ? act_of[p] : -0x7fffffff;
+    if (on[j]) {
+      fA[p] = __ldcg(S.xin + so + p);
+      fB[p] = nb[j].scale(__ldcg(S.lin + so + ng + p));
+    }
+  }
+  stage_drv::group_sync(g, R.tps);
 
   // K_i (eq. 9), coefficients, norms
-  double mx = 0.0, sq = 0.0;
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    const double w = f.W[p], v = f.V[p], lw = f.LW[p], lv = f.LV[p];
+  unsigned long long mx = 0ull;
+  double sq = 0.0;
+  T k1w[PPT], r7[PPT], k3w[PPT], k3v[PPT], rED[PPT], axw[PPT], kw3[PPT];
+  const double cl = I.cl, bia = I.bia, hqf = last ? h * I.qf : 0.0;
+#pragma unroll
+  for (int j = 0; j < PPT; ++j) {
+    const int p = t + j * R.tps;
+    k1w[j] = r7[j] = k3w[j] = k3v[j] = rED[j] = axw[j] = kw3[j] = T(0);
+    if (!on[j]) continue;
+    const double w = fA[p], lv = nb[j].unscale(fB[p]);
+    const double v = __ldcg(S.xin + so + ng + p), lw = __ldcg(S.lin + so + p);
     const double wr = A.wref[I.w_off + p];
-    const int ap = act_of[p];
-    const double force = ap >= 0 ? I.gain * sU[ap] : 0.0;
-    const double g = (I.c * L.lap(f.W, p) - I.b * v - I.kappa * w * w * w + force) * ia;
-    const double wprev = (s == 0) ? A.x0[Ly.g_off + p] : S.xin[so - nx + p];
-    const double vprev = (s == 0) ? A.x0[Ly.g_off + ng + p] : S.xin[so - nx + ng + p];
-    const double lwn = last ? h * I.qf * (w - wr) : S.lin[so + nx + p];
-    const double lvn = last ? 0.0 : S.lin[so + nx + ng + p];
-    const double ltv = L.lapT(f.LV, p);  // (L^T lambda_V)(p)
-    const double K1W = wprev - w + h * v;
-    const double K1V = vprev - v + h * g;
-    const double K3W = lwn - lw + h * (I.q * (w - wr) + (I.c * ltv - 3.0 * I.kappa * w * w * lv) * ia);
-    const double K3V = lvn - lv + h * (I.qv * v + lw - I.b * ia * lv);
-    mx = stage_drv::nan_max(mx, stage_drv::nan_max(stage_drv::nan_max(fabs(K1W), fabs(K1V)),
-                                                   stage_drv::nan_max(fabs(K3W), fabs(K3V))));
+    const double* prev = (s == 0) ? A.x0 + Ly.g_off + p : S.xin + so - nx + p;
+    const double wp = __ldcg(prev), vp = __ldcg(prev + ng);
+    const double dw = w - wr;
+    const double lwn = last ? hqf * dw : __ldcg(S.lin + so + nx + p);
+    const double lvn = last ? 0.0 : __ldcg(S.lin + so + nx + ng + p);
+    const double lap = nb[j].sum(fA) - d2 * w;             // (L W)(p) / lw
+    const double lapt = nb[j].unscale(nb[j].sum(fB)) - d2 * lv;  // (L^T lambda_V)(p) / lw
+    const double kw = I.kia * w, kww = kw * w;
+    double gg = cl * lap - bia * v - kww * w;
+    double u = 0.0;
+    if (ap[j] >= 0) {
+      u = __ldcg(S.uin + uo + ap[j]);
+      gg += I.gia * u;
+    }
+    const double K1W = wp - w + h * v;
+    const double K1V = vp - v + h * gg;
+    const double kww3 = 3.0 * kww;
+    const double K3W = lwn - lw + h * (I.q * dw + (cl * lapt - kww3 * lv));
+    const double K3V = lvn - lv + h * (I.qv * v + lw - bia * lv);
+    mx = max(mx, max(max(stage_drv::abs_bits(K1W), stage_drv::abs_bits(K1V)),
+                     max(stage_drv::abs_bits(K3W), stage_drv::abs_bits(K3V))));
     sq += K1W * K1W + K1V * K1V + K3W * K3W + K3V * K3V;
-    // red-black half 1: the right-hand side takes the even neighbours'
-    // directions (state rows: M_L Delta x_{i-1}; costate rows: M_U Delta
-    // lambda_{i+1}); the norms above stay those of K(S^k)
-    double k1w = K1W, k1v = K1V, k3w = K3W, k3v = K3V;
-    if (A.rb && A.half == 1) {
+    if (ap[j] >= 0) {
+      const double K2 = h * (I.r * (u - A.uref[I.a_off + ap[j]]) + I.gia * lv);
+      mx = max(mx, stage_drv::abs_bits(K2));
+      sq += K2 * K2;
+      sK2[g * MAX_NU + ap[j]] = (T)K2;
+      sV3[g * MAX_NU + ap[j]] = T(0);
+    }
+    // red-black half 1: the right-hand side takes the even neighbours' new
+    // x_{i-1}, lambda_{i+1} (half 0 has written them to the other buffer);
+    // the norms above stay those of K(S^k)
+    double c1w = K1W, c1v = K1V, c3w = K3W, c3v = K3V;
+    if (gs) {
       if (s > 0) {
-        k1w -= S.dx[so - nx + p];
-        k1v -= S.dx[so - nx + ng + p];
+        c1w += __ldcg(S.xout + so - nx + p) - wp;
+        c1v += __ldcg(S.xout + so - nx + ng + p) - vp;
       }
       if (!last) {
-        k3w -= S.dl[so + nx + p];
-        k3v -= S.dl[so + nx + ng + p];
+        c3w += __ldcg(S.lout + so + nx + p) - lwn;
+        c3v += __ldcg(S.lout + so + nx + ng + p) - lvn;
       }
     }
-    f.K1W[p] = (T)k1w;
-    f.K1V[p] = (T)k1v;
-    f.K3W[p] = (T)k3w;
-    f.K3V[p] = (T)k3v;
-    f.WT[p] = (T)w;
+    k1w[j] = (T)c1w;
+    r7[j] = (T)c1v;
+    k3w[j] = (T)c3w;
+    k3v[j] = (T)c3v;
+    kw3[j] = (T)kww3;
     // E's diagonal: h grad_V g - 1 + h^2 grad_W g at (p, p)
-    f.ED[p] = (T)(-(1.0 + h * I.b * ia) + h * h * (I.c * L.Ld[p] - 3.0 * I.kappa * w * w) * ia);
-    f.AXW[p] = (T)(h * (I.q - 6.0 * I.kappa * w * lv * ia) + (last ? h * I.qf : 0.0));
+    rED[j] = stage_drv::rcp((T)(I.ed0 - I.hh3 * kww));
+    axw[j] = (T)(h * (I.q - 6.0 * kw * lv) + hqf);
+    fD[p] = k1w[j];
   }
-  __syncthreads();
-  for (int a = threadIdx.x; a < nu; a += THREADS) {
-    const double K2 = h * (I.r * (sU[a] - A.uref[I.a_off + a]) + I.gain * ia * f.LV[apt[a]]);
-    mx = stage_drv::nan_max(mx, fabs(K2));
-    sq += K2 * K2;
-    sK2[a] = (T)K2;
-    sV3[a] = T(0);
-  }
-  __syncthreads();
-  stage_drv::block_max_sum(mx, sq, red, THREADS);
-  if (stage_drv::publish_norms(C, b, mx, sq)) return;  // norms only
+  stage_drv::warp_norms(mx, sq, red);
+  stage_drv::group_sync(g, R.tps);
+  if (t == 0) stage_drv::publish_norms(C, b, red, R.tps);
+  if (norms_only) return;
 
-  // u fixed-point iteration (Sec. 5.2): y = P^{-1}(F_u v3 - b1, -b2),
-  // v3 = (b3 + F_u^T y_lambda) / A_uu from v3 = 0, then the final
-  // P^{-1}(b1 - F_u v3, b2).  F_u = [0; h B / a]; A_uu = h r + gamma.
-  const T fu = (T)(h * I.gain * ia), auu = (T)(h * I.r + I.gamma);
+  // u fixed-point iteration (Sec. 5.2) on the direction y = P^{-1}(K_1 - F_u
+  // v3, K_3): v3 = (K_2 - F_u^T y_lambda) / A_uu from v3 = 0, then the last y.
+  // F_u = [0; h B / a]; A_uu = h r + gamma.
+  const T hT = (T)h, clT = (T)cl, sT = (T)I.se, d2T = (T)d2, axv = (T)(h * I.qv);
+  const T fu = (T)I.fu, rauu = (T)I.rauu;
+#pragma unroll
+  for (int j = 0; j < PPT; ++j)  // K1V + h grad_W g K1W
+    r7[j] += hT * (clT * (nb[j].sum(fD) - d2T * k1w[j]) - kw3[j] * k1w[j]);
+  T v7[PPT], t9[PPT], v9[PPT];
+#pragma unroll
+  for (int j = 0; j < PPT; ++j) v7[j] = t9[j] = v9[j] = T(0);
+  const int n_lo = A.n_lo;
+  T *ex = fC, *ex2 = fD;  // the next exchange's field, the other one
   for (int itu = 0; itu <= A.n_u_it; ++itu) {
-    const bool final_pass = (itu == A.n_u_it);
-    for (int p = threadIdx.x; p < ng; p += THREADS) {
-      const int ap = act_of[p];
-      const T fuv = ap >= 0 ? fu * sV3[ap] : T(0);
-      f.B6[p] = final_pass ? f.K1W[p] : -f.K1W[p];
-      f.B7[p] = final_pass ? f.K1V[p] - fuv : fuv - f.K1V[p];
-      f.B8[p] = final_pass ? f.K3W[p] : -f.K3W[p];
-      f.B9[p] = final_pass ? f.K3V[p] : -f.K3V[p];
+    // the points that this u-iteration can change: all of them at first; with
+    // n_lo = 2 the two fields hold the same sweeps every time (C the first
+    // of E, D the first of E^T), so later ones store and recompute the points
+    // at most 0, 1, 2 grid steps from an actuator
+    const int near0 = (itu == 0 || n_lo != 2) ? 0x7fffffff : 0;
+    const int near1 = near0 ? near0 : 1, near2 = near0 ? near0 : 2;
+    T rhs[PPT], c[PPT];
+#pragma unroll
+    for (int j = 0; j < PPT; ++j) {
+      rhs[j] = ap[j] >= 0 ? r7[j] - fu * sV3[g * MAX_NU + ap[j]] : r7[j];
+      c[j] = rhs[j] * rED[j];
     }
-    __syncthreads();
-    p_inv<T>(A, I, LT, f);
-    if (final_pass) break;
-    for (int a = threadIdx.x; a < nu; a += THREADS) sV3[a] = (sK2[a] + fu * f.Y9[apt[a]]) / auu;
-    __syncthreads();
+    for (int sw = 1; sw < n_lo; ++sw) {  // E v7 = r7 - F_u v3
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+        if (on[j] && -ap[j] <= near0) ex[t + j * R.tps] = c[j];
+      stage_drv::group_sync(g, R.tps);
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+        if (-ap[j] <= near1) c[j] = (rhs[j] - sT * nb[j].sum(ex)) * rED[j];
+      T* x = ex;
+      ex = ex2;
+      ex2 = x;
+    }
+#pragma unroll
+    for (int j = 0; j < PPT; ++j)
+      if (-ap[j] <= near1) {
+        v7[j] = c[j];
+        const T v6 = hT * c[j] - k1w[j];
+        t9[j] = (k3v[j] - axv * c[j]) + hT * (k3w[j] - axw[j] * v6);
+        c[j] = t9[j] * rED[j];
+      }
+    for (int sw = 1; sw < n_lo; ++sw) {  // E^T v9 = b9 + h b8
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+        if (on[j] && -ap[j] <= near1) ex[t + j * R.tps] = nb[j].scale(c[j]);
+      stage_drv::group_sync(g, R.tps);
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+        if (-ap[j] <= near2) c[j] = (t9[j] - sT * nb[j].unscale(nb[j].sum(ex))) * rED[j];
+      T* x = ex;
+      ex = ex2;
+      ex2 = x;
+    }
+#pragma unroll
+    for (int j = 0; j < PPT; ++j) {
+      if (-ap[j] <= near2) v9[j] = c[j];
+      if (itu < A.n_u_it && ap[j] >= 0)
+        sV3[g * MAX_NU + ap[j]] = (sK2[g * MAX_NU + ap[j]] - fu * v9[j]) * rauu;
+    }
   }
-  // direction (Delta x, Delta u, Delta lambda) = (v5, v3, v4)
-  for (int p = threadIdx.x; p < ng; p += THREADS) {
-    S.dx[so + p] = (double)f.Y6[p];
-    S.dx[so + ng + p] = (double)f.Y7[p];
-    S.dl[so + p] = (double)f.Y8[p];
-    S.dl[so + ng + p] = (double)f.Y9[p];
+  // v8 = h grad_W g^T v9 - b8, and S^{k+1} = S^k - (v5, v3, v4)
+#pragma unroll
+  for (int j = 0; j < PPT; ++j)
+    if (on[j]) ex[t + j * R.tps] = nb[j].scale(v9[j]);
+  stage_drv::group_sync(g, R.tps);
+#pragma unroll
+  for (int j = 0; j < PPT; ++j) {
+    const int p = t + j * R.tps;
+    if (!on[j]) continue;
+    const T gwt = clT * (nb[j].unscale(nb[j].sum(ex)) - d2T * v9[j]) - kw3[j] * v9[j];
+    const T v6 = hT * v7[j] - k1w[j];
+    const T v8 = hT * gwt - (k3w[j] - axw[j] * v6);
+    S.xout[so + p] = fA[p] - (double)v6;
+    S.xout[so + ng + p] = __ldcg(S.xin + so + ng + p) - (double)v7[j];
+    S.lout[so + p] = __ldcg(S.lin + so + p) - (double)v8;
+    S.lout[so + ng + p] = nb[j].unscale(fB[p]) - (double)v9[j];
+    if (ap[j] >= 0)
+      S.uout[uo + ap[j]] = __ldcg(S.uin + uo + ap[j]) - (double)sV3[g * MAX_NU + ap[j]];
   }
-  for (int a = threadIdx.x; a < nu; a += THREADS) S.du[uo + a] = (double)sV3[a];
+}
+
+// (L v)(p) over a stage's grid, one axis after the other.
+__device__ __forceinline__ double lap_at(const WInst& I, const double* v, int p) {
+  double acc = -2.0 * I.dim * v[p];
+  for (int axis = 0; axis < I.dim; ++axis) {
+    const int st = axis ? I.m : 1, i = axis ? p / I.m : p % I.m;
+    const bool lo = i > 0, hi = i < I.m - 1;
+    if (I.neu) {  // the mirrored point
+      acc += v[lo ? p - st : p + st] + v[hi ? p + st : p - st];
+    } else {
+      acc += (lo ? v[p - st] : 0.0) + (hi ? v[p + st] : 0.0);
+    }
+  }
+  return I.lw * acc;
 }
 
 // The plant (Sec. 5.3): the true system x = (W, V) (device [sum 2 n_g], in
@@ -302,8 +327,6 @@ __global__ void __launch_bounds__(THREADS) k_wave_plant(WArgs A, const Layout* l
   double* W = smem;
   double* V = W + ng;
   double* F = V + ng;
-  Stencil<double> L{A.Lc + I.t_off * ELL, A.Ltc + I.t_off * ELL, A.Lv + I.t_off * ELL,
-                    A.Ltv + I.t_off * ELL, A.Ld + I.t_off};
   const int* act_of = A.act_of + I.t_off;
   for (int p = threadIdx.x; p < ng; p += THREADS) {
     W[p] = x[Ly.g_off + p];
@@ -318,7 +341,7 @@ __global__ void __launch_bounds__(THREADS) k_wave_plant(WArgs A, const Layout* l
     int cnt = 0;
     for (int p = threadIdx.x; p < ng; p += THREADS, ++cnt) {
       const double w = W[p];
-      const double g = (I.c * L.lap(W, p) - I.b * V[p] - I.kappa * w * w * w + F[p]) * ia;
+      const double g = (I.c * lap_at(I, W, p) - I.b * V[p] - I.kappa * w * w * w + F[p]) * ia;
       vn[cnt] = V[p] + tau * g;
     }
     __syncthreads();
@@ -347,19 +370,15 @@ struct nmpc_wave {
   long long n_a = 0, n_w = 0;  // sum n_u, sum n_g
   int ng_max = 0;
   WInst* inst_d = nullptr;
-  int *act_of = nullptr, *act_pt = nullptr, *Lc = nullptr, *Ltc = nullptr;
-  double *Lv = nullptr, *Ltv = nullptr, *Ld = nullptr;
-  float *Lvf = nullptr, *Ltvf = nullptr, *Ldf = nullptr;
+  int *act_of = nullptr, *act_pt = nullptr;
   double *wref = nullptr, *uref = nullptr;
-  size_t smem = 0;
 };
 
 namespace {
 
 void free_wave(nmpc_wave* h) {
   stage_drv::driver_free(h->drv);
-  void* ptrs[] = {h->inst_d, h->act_of, h->act_pt, h->Lc, h->Ltc, h->Lv, h->Ltv, h->Ld, h->Lvf,
-                  h->Ltvf, h->Ldf, h->wref, h->uref};
+  void* ptrs[] = {h->inst_d, h->act_of, h->act_pt, h->wref, h->uref};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -387,14 +406,6 @@ WArgs make_args(const nmpc_wave* h) {
   A.inst = h->inst_d;
   A.act_of = h->act_of;
   A.act_pt = h->act_pt;
-  A.Lc = h->Lc;
-  A.Lv = h->Lv;
-  A.Ltc = h->Ltc;
-  A.Ltv = h->Ltv;
-  A.Ld = h->Ld;
-  A.Lvf = h->Lvf;
-  A.Ltvf = h->Ltvf;
-  A.Ldf = h->Ldf;
   A.x0 = h->drv.x0;
   A.wref = h->wref;
   A.uref = h->uref;
@@ -404,19 +415,35 @@ WArgs make_args(const nmpc_wave* h) {
   return A;
 }
 
+// k_wave_dir for a group of stages.
+using DirKernel = void (*)(WArgs, stage_drv::Ctl, stage_drv::Iter, stage_drv::Range);
+template <typename T, int PPT>
+DirKernel dir_kernel_of(bool neu, bool d2) {
+  if (neu) return d2 ? wave_dev::k_wave_dir<T, PPT, true, true> : wave_dev::k_wave_dir<T, PPT, true, false>;
+  return d2 ? wave_dev::k_wave_dir<T, PPT, false, true> : wave_dev::k_wave_dir<T, PPT, false, false>;
+}
+DirKernel dir_kernel(bool mixed, const stage_drv::Group& g) {
+  if (mixed) return g.ppt == 1 ? dir_kernel_of<float, 1>(g.neu, g.d2) : dir_kernel_of<float, 2>(g.neu, g.d2);
+  return g.ppt == 1 ? dir_kernel_of<double, 1>(g.neu, g.d2) : dir_kernel_of<double, 2>(g.neu, g.d2);
+}
+size_t stage_smem(bool mixed, const stage_drv::Group& g) {
+  return mixed ? wave_dev::stage_bytes<float>(g.ng_max) : wave_dev::stage_bytes<double>(g.ng_max);
+}
+
 struct WaveDir {
   const nmpc_wave* h;
   cudaStream_t st;
   cudaError_t operator()(const stage_drv::Ctl& C, const stage_drv::Iter& S) const {
     WArgs A = make_args(h);
+    const bool mixed = h->opts.precision == NMPC_MIXED;
     for (int half = 0; half < (A.rb ? 2 : 1); ++half) {
       A.half = half;
-      if (h->opts.precision == NMPC_MIXED)
-        wave_dev::k_wave_dir<float><<<h->drv.n_work, wave_dev::THREADS, h->smem, st>>>(A, C, S);
-      else
-        wave_dev::k_wave_dir<double><<<h->drv.n_work, wave_dev::THREADS, h->smem, st>>>(A, C, S);
-      const cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
+      for (const stage_drv::Group& g : h->drv.groups) {
+        const cudaError_t e =
+            stage_drv::launch_stages(dir_kernel(mixed, g), stage_smem(mixed, g),
+                                     stage_drv::range_of(g, A.rb != 0, half), A, C, S, st);
+        if (e != cudaSuccess) return e;
+      }
     }
     return cudaSuccess;
   }
@@ -464,8 +491,8 @@ int nmpc_wave_setup(const nmpc_wave_desc* descs, int n, const nmpc_wave_opts* op
   nmpc_wave* h = new (std::nothrow) nmpc_wave();
   if (!h) return NMPC_ERR_CUDA;
   h->opts = o;
-  std::vector<int> act_of, act_pt, Lc, Ltc;
-  std::vector<double> Lv, Ltv, Ld;
+  std::vector<int> act_of, act_pt;
+  std::vector<stage_drv::GridKind> grid;
   long long n_pts = 0;
   for (int b = 0; b < n; ++b) {
     const nmpc_wave_desc& d = descs[b];
@@ -489,11 +516,13 @@ int nmpc_wave_setup(const nmpc_wave_desc* descs, int n, const nmpc_wave_opts* op
     I.r = d.r;
     I.qf = d.qf;
     I.gamma = d.gamma;
-    std::vector<int> ao(I.ng, -1);
-    for (int a = 0; a < d.n_u; ++a) ao[d.act_cell[a]] = a;
+    I.neu = d.bc == 0 ? 1 : 0;
+    I.lw = stage_drv::neighbour_weight(d.m, d.bc);
+    wave_dev::derive(I);
+    const std::vector<int> ao = stage_drv::actuator_map(d.dim, d.m, d.n_u, d.act_cell);
     act_of.insert(act_of.end(), ao.begin(), ao.end());
     for (int a = 0; a < d.n_u; ++a) act_pt.push_back(d.act_cell[a]);
-    stage_drv::append_ell(d.dim, d.m, d.bc == 0 ? 0 : 1, Lc, Lv, Ltc, Ltv, Ld);
+    grid.push_back(stage_drv::GridKind{d.dim, d.m, I.ng, d.bc == 0});
     stage_drv::Layout L{};
     L.N = I.N;
     L.nx = 2 * I.ng;
@@ -506,43 +535,22 @@ int nmpc_wave_setup(const nmpc_wave_desc* descs, int n, const nmpc_wave_opts* op
     h->ng_max = std::max(h->ng_max, I.ng);
     h->inst_h.push_back(I);
   }
-  const size_t tsz = o.precision == NMPC_MIXED ? sizeof(float) : sizeof(double);
-  h->smem = (size_t)h->ng_max * (wave_dev::F64_FIELDS * sizeof(double) + wave_dev::T_FIELDS * tsz);
-  cudaError_t e = stage_drv::driver_alloc(h->drv);
+  cudaError_t e = stage_drv::driver_alloc(h->drv, grid, false);
   auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   A(stage_drv::dalloc(&h->inst_d, n));
   A(stage_drv::dalloc(&h->act_of, act_of.size()));
   A(stage_drv::dalloc(&h->act_pt, act_pt.size()));
-  A(stage_drv::dalloc(&h->Lc, Lc.size()));
-  A(stage_drv::dalloc(&h->Ltc, Ltc.size()));
-  A(stage_drv::dalloc(&h->Lv, Lv.size()));
-  A(stage_drv::dalloc(&h->Ltv, Ltv.size()));
-  A(stage_drv::dalloc(&h->Ld, Ld.size()));
   A(stage_drv::dalloc(&h->wref, h->n_w));
   A(stage_drv::dalloc(&h->uref, h->n_a));
   A(stage_drv::upload(h->inst_d, h->inst_h));
   A(stage_drv::upload(h->act_of, act_of));
   A(stage_drv::upload(h->act_pt, act_pt));
-  A(stage_drv::upload(h->Lc, Lc));
-  A(stage_drv::upload(h->Ltc, Ltc));
-  A(stage_drv::upload(h->Lv, Lv));
-  A(stage_drv::upload(h->Ltv, Ltv));
-  A(stage_drv::upload(h->Ld, Ld));
-  {
-    const std::vector<float> Lvf(Lv.begin(), Lv.end()), Ltvf(Ltv.begin(), Ltv.end()),
-        Ldf(Ld.begin(), Ld.end());
-    A(stage_drv::dalloc(&h->Lvf, Lvf.size()));
-    A(stage_drv::dalloc(&h->Ltvf, Ltvf.size()));
-    A(stage_drv::dalloc(&h->Ldf, Ldf.size()));
-    A(stage_drv::upload(h->Lvf, Lvf));
-    A(stage_drv::upload(h->Ltvf, Ltvf));
-    A(stage_drv::upload(h->Ldf, Ldf));
-  }
-  if (h->smem > 48 * 1024) {
-    A(cudaFuncSetAttribute(wave_dev::k_wave_dir<double>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem));
-    A(cudaFuncSetAttribute(wave_dev::k_wave_dir<float>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem));
+  for (const stage_drv::Group& g : h->drv.groups) {
+    const bool mixed = o.precision == NMPC_MIXED;
+    const size_t bytes = stage_smem(mixed, g) * g.spc;
+    if (bytes > 48 * 1024)
+      A(cudaFuncSetAttribute(dir_kernel(mixed, g), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)bytes));
   }
   if (e != cudaSuccess) {
     fprintf(stderr, "nmpc_wave_setup: %s\n", cudaGetErrorString(e));
