@@ -164,6 +164,10 @@ typedef struct {
                       registers (8 per lane at most), every pass of the
                       iteration without a block barrier; full-field
                       u-iteration (u_local does not apply there).
+                      Where every instance is on this path, with the Jacobi
+                      upper layer and use_graph, a solve is one launch per
+                      size class: each instance's CTAs keep its iterates in
+                      shared memory to the end (same iterates).
                       0 = auto (every such instance), 1 = the same,
                       2 = never (cluster path)                              */
   int variant;      /* NMPC_VARIANT_JACOBI (default) or NMPC_VARIANT_REDBLACK:
@@ -379,7 +383,8 @@ int64_t nmpc_launch_count(const nmpc_handle* h);
    strip path's are in nmpc_strip_plan, the line path's in nmpc_line_plan),
    out[10] iteration steps launched
    (one per iteration, whichever kernels it takes; one per solve when
-   persistent) since setup.  Returns NMPC_ERR_BAD_ARG for a null handle or array. */
+   persistent or when a solve's 1D instances run as whole-instance launches)
+   since setup.  Returns NMPC_ERR_BAD_ARG for a null handle or array. */
 int nmpc_launch_plan(const nmpc_handle* h, int64_t* out);
 
 /* Strip path of the handle (opts.strips): out[0] strips per iteration (work

@@ -15,6 +15,7 @@
 
 #include "../../include/nmpc.h"
 #include "nmpc_kernels.cuh"
+#include "nmpc_line_inst.h"
 
 using nmpc_dev::InstDev;
 using nmpc_dev::IterArgs;
@@ -52,8 +53,8 @@ struct nmpc_handle {
   double* lb[3] = {nullptr, nullptr, nullptr};
   // control
   int* ictl = nullptr;  // iter_k, closed-loop step, n_active, running line items, grid barrier
-                        // and item counters [4..9], running count for the strip plan [10]
-                        // words [4], the persistent line launch's item counters [2]
+                        // and item counters [4..9], running count for the strip plan [10],
+                        // retry word of the whole-instance launches [11]
   unsigned long long* res_inf = nullptr;
   unsigned long long* res_err = nullptr;
   double* res_sq = nullptr;
@@ -123,6 +124,10 @@ struct nmpc_handle {
   int line_solve_grid = 0;       // its CTAs (all resident at once)
   int n_line_inst = 0;
   size_t line_smem = 0;
+  // whole-instance solves of the 1D instances (k_line_inst; empty: one launch
+  // per iteration)
+  std::vector<LineInstLaunch> line_inst;
+  int* line_inst_d = nullptr;  // the instances in launch order
   long long launches = 0;
   // per-kernel CUDA-event timing (nmpc_kernel_timing): event pairs around
   // launches that are not being captured, summed per kernel kind
@@ -185,7 +190,7 @@ void free_all(nmpc_handle* h) {
                   h->xb[0], h->xb[1], h->xb[2], h->ub[0], h->ub[1], h->ub[2],
                   h->lb[0], h->lb[1], h->lb[2], h->ictl, h->res_inf, h->res_err, h->res_sq,
                   h->res_first, h->status, h->iters, h->final_buf, h->fin_inf,
-                  h->fin_2, h->f64_count, h->full0, h->scratch, h->strips_d, h->tail_d, h->patches_d, h->lines_d, h->lines_act_d,
+                  h->fin_2, h->f64_count, h->full0, h->scratch, h->strips_d, h->tail_d, h->patches_d, h->lines_d, h->lines_act_d, h->line_inst_d,
                   h->v3_d};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -1028,6 +1033,7 @@ FinalArgs make_final(nmpc_handle* h, double* u_out) {
   F.res_sq = h->res_sq;
   F.tol = h->opts.tol;
   F.max_iter = h->opts.max_iter;
+  F.retry = h->ictl + 11;
   return F;
 }
 
@@ -1119,45 +1125,61 @@ int solve_core(nmpc_handle* h, int horizon, const double* weights, int init, dou
     }
   }
   const int chunk = std::max(1, h->opts.check_every);
-  bool loop_graph = false;
-  if (!done && h->opts.use_graph) {
-    // the whole loop on the device: one graph launch, no host polls
-    int rc = build_loop_graph(h, A, chunk);
-    if (rc != NMPC_OK) return rc;
-    CK(cudaGraphLaunch(h->loop_exec, st));
-    loop_graph = true;
-    done = true;
-  }
-  long long launched = 0;
-  while (!done && launched <= h->opts.max_iter) {
-    int rc = run_chunk(h, A, st, chunk);
-    if (rc != NMPC_OK) return rc;
-    launched += chunk;
-    CK(cudaMemcpyAsync(h->h_active, h->ictl + 2, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (*h->h_active == 0) break;
-  }
-  FinalArgs F = make_final(h, u_out);
-  nmpc_dev::k_finalize_status<<<(h->n_inst + 127) / 128, 128, 0, st>>>(F);
-  nmpc_dev::k_gather_final<<<per_instance_grid(h), 256, 0, st>>>(F);
-  h->launches += 2;
-  CK(cudaGetLastError());
-  h->has_state = true;
   const int n = h->n_inst;
-  CK(cudaMemcpyAsync(h->h_status, h->status, n * sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h->h_iters, h->iters, n * sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h->h_f64, h->f64_count, n * sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h->h_fin, h->fin_inf, n * sizeof(double), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h->h_fin + n, h->fin_2, n * sizeof(double), cudaMemcpyDeviceToHost, st));
-  if (loop_graph)
-    CK(cudaMemcpyAsync(h->h_active, h->ictl, 8 * sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (loop_graph) {
-    // launch accounting: the loop ran iter_k / chunk chunks
-    const long long runs = (h->h_active[0] + chunk - 1) / chunk;
-    h->launches += 1 + runs * (chunk_launches(h, chunk) + 1);  // + the condition kernels
-    h->iter_launches += runs * chunk;
+  bool by_instance = !done && !h->line_inst.empty();
+  for (;;) {
+    bool loop_graph = false;
+    if (by_instance) {
+      // every 1D instance solved to the end by its own CTAs
+      CK(line_inst_solve(h->line_inst, A, h->line_inst_d, h->ictl + 11, st));
+      h->launches += (long long)h->line_inst.size();
+      h->iter_launches++;
+      done = true;
+    }
+    if (!done && h->opts.use_graph) {
+      // the whole loop on the device: one graph launch, no host polls
+      int rc = build_loop_graph(h, A, chunk);
+      if (rc != NMPC_OK) return rc;
+      CK(cudaGraphLaunch(h->loop_exec, st));
+      loop_graph = true;
+      done = true;
+    }
+    long long launched = 0;
+    while (!done && launched <= h->opts.max_iter) {
+      int rc = run_chunk(h, A, st, chunk);
+      if (rc != NMPC_OK) return rc;
+      launched += chunk;
+      CK(cudaMemcpyAsync(h->h_active, h->ictl + 2, sizeof(int), cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      if (*h->h_active == 0) break;
+    }
+    FinalArgs F = make_final(h, u_out);
+    nmpc_dev::k_finalize_status<<<(h->n_inst + 127) / 128, 128, 0, st>>>(F);
+    nmpc_dev::k_gather_final<<<per_instance_grid(h), 256, 0, st>>>(F);
+    h->launches += 2;
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(h->h_status, h->status, n * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->h_iters, h->iters, n * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->h_f64, h->f64_count, n * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->h_fin, h->fin_inf, n * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h->h_fin + n, h->fin_2, n * sizeof(double), cudaMemcpyDeviceToHost, st));
+    if (loop_graph || by_instance)
+      CK(cudaMemcpyAsync(h->h_active, h->ictl, 12 * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (loop_graph) {
+      // launch accounting: the loop ran iter_k / chunk chunks
+      const long long runs = (h->h_active[0] + chunk - 1) / chunk;
+      h->launches += 1 + runs * (chunk_launches(h, chunk) + 1);  // + the condition kernels
+      h->iter_launches += runs * chunk;
+    }
+    if (!by_instance || h->h_active[11] == 0) break;
+    // an instance diverged on its split residual: iterate from S^0 (nothing
+    // of the state before the solve has been overwritten)
+    by_instance = done = false;
+    rc0 = start();
+    if (rc0 != NMPC_OK) return rc0;
   }
+  h->has_state = true;
   int rc = NMPC_OK;
   for (int b = 0; b < n; ++b) {
     if (stats) {
@@ -1587,6 +1609,18 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       cudaGetLastError();
     }
   }
+  // whole-instance solves where every stage of the handle is on the line path
+  // (Jacobi upper layer: the red-black order's norms need the neighbours that
+  // half 0 overwrites) and the solve loop is a graph otherwise (use_graph = 0
+  // asks for plain per-iteration launches)
+  std::vector<int> line_list;
+  if (h->n_line_inst == n_instances && o.variant == NMPC_VARIANT_JACOBI && o.use_graph &&
+      !h->line_persistent) {
+    std::vector<int> all(n_instances);
+    for (int b = 0; b < n_instances; ++b) all[b] = b;
+    h->line_inst = line_inst_plan(h->inst_h, all, std::max(1, h->num_sms), max_optin, &line_list);
+    if (h->line_inst.empty()) line_list.clear();
+  }
   if (h->n_strips > 0 && two) {
     h->strip2 = true;
     h->strip_x = tx;
@@ -1683,6 +1717,8 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   A(dev_alloc(&h->patches_d, h->n_patches));
   A(dev_alloc(&h->lines_d, h->n_lines));
   A(dev_alloc(&h->lines_act_d, h->n_lines));
+  A(dev_alloc(&h->line_inst_d, line_list.size()));
+  if (!h->line_inst.empty()) A(line_inst_configure(max_optin));
   A(dev_alloc(&h->v3_d, h->n_strips > 0 ? h->n_u : 0));
   A(dev_alloc(&h->act_d, act_all.size()));
   A(dev_alloc(&h->x0_d, h->n_g));
@@ -1711,7 +1747,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
     h->scratch_stride = (long long)((work_bytes + 255) & ~size_t(255));
     A(cudaMalloc((void**)&h->scratch, (size_t)h->scratch_stride * h->grid));
   }
-  A(cudaMallocHost((void**)&h->h_active, 8 * sizeof(int)));
+  A(cudaMallocHost((void**)&h->h_active, 12 * sizeof(int)));
   A(cudaMallocHost((void**)&h->h_status, n_instances * sizeof(int)));
   A(cudaMallocHost((void**)&h->h_iters, n_instances * sizeof(int)));
   A(cudaMallocHost((void**)&h->h_f64, n_instances * sizeof(int)));
@@ -1731,6 +1767,9 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
                    cudaMemcpyHostToDevice));
     if (!lines.empty())
       A(cudaMemcpy(h->lines_d, lines.data(), lines.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    if (!line_list.empty())
+      A(cudaMemcpy(h->line_inst_d, line_list.data(), line_list.size() * sizeof(int),
+                   cudaMemcpyHostToDevice));
     A(cudaMemcpy(h->act_d, act_all.data(), act_all.size() * sizeof(int), cudaMemcpyHostToDevice));
     A(cudaMemset(h->ictl, 0, 12 * sizeof(int)));
     A(cudaDeviceSynchronize());

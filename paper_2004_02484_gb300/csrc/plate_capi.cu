@@ -576,13 +576,6 @@ int nmpc_plate_setup(const nmpc_plate_desc* descs, int n, const nmpc_plate_opts*
   A(stage_drv::upload(h->inst_d, h->inst_h));
   A(stage_drv::upload(h->pt_state, pt_state));
   A(stage_drv::upload(h->act_pt, act_pt));
-  for (const stage_drv::Group& g : h->drv.groups) {
-    const bool mixed = o.precision == NMPC_MIXED;
-    const size_t bytes = stage_smem(mixed, g) * g.spc;
-    if (bytes > 48 * 1024)
-      A(cudaFuncSetAttribute(dir_kernel(mixed, g), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bytes));
-  }
   if (e != cudaSuccess) {
     fprintf(stderr, "nmpc_plate_setup: %s\n", cudaGetErrorString(e));
     free_plate(h);

@@ -545,13 +545,6 @@ int nmpc_wave_setup(const nmpc_wave_desc* descs, int n, const nmpc_wave_opts* op
   A(stage_drv::upload(h->inst_d, h->inst_h));
   A(stage_drv::upload(h->act_of, act_of));
   A(stage_drv::upload(h->act_pt, act_pt));
-  for (const stage_drv::Group& g : h->drv.groups) {
-    const bool mixed = o.precision == NMPC_MIXED;
-    const size_t bytes = stage_smem(mixed, g) * g.spc;
-    if (bytes > 48 * 1024)
-      A(cudaFuncSetAttribute(dir_kernel(mixed, g), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bytes));
-  }
   if (e != cudaSuccess) {
     fprintf(stderr, "nmpc_wave_setup: %s\n", cudaGetErrorString(e));
     free_wave(h);
