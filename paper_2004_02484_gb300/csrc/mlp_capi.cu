@@ -27,6 +27,24 @@ namespace {
     }                                                              \
   } while (0)
 
+// kernel<<<grid, block, smem, st>>>(args...) that may start while the kernel
+// before it on the stream ends (it waits for it; see pdl_wait).
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 int grid_for(long long n, int threads) {
   long long b = (n + threads - 1) / threads;
   return (int)std::min<long long>(std::max<long long>(b, 1), 4096);
@@ -108,8 +126,7 @@ cudaError_t gemm(const __nv_bfloat16* A, const __nv_bfloat16* B, const float* bi
                  cudaStream_t st, float* ws = nullptr, size_t ws_elems = 0) {
   mlp_dev::GemmArgs g{A, B, bias, C, Cb, M, N, K, lda, ldb, ldc, epi};
   if (M <= mlp_dev::GEMV_MAX_M) {
-    mlp_dev::k_gemv_bf16<<<(N + 7) / 8, 256, 0, st>>>(g);
-    return cudaGetLastError();
+    return launch_pdl(mlp_dev::k_gemv_bf16, dim3((N + 7) / 8), dim3(256), 0, st, g);
   }
   CUtensorMap ta, tb;
   if (g_gemm_path == 0 && tma_ok(A, lda, K) && tma_ok(B, ldb, K) && make_map(&ta, A, M, K, lda) &&
@@ -141,17 +158,17 @@ cudaError_t gemm(const __nv_bfloat16* A, const __nv_bfloat16* B, const float* bi
     mlp_dev::TcArgs t{M, N, K, kb_per, n_kb, bias, C, Cb, ldc, epi, vec_ok,
                       split > 1 ? ws : nullptr, tc_error_ptr()};
     dim3 grid(tiles_n, tiles_m, split);
-    mlp_dev::k_gemm_tc<<<grid, mlp_dev::TC_THREADS, mlp_dev::TC_SMEM, st>>>(ta, tb, t);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(mlp_dev::k_gemm_tc, grid, dim3(mlp_dev::TC_THREADS),
+                               mlp_dev::TC_SMEM, st, ta, tb, t);
     if (e != cudaSuccess || split == 1) return e;
-    const long long total = (long long)M * N;
-    const int blocks = (int)std::min<long long>((total + 255) / 256, 4096);
-    mlp_dev::k_splitk_epilogue<<<blocks, 256, 0, st>>>(ws, split, M, N, bias, epi, C, Cb, ldc);
-    return cudaGetLastError();
+    const int vec = (N % 4 == 0) ? 1 : 0;
+    const long long work = (long long)M * N / (vec ? 4 : 1);
+    const int blocks = (int)std::min<long long>((work + 255) / 256, 4096);
+    return launch_pdl(mlp_dev::k_splitk_epilogue, dim3(blocks), dim3(256), 0, st, ws, split, M, N,
+                      bias, epi, C, Cb, ldc, vec);
   }
   dim3 grid((N + mlp_dev::BN - 1) / mlp_dev::BN, (M + mlp_dev::BM - 1) / mlp_dev::BM);
-  mlp_dev::k_gemm_bf16<<<grid, mlp_dev::GEMM_THREADS, 0, st>>>(g);
-  return cudaGetLastError();
+  return launch_pdl(mlp_dev::k_gemm_bf16, grid, dim3(mlp_dev::GEMM_THREADS), 0, st, g);
 }
 
 // Launches gemm() issues for these operands (for launch accounting).
@@ -168,8 +185,7 @@ int gemm_launches(const void* A, const void* B, int M, int N, int K, int lda, in
 cudaError_t transpose(const __nv_bfloat16* in, __nv_bfloat16* out, int rows, int cols,
                       cudaStream_t st) {
   dim3 grid((cols + 31) / 32, (rows + 31) / 32);
-  mlp_dev::k_transpose_bf16<<<grid, dim3(32, 8), 0, st>>>(in, out, rows, cols);
-  return cudaGetLastError();
+  return launch_pdl(mlp_dev::k_transpose_bf16, grid, dim3(32, 8), 0, st, in, out, rows, cols);
 }
 
 }  // namespace
@@ -302,7 +318,7 @@ int nmpc_mlp_create(int n_layers, const int* widths, int max_batch, uint64_t see
     fal(&m->vW[l], nin * nout); fal(&m->b[l], nout); fal(&m->gb[l], nout);
     fal(&m->mb[l], nout); fal(&m->vb[l], nout);
     bal(&m->Wb[l], nin * nout); bal(&m->WTb[l], nin * nout);
-    fal(&m->z[l], (size_t)B * nout);
+    fal(&m->z[l], l < n_layers - 1 ? (size_t)B * nout : 0);  // the last layer's is y
     m->n_params += (long long)nin * nout + nout;
   }
   for (int l = 0; l <= n_layers; ++l) {
@@ -413,25 +429,18 @@ int nmpc_mlp_set_grads(nmpc_mlp* m, const float* host) {
 
 static int forward_impl(nmpc_mlp* m, const float* x, int B, float* y, cudaStream_t st) {
   const int n_in = m->w[0];
-  mlp_dev::k_cast_bf16<<<grid_for((long long)B * n_in, 256), 256, 0, st>>>(x, m->a[0],
-                                                                        (long long)B * n_in);
-  MCK(cudaGetLastError());
+  MCK(launch_pdl(mlp_dev::k_cast_bf16, dim3(grid_for((long long)B * n_in, 256)), dim3(256), 0, st, x,
+                 m->a[0], (long long)B * n_in));
   m->launches++;
   for (int l = 0; l < m->L; ++l) {
     const int nin = m->w[l], nout = m->w[l + 1];
     const bool last = (l == m->L - 1);
     // z = a W^T + b (fp32 kept for the backward pass) and, for a hidden
-    // layer, GELU(z) as bf16: both from one product
-    MCK(gemm(m->a[l], m->Wb[l], m->b[l], m->z[l], last ? nullptr : m->a[l + 1], B, nout, nin, nin,
-             nin, nout, last ? mlp_dev::EPI_NONE : mlp_dev::EPI_Z_GELU, st, m->ws, m->ws_elems));
+    // layer, GELU(z) as bf16: both from one product; the last layer's z is y
+    MCK(gemm(m->a[l], m->Wb[l], m->b[l], last ? y : m->z[l], last ? nullptr : m->a[l + 1], B, nout,
+             nin, nin, nin, nout, last ? mlp_dev::EPI_NONE : mlp_dev::EPI_Z_GELU, st, m->ws,
+             m->ws_elems));
     m->launches += gemm_launches(m->a[l], m->Wb[l], B, nout, nin, nin, nin, m->ws != nullptr);
-  }
-  const int nout = m->w[m->L];
-  if (y != m->z[m->L - 1]) {
-    const long long ny = (long long)B * nout;
-    mlp_dev::k_copy_f32<<<grid_for(ny, 256), 256, 0, st>>>(m->z[m->L - 1], y, ny);
-    MCK(cudaGetLastError());
-    m->launches++;
   }
   return NMPC_MLP_OK;
 }
@@ -450,14 +459,14 @@ int nmpc_mlp_backward(nmpc_mlp* m, const float* x, const float* target, int B, f
   const int nout_all = m->w[m->L];
   MCK(cudaMemsetAsync(m->loss, 0, sizeof(float), st));
   const long long ny = (long long)B * nout_all;
-  mlp_dev::k_mse<<<grid_for(ny, 256), 256, 0, st>>>(m->y, target, ny, m->dz, m->dz16, m->loss);
-  MCK(cudaGetLastError());
+  MCK(launch_pdl(mlp_dev::k_mse, dim3(std::min(grid_for(ny, 256), 8 * num_sms())), dim3(256), 0, st,
+                 m->y, target, ny, m->dz, m->dz16, m->loss));
   m->launches++;
   for (int l = m->L - 1; l >= 0; --l) {
     const int nin = m->w[l], nout = m->w[l + 1];
     // dz (fp32 in m->dz, bf16 in m->dz16) holds dL/dz_l, [B, nout]
-    mlp_dev::k_bias_grad<<<(nout + 127) / 128, 128, 0, st>>>(m->dz, m->gb[l], B, nout);
-    MCK(cudaGetLastError());
+    MCK(launch_pdl(mlp_dev::k_bias_grad, dim3((nout + mlp_dev::BG_COLS - 1) / mlp_dev::BG_COLS),
+                   dim3(mlp_dev::BG_COLS * mlp_dev::BG_ROWS), 0, st, m->dz, m->gb[l], B, nout));
     // gW[o, i] = sum_b dz[b, o] a_l[b, i]: A = dz^T [nout, B], B-operand = a_l^T [nin, B]
     MCK(transpose(m->dz16, m->dzT, B, nout, st));
     MCK(transpose(m->a[l], m->aT[l], B, nin, st));
@@ -469,9 +478,8 @@ int nmpc_mlp_backward(nmpc_mlp* m, const float* x, const float* target, int B, f
       MCK(gemm(m->dz16, m->WTb[l], nullptr, m->da, nullptr, B, nin, nout, nout, nout, nin,
                mlp_dev::EPI_NONE, st, m->ws, m->ws_elems));
       const long long n = (long long)B * nin;
-      mlp_dev::k_gelu_backward<<<grid_for(n, 256), 256, 0, st>>>(m->da, m->z[l - 1], m->dz,
-                                                                m->dz16, n);
-      MCK(cudaGetLastError());
+      MCK(launch_pdl(mlp_dev::k_gelu_backward, dim3(grid_for(n, 256)), dim3(256), 0, st, m->da,
+                     m->z[l - 1], m->dz, m->dz16, n));
       m->launches += 1 + gemm_launches(m->dz16, m->WTb[l], B, nin, nout, nout, nout,
                                        m->ws != nullptr);
     }

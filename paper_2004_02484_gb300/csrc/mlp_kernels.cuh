@@ -20,6 +20,14 @@
 
 namespace mlp_dev {
 
+// Kernels of the network's passes overlap their launch with the end of the
+// kernel before (programmatic dependent launch): the next launch may start,
+// then wait for the previous one's writes (no-ops for plain launches).  A
+// pass is a chain of ten to forty kernels of a few microseconds, about half
+// of which was the gap between them.
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 constexpr int BM = 128, BN = 128, BK = 32, PAD = 8, LDS = BK + PAD;  // bf16 elements
 constexpr int GEMM_THREADS = 256;
 enum { EPI_NONE = 0, EPI_GELU = 1, EPI_Z_GELU = 2 };
@@ -94,6 +102,8 @@ struct GemmArgs {
 };
 
 __global__ void __launch_bounds__(GEMM_THREADS) k_gemm_bf16(GemmArgs g) {
+  pdl_next();
+  pdl_wait();
   __shared__ __align__(16) __nv_bfloat16 sA[2][BM * LDS];
   __shared__ __align__(16) __nv_bfloat16 sB[2][BN * LDS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -191,6 +201,8 @@ __global__ void __launch_bounds__(GEMM_THREADS) k_gemm_bf16(GemmArgs g) {
 constexpr int GEMV_MAX_M = 8;
 
 __global__ void __launch_bounds__(256) k_gemv_bf16(GemmArgs g) {
+  pdl_next();
+  pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = blockIdx.x * 8 + warp;
   if (n >= g.N) return;
@@ -232,6 +244,8 @@ __global__ void __launch_bounds__(256) k_gemv_bf16(GemmArgs g) {
 
 // out[c, r] = in[r, c] (bf16), 32 x 32 tiles through shared memory
 __global__ void k_transpose_bf16(const __nv_bfloat16* in, __nv_bfloat16* out, int rows, int cols) {
+  pdl_next();
+  pdl_wait();
   __shared__ __nv_bfloat16 t[32][33];
   const int c = blockIdx.x * 32 + threadIdx.x;
   for (int dy = threadIdx.y; dy < 32; dy += blockDim.y) {
@@ -246,27 +260,25 @@ __global__ void k_transpose_bf16(const __nv_bfloat16* in, __nv_bfloat16* out, in
   }
 }
 
-// out = in (a kernel rather than a copy node, so that the forward pass can be
-// captured into any graph, conditional bodies included)
-__global__ void k_copy_f32(const float* in, float* out, long long n) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x)
-    out[e] = in[e];
-}
-
 __global__ void k_cast_bf16(const float* in, __nv_bfloat16* out, long long n) {
+  pdl_next();
+  pdl_wait();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x)
     out[e] = __float2bfloat16_rn(in[e]);
 }
 
 __global__ void k_cast_f64(const float* in, double* out, long long n) {
+  pdl_next();
+  pdl_wait();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x)
     out[e] = (double)in[e];
 }
 
 __global__ void k_cast_f64_f32(const double* in, float* out, long long n) {
+  pdl_next();
+  pdl_wait();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x)
     out[e] = (float)in[e];
@@ -276,6 +288,8 @@ __global__ void k_cast_f64_f32(const double* in, float* out, long long n) {
 // into float32 [n_img][(my/f) (mx/f)] (sums in float64).
 __global__ void k_pool_avg(const double* src, float* dst, int n_img, int mx, int my, int f,
                            long long dst_stride) {
+  pdl_next();
+  pdl_wait();
   const int ox = mx / f, oy = my / f;
   const long long n = (long long)n_img * ox * oy;
   const double inv = 1.0 / ((double)f * f);
@@ -292,9 +306,14 @@ __global__ void k_pool_avg(const double* src, float* dst, int n_img, int mx, int
   }
 }
 
-// loss = mean((y - t)^2) over B*N; dy = 2 (y - t) / (B*N) written as bf16 (and fp32)
-__global__ void k_mse(const float* y, const float* t, long long n, float* dy32,
-                      __nv_bfloat16* dy16, float* loss_acc) {
+// loss = mean((y - t)^2) over B*N; dy = 2 (y - t) / (B*N) written as bf16 (and
+// fp32).  One atomic add a block: a warp's each, on one address, took 52 us of
+// a 256 x 6800 batch.
+__global__ void __launch_bounds__(256) k_mse(const float* y, const float* t, long long n,
+                                             float* dy32, __nv_bfloat16* dy16, float* loss_acc) {
+  __shared__ float part[8];
+  pdl_next();
+  pdl_wait();
   float acc = 0.0f;
   const float scale = 2.0f / (float)n;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
@@ -306,12 +325,20 @@ __global__ void k_mse(const float* y, const float* t, long long n, float* dy32,
     dy16[e] = __float2bfloat16_rn(gval);
   }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss_acc, acc / (float)n);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.0f;
+    for (int w = 0; w < 8; ++w) s += part[w];
+    atomicAdd(loss_acc, s / (float)n);
+  }
 }
 
 // dz = da * GELU'(z) (hidden layers); written as bf16 for the next GEMMs and fp32
 __global__ void k_gelu_backward(const float* da, const float* z, float* dz32,
                                 __nv_bfloat16* dz16, long long n) {
+  pdl_next();
+  pdl_wait();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x) {
     const float v = da[e] * gelu_grad(z[e]);
@@ -320,13 +347,25 @@ __global__ void k_gelu_backward(const float* da, const float* z, float* dz32,
   }
 }
 
-// db[n] = sum_b dz[b, n]
-__global__ void k_bias_grad(const float* dz, float* db, int B, int N) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
+// db[n] = sum_b dz[b, n]: 32 columns a block, 32 rows at a time (one thread a
+// column walked the batch serially: 17 us for 256 rows, whatever the width).
+constexpr int BG_COLS = 32, BG_ROWS = 32;
+__global__ void __launch_bounds__(BG_COLS* BG_ROWS) k_bias_grad(const float* dz, float* db, int B,
+                                                                int N) {
+  __shared__ float part[BG_ROWS][BG_COLS + 1];
+  pdl_next();
+  pdl_wait();
+  const int c = threadIdx.x % BG_COLS, r = threadIdx.x / BG_COLS;
+  const int n = blockIdx.x * BG_COLS + c;
   float s = 0.0f;
-  for (int b = 0; b < B; ++b) s += dz[(long long)b * N + n];
-  db[n] = s;
+  if (n < N)
+    for (int b = r; b < B; b += BG_ROWS) s += dz[(long long)b * N + n];
+  part[r][c] = s;
+  __syncthreads();
+  if (r == 0 && n < N) {
+    for (int q = 1; q < BG_ROWS; ++q) s += part[q][c];
+    db[n] = s;
+  }
 }
 
 // Adam (Kingma & Ba 2015) on fp32 master weights, then the bf16 copy

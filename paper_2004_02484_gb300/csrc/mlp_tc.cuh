@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const int kb1 = min(g.n_kb, kb0 + g.kb_per_split);
   const int nk = max(0, kb1 - kb0);
 
+  pdl_next();
   if (threadIdx.x == 0) {
     s_fail = 0;
     s_issued = 0;
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tslot_ptr;
+  pdl_wait();  // the operands, and the outputs' readers, of earlier kernels
 
   if (warp == 0 && lane == 0) {
     // producer: wait for a free stage, then both tiles of the next K block
@@ -311,10 +313,34 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 }
 
 // Split-K: C = sum over the slices of the workspace (fixed order) + bias,
-// optional GELU; FP32 and/or BF16 outputs.
-__global__ void k_splitk_epilogue(const float* ws, int split, int M, int N, const float* bias,
-                                  int epi, float* C, __nv_bfloat16* Cb, int ldc) {
+// optional GELU; FP32 and/or BF16 outputs.  vec: four columns a thread (N a
+// multiple of 4), the slices' loads in flight together.
+__global__ void __launch_bounds__(256) k_splitk_epilogue(const float* ws, int split, int M, int N,
+                                                         const float* bias, int epi, float* C,
+                                                         __nv_bfloat16* Cb, int ldc, int vec) {
+  pdl_next();
+  pdl_wait();
   const long long total = (long long)M * N;
+  if (vec) {
+    for (long long i = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x); i < total;
+         i += 4 * (long long)gridDim.x * blockDim.x) {
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+      for (int s = 0; s < split; ++s) {
+        const float4 w = *reinterpret_cast<const float4*>(ws + (long long)s * total + i);
+        x.x += w.x;
+        x.y += w.y;
+        x.z += w.z;
+        x.w += w.w;
+      }
+      const int m = (int)(i / N), n = (int)(i - (long long)m * N);
+      epilogue_store(x.x, m, n, bias, epi, C, Cb, ldc);
+      epilogue_store(x.y, m, n + 1, bias, epi, C, Cb, ldc);
+      epilogue_store(x.z, m, n + 2, bias, epi, C, Cb, ldc);
+      epilogue_store(x.w, m, n + 3, bias, epi, C, Cb, ldc);
+    }
+    return;
+  }
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     float x = 0.0f;
