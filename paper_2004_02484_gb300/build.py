@@ -1,7 +1,7 @@
 """Build the sm_103a shared library ``_lib/libnmpc_gb300.so`` with nvcc.
 
-Five translation units (the solver's C ABI with its kernels, the
-whole-instance solves of 1D problems, the learned warm start's network, the pinned-actuator solver of the paper's plate and
+Six translation units (the solver's C ABI with its kernels, the whole-instance
+solves of 1D problems, the strips of batches of small 2D stages, the learned warm start's network, the pinned-actuator solver of the paper's plate and
 the second-order-in-time solver), compiled in parallel in-tree and linked
 into one library; the outputs are git-ignored.  ``build()`` rebuilds only when a
 source is newer than the library.
@@ -18,6 +18,7 @@ ROOT = os.path.dirname(HERE)
 LIB_DIR = os.path.join(HERE, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libnmpc_gb300.so")
 SOURCES = [os.path.join(HERE, "csrc", "nmpc_capi.cu"), os.path.join(HERE, "csrc", "nmpc_line_inst.cu"),
+           os.path.join(HERE, "csrc", "nmpc_strip_d64.cu"),
            os.path.join(HERE, "csrc", "mlp_capi.cu"),
            os.path.join(HERE, "csrc", "plate_capi.cu"), os.path.join(HERE, "csrc", "wave_capi.cu")]
 # every source and header the library is built from

@@ -16,6 +16,7 @@
 #include "../../include/nmpc.h"
 #include "nmpc_kernels.cuh"
 #include "nmpc_line_inst.h"
+#include "nmpc_strip_d64.h"
 
 using nmpc_dev::InstDev;
 using nmpc_dev::IterArgs;
@@ -106,6 +107,9 @@ struct nmpc_handle {
   int strip_x = 0, strip_y = 0, strip_threads = 0, strip_region = 0;
   int n_strip_inst = 0;
   bool strip2 = false;  // two grid columns per lane (k_strip2)
+  // a batch of stages that would also fit a cluster: the strips' split residual
+  // is the cluster path's (strip_d64), whole rows per warp (strip_fw)
+  bool strip_d64 = false, strip_fw = false;
   // the tail plan of k_strip2: strips of tail_y own rows for the launches
   // that run with at most tail_below instances still running
   int4* tail_d = nullptr;
@@ -236,7 +240,7 @@ IterArgs make_args(nmpc_handle* h) {
   // float32-truncated values: they move in steps of 2^-23 |x|, so its
   // iteration cannot settle far below ~1e-6; such handles switch to the
   // float64 residual by then at the latest
-  A.split_min = (h->n_strips > 0) ? std::max(h->opts.split_min, STRIP_SPLIT_FLOOR)
+  A.split_min = (h->n_strips > 0 && !h->strip_d64) ? std::max(h->opts.split_min, STRIP_SPLIT_FLOOR)
                                   : h->opts.split_min;
   A.max_iter = h->opts.max_iter;
   A.n_lo = h->opts.n_lo;
@@ -616,17 +620,19 @@ cudaError_t launch_patch(const nmpc_handle* h, const IterArgs& A, cudaStream_t s
   // which records the running-instance count for it
   if (h->n_tail > 0 && mode == nmpc_dev::MODE_SOLVE) count = std::max(count, 1);
   if (count == 0) return cudaSuccess;
+  const int per = h->strip_d64 ? PATCH_D64_ITEMS : PATCH_WARPS;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((count + PATCH_WARPS - 1) / PATCH_WARPS));
+  cfg.gridDim = dim3((unsigned)((count + per - 1) / per));
   cfg.blockDim = dim3(32 * PATCH_WARPS);
-  cfg.dynamicSmemBytes = h->patch_smem;
+  cfg.dynamicSmemBytes = h->strip_d64 ? 0 : h->patch_smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = (mode == nmpc_dev::MODE_SOLVE) ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, patch_kernel<T>(h->opts.n_lo), A, mode, j);
+  return cudaLaunchKernelEx(
+      &cfg, h->strip_d64 ? patch_d64_kernel(h->opts.n_lo) : patch_kernel<T>(h->opts.n_lo), A, mode, j);
 }
 
 template <typename T>
@@ -647,8 +653,10 @@ cudaError_t launch_strip(const nmpc_handle* h, const IterArgs& A, cudaStream_t s
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = (mode == nmpc_dev::MODE_SOLVE) ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, strip_kernel<T>(h->opts.n_lo, rb_half1(A, j), h->strip2), A,
-                            mode, j);
+  const TileKernel kern = h->strip_d64
+                              ? strip_d64_kernel(h->opts.n_lo, rb_half1(A, j), h->strip_fw)
+                              : strip_kernel<T>(h->opts.n_lo, rb_half1(A, j), h->strip2);
+  return cudaLaunchKernelEx(&cfg, kern, A, mode, j);
 }
 
 cudaError_t launch_line(const nmpc_handle* h, const IterArgs& A, cudaStream_t st, int mode, int j) {
@@ -1518,7 +1526,39 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       if ((I.mx & 1) || (I.s_off & 1) || (I.g_off & 1)) two = false;
     }
   }
-  const int tx = two ? 64 - 2 * nmpc_dev::strip2_pad(o.n_lo) : 32 - 2 * E;
+  // Batches of smaller stages (no instance needs strips by its size, no
+  // cluster shape asked for): strips as soon as a launch holds more stages
+  // than the device keeps clusters resident.  Up to there an iteration is one
+  // wave of clusters (64x64, N = 50: one instance 24.6 us, strips 30), above it
+  // the waves add up (two instances 46.5 against 31 us, 16: 265 against 67, 128:
+  // 2036 against 406; 32x32, N = 20: 8 instances 20.5 against 31, 16: 50 against
+  // 35; red-black 64x64: two instances 50 against 80, four 96 against 86).
+  bool d64 = false, fw = false;
+  if (my_max == 0 && o.strips == 0 && two && !o.cluster && !o.threads && !o.cells && !o.u_local &&
+      !o.persistent) {
+    fw = d64 = true;
+    int stages = 0;
+    for (const InstDev& I : h->inst_h) {
+      d64 = d64 && I.mx >= 24 && strip_eligible(I, act_all.data() + I.act_off, o) && !(I.mx & 1) &&
+            !(I.s_off & 1) && !(I.g_off & 1);
+      fw = fw && I.mx <= 64;
+      stages += h->rb ? (I.N + 1) / 2 : I.N;
+    }
+    if (d64) {
+      const LaunchPlan P0 = plan_launch(h->inst_h.data(), n_instances, stages, o, h->mixed,
+                                        std::max(1, h->num_sms), max_optin);
+      d64 = !P0.smem_mode ||
+            stages > clusters_resident(P0.csize, P0.threads, P0.cpt, P0.smem, h->mixed);
+    }
+    fw = fw && d64;
+    if (d64) {
+      std::fill(on_strips.begin(), on_strips.end(), 1);
+      for (const InstDev& I : h->inst_h) my_max = std::max(my_max, I.my);
+    }
+  }
+  h->strip_d64 = d64;
+  h->strip_fw = fw;
+  const int tx = two ? (fw ? 64 : 64 - 2 * nmpc_dev::strip2_pad(o.n_lo)) : 32 - 2 * E;
   if (my_max > 0) {
     long long whole = 0;  // strips with whole columns
     for (int b = 0; b < n_instances; ++b)
@@ -1528,6 +1568,24 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       }
     if (o.strip_rows) {
       ty = std::min(o.strip_rows, my_max);
+    } else if (d64) {
+      // a row step takes about 1.5 us whatever the number of resident warps
+      // (12 a SM), so a launch takes its waves times the rows of a strip's
+      // region and pipeline: the split of the columns with the fewest
+      const long long room = 4LL * STRIP2_MIN_BLOCKS * std::max(1, h->num_sms);
+      long long best = 0;
+      for (int segs = 1; segs == 1 || (my_max + segs - 1) / segs >= 8; ++segs) {
+        const int rows = (my_max + segs - 1) / segs;
+        long long warps = 0;
+        for (const InstDev& I : h->inst_h)
+          warps += (long long)(h->rb ? (I.N + 1) / 2 : I.N) * ((I.mx + tx - 1) / tx) *
+                   ((I.my + rows - 1) / rows);
+        const long long cost = ((warps + room - 1) / room) * (rows + 3 * E);
+        if (segs == 1 || cost < best) {
+          best = cost;
+          ty = rows;
+        }
+      }
     } else {
       const long long target = 4LL * std::max(1, h->num_sms) * 32;
       const long long segs = std::max(1LL, (target + whole - 1) / whole);
@@ -1639,6 +1697,17 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
     } else {
       h->n_tail_even = 0;
     }
+    if (d64)
+      for (int rbn = 0; rbn < 2; ++rbn) {
+        const cudaError_t e2 = cudaFuncSetAttribute(
+            strip_d64_kernel(o.n_lo, rbn != 0, fw), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            max_optin);
+        if (e2 != cudaSuccess) {
+          fprintf(stderr, "nmpc: kernel attribute: %s\n", cudaGetErrorString(e2));
+          delete h;
+          return NMPC_ERR_CUDA;
+        }
+      }
     h->strip_threads = 32 * nmpc_dev::STRIP2_WARPS;
     h->strip_region = 64 * (ty + 2 * E);
     constexpr int NF1 = nmpc_dev::strip_fields(true);
@@ -1821,8 +1890,16 @@ static int oneshot(nmpc_handle* h, const double* xi, const double* ui, const dou
   if (h->strip2) {
     // k_strip2 moves x, lambda as 16-byte column pairs
     auto misaligned = [](const void* p) { return ((uintptr_t)p & 15u) != 0; };
-    if (misaligned(xi) || misaligned(li) || misaligned(xo) || misaligned(lo))
-      return NMPC_ERR_BAD_ARG;
+    const bool in_off = misaligned(xi) || misaligned(li);
+    if (misaligned(xo) || misaligned(lo) || (in_off && !h->strip_d64)) return NMPC_ERR_BAD_ARG;
+    if (in_off) {
+      // stages that a cluster path would read at any alignment (the outputs
+      // are the handle's buffers 0 first, so 1 is free)
+      CK(cudaMemcpyAsync(h->xb[1], xi, h->n_s * sizeof(double), cudaMemcpyDeviceToDevice, st));
+      CK(cudaMemcpyAsync(h->lb[1], li, h->n_s * sizeof(double), cudaMemcpyDeviceToDevice, st));
+      xi = h->xb[1];
+      li = h->lb[1];
+    }
   }
   IterArgs A = make_args(h);
   A.xin[0] = xi;

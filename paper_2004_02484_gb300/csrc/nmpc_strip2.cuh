@@ -14,6 +14,15 @@
 // is entirely inside or outside the grid: even grid width, even region
 // origin) and the update stores column pairs.
 //
+// Two variants serve stages that would also fit a thread-block cluster, in
+// batches large enough to fill the GPU with strips:
+//   D64  the split residual in the cluster path's form (the O(1) differences
+//        in float64, Lap Phi(x) from Phi), so that a handle's convergence
+//        rule and rounding bound are those of its cluster path;
+//   FW   grids of at most 64 columns: a warp holds whole rows, no padding
+//        columns are recomputed and the outer lanes' missing neighbours are
+//        the Dirichlet zeros.
+//
 // Requirements checked by the host: float32 lower layer, n_lo <= 2, every
 // strip instance with an even grid width and even offsets of its state and
 // x0 / ref arrays (16-byte aligned pairs).
@@ -86,7 +95,7 @@ __device__ __forceinline__ D2 operator*(double s, D2 a) { return D2{s * a.x, s *
 
 // Three-row window of a column-pair field: w0 = row above, w1 = centre, w2 =
 // row below the consumer's row.
-template <typename V>
+template <typename V, bool FW = false>
 struct Win2 {
   V w0, w1, w2;
   __device__ __forceinline__ void push(V v) {
@@ -96,19 +105,33 @@ struct Win2 {
   }
   // the centre's left and right neighbours (one shuffle each: lane l - 1's
   // second column, lane l + 1's first column)
+  // (FW: zero beyond the region's ends)
   __device__ __forceinline__ V left() const {
-    return V{__shfl_up_sync(0xffffffffu, w1.y, 1), w1.x};
+    auto v = __shfl_up_sync(0xffffffffu, w1.y, 1);
+    if (FW && (threadIdx.x & 31) == 0) v = 0;
+    return V{v, w1.x};
   }
   __device__ __forceinline__ V right() const {
-    return V{w1.y, __shfl_down_sync(0xffffffffu, w1.x, 1)};
+    auto v = __shfl_down_sync(0xffffffffu, w1.x, 1);
+    if (FW && (threadIdx.x & 31) == 31) v = 0;
+    return V{w1.y, v};
   }
 };
-__device__ __forceinline__ F2 nsum2(const Win2<F2>& w, F2 cx, F2 cy) {
+template <bool FW>
+__device__ __forceinline__ F2 nsum2(const Win2<F2, FW>& w, F2 cx, F2 cy) {
   return fma2(cx, w.left() + w.right(), cy * (w.w0 + w.w2));
 }
-__device__ __forceinline__ D2 nsum2(const Win2<D2>& w, double cx, double cy) {
+template <bool FW>
+__device__ __forceinline__ D2 nsum2(const Win2<D2, FW>& w, double cx, double cy) {
   const D2 l = w.left(), r = w.right();
   return D2{cx * (l.x + r.x) + cy * (w.w0.x + w.w2.x), cx * (l.y + r.y) + cy * (w.w0.y + w.w2.y)};
+}
+
+// cx (left + right) + cy (above + below), rounded as on the cluster path
+template <bool FW>
+__device__ __forceinline__ F2 lap_nb(const Win2<F2, FW>& w, F2 cx, F2 cy) {
+  const F2 h = w.left() + w.right(), v = w.w0 + w.w2;
+  return fma2(cx, h, cy * v);
 }
 
 // Shared memory of one two-column strip warp: input rings of 64 doubles per
@@ -129,13 +152,13 @@ __device__ __forceinline__ void cp_async16_zfill(void* dst_smem, const void* src
                "r"(valid ? 16 : 0));
 }
 
-template <int n_lo, bool FULL, bool RBN, bool GSN = false>
+template <int n_lo, bool FULL, bool RBN, bool GSN = false, bool D64 = false, bool FW = false>
 __device__ __forceinline__ void strip2_body(const IterArgs& A,
                                             StripShared2<strip_ring_rows(n_lo), strip_fields(RBN)>& ws,
                                             int lane, int b, int s, int k, int rd, int x0, int y0,
                                             int strip_y, bool resid_only) {
   constexpr int E = 2 * n_lo - 1;
-  constexpr int P = strip2_pad(n_lo);
+  constexpr int P = FW ? 0 : strip2_pad(n_lo);
   constexpr int RING = strip_ring_rows(n_lo);
   constexpr int NF = strip_fields(RBN);
   constexpr bool full = FULL;
@@ -148,7 +171,7 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
   const int RH = own_rows + 2 * E;
   const int gx = x0 - P + 2 * lane;               // even; the pair is gx, gx + 1
   const bool gx_ok = gx >= 0 && gx < I.mx;        // both columns (even width)
-  const bool own_lane = lane >= n_lo && lane < 32 - n_lo && gx_ok;
+  const bool own_lane = (FW || (lane >= n_lo && lane < 32 - n_lo)) && gx_ok;
   const int gy0 = y0 - E;
 
   // actuators in reach, sorted by (row, region column, index)
@@ -246,18 +269,19 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
   const double cxd = I.cx, cyd = I.cy, dcd = I.dcoef, hd = I.h, k0d = I.k0, k1d = I.k1;
   const double qd = I.q, b0d = I.b0, hqfd = I.hqf;
   const F2 fcx = bc2(I.fcx), fcy = bc2(I.fcy), fdc = bc2(I.fdc), fh = bc2(I.fh);
-  const F2 fk0 = bc2(I.fk0), fk1 = bc2(I.fk1), fk1h = bc2(I.fk1h), fq = bc2(I.fq);
+  const F2 fk0 = bc2(I.fk0), fk1 = bc2(I.fk1), fk1h = bc2(I.fk1h), fq = bc2(I.fq), mdc = bc2(-I.fdc);
   const F2 fb0 = bc2(I.fb0), fk01 = bc2(I.fk01), one = bc2(1.0f);
   const F2 hqff = bc2(last ? I.fhqf : 0.0f);
   const double* uin_s = A.uin[rd] + I.u_off + (long long)s * nu;
   const double* v3_s = A.v3g + I.u_off + (long long)s * nu;
 
   Norms nm{0.0f, 0.0f, make_float4(0.f, 0.f, 0.f, 0.f), 0.0, 0.0, 0.0f};
-  Win2<D2> phd{}, lad{};
-  Win2<F2> laf{}, xvf{};
-  Win2<F2> pw[E > 1 ? E - 1 : 1];
+  Win2<D2, FW> phd{}, lad{};
+  Win2<F2, FW> laf{}, xvf{};  // D64: xvf holds Phi(x)
+  F2 xv0 = F2{0.f, 0.f}, xv1 = F2{0.f, 0.f};  // D64: x of the last two rows
+  Win2<F2, FW> pw[E > 1 ? E - 1 : 1];
 #pragma unroll
-  for (int m = 0; m < (E > 1 ? E - 1 : 1); ++m) pw[m] = Win2<F2>{};
+  for (int m = 0; m < (E > 1 ? E - 1 : 1); ++m) pw[m] = Win2<F2, FW>{};
   Shift<F2, E - 1> sdp, srg;
   Shift<F2, n_lo - 1> sk3, sax, sv1;
   Shift<F2, n_lo - 1> sv5, sw1;
@@ -275,7 +299,13 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
       } else {
         const F2 xv = d2f2(x), lf = d2f2(l);
         laf.push(lf);
-        xvf.push(xv);
+        if constexpr (D64) {
+          xv1 = xv0;
+          xv0 = xv;
+          xvf.push(fk0 * fma2(fk1h * xv, xv, xv));
+        } else {
+          xvf.push(xv);
+        }
         if (j < RH) {
           nm.mg.x = fmaxf(nm.mg.x, fmaxf(fabsf(xv.x), fabsf(xv.y)));
           nm.mg.y = fmaxf(nm.mg.y, fmaxf(fabsf(lf.x), fabsf(lf.y)));
@@ -351,6 +381,42 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
         dp = F2{d2f(dphx), d2f(dphy)};
         const double hq = last ? hqfd : 0.0;
         ax = F2{d2f(hd * (qd + k0d * k1d * mu.x) + hq), d2f(hd * (qd + k0d * k1d * mu.y) + hq)};
+      } else if constexpr (D64) {
+        // the cluster path's split form: the same terms, rounded alike
+        const F2 xv = xv1, rv = *reinterpret_cast<const F2*>(qs + RS_RF * 64);
+        const F2 lphi = fma2(mdc, xvf.w1, lap_nb(xvf, fcx, fcy));
+        const F2 mu = fma2(mdc, laf.w1, lap_nb(laf, fcx, fcy));
+        const F2 dphi = fk0 * fma2(fk1, xv, one);
+        const F2 s1 = fma2(fb0, srcf, lphi);
+        const F2 dr = xv - rv;
+        const F2 s3 = fma2(dphi, mu, fq * dr);
+        const double2 ln = last ? make_double2(0.0, 0.0) : ld2(qs + RS_LN * 64);
+        const F2 dx = F2{d2f(xp.x - x.x), d2f(xp.y - x.y)};
+        const F2 dl = F2{d2f(ln.x - lam.x), d2f(ln.y - lam.y)};
+        const F2 K1f = fma2(fh, s1, dx);
+        const F2 K3h = fma2(fh, s3, dl);
+        F2 K3f = K3h;
+        if (last)  // the product rounded on its own (packed operations would be contracted)
+          K3f = F2{__fadd_rn(K3h.x, __fmul_rn(hqff.x, dr.x)), __fadd_rn(K3h.y, __fmul_rn(hqff.y, dr.y))};
+        const float k1m = fmax_nan(fabsf(K1f.x), fabsf(K1f.y)), k3m = fmax_nan(fabsf(K3f.x), fabsf(K3f.y));
+        const F2 sq2 = fma2(K1f, K1f, K3f * K3f);
+        if (own) {
+          nm.mg.z = fmaxf(nm.mg.z, fmaxf(fmaxf(fabsf(dx.x), fabsf(dl.x)),
+                                         fmaxf(fabsf(dx.y), fabsf(dl.y))));
+          nm.mg.w = fmaxf(nm.mg.w, fmaxf(fabsf(rv.x), fabsf(rv.y)));
+          nm.fmax = fmax_nan(nm.fmax, fmax_nan(k1m, k3m));
+          nm.fsq += sq2.x + sq2.y;
+        }
+        if constexpr (RBN) {
+          const double2 xpn = ld2(qs + RS_XPN * 64), lnn = ld2(qs + RS_LNN * 64);
+          K1 = fma2(fh, s1, F2{d2f(xpn.x - x.x), d2f(xpn.y - x.y)});
+          K3 = last ? K3f : fma2(fh, s3, F2{d2f(lnn.x - lam.x), d2f(lnn.y - lam.y)});
+        } else {
+          K1 = K1f;
+          K3 = K3f;
+        }
+        dp = dphi;
+        ax = fma2(fh, fma2(fk01, mu, fq), hqff);
       } else {
         // Lap Phi(x) in difference form (see k_strip)
         const F2 xv = xvf.w1, rv = *reinterpret_cast<const F2*>(qs + RS_RF * 64);
@@ -521,7 +587,7 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
     if constexpr (!full) {
       float usum = 0.0f;
       for (int a = 0; a < nu; ++a) usum += fabsf(d2f(A.uin[rd][I.u_off + (long long)s * nu + a]));
-      e = split_bound(I, last, mags, usum, true, nm.gm);
+      e = D64 ? split_bound(I, last, mags, usum) : split_bound(I, last, mags, usum, true, nm.gm);
     }
     publish_residual(A, slot_k, b, k, rmax, rsq, e, full);
   }
@@ -530,7 +596,7 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
 // One upper-layer iteration over the strip work list with two columns per
 // lane (the strip list's x0 advance by 64 - 2 strip2_pad(n_lo)); control flow
 // as k_strip.
-template <int n_lo, bool RBN>
+template <int n_lo, bool RBN, bool D64 = false, bool FW = false>
 __global__ void __launch_bounds__(STRIP2_WARPS * 32, STRIP2_MIN_BLOCKS)
     k_strip2(IterArgs A, int MODE, int j_launch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -575,10 +641,10 @@ __global__ void __launch_bounds__(STRIP2_WARPS * 32, STRIP2_MIN_BLOCKS)
     resid_only = (k == A.max_iter);
   }
   if (full)
-    strip2_body<n_lo, true, RBN>(A, ws, lane, b, s, k, rd, x0, y0, sy, resid_only);
-  else if (RBN && MODE == MODE_SOLVE)
+    strip2_body<n_lo, true, RBN, false, D64, FW>(A, ws, lane, b, s, k, rd, x0, y0, sy, resid_only);
+  else if (RBN && !D64 && MODE == MODE_SOLVE)
     strip2_body<n_lo, false, false, true>(A, *reinterpret_cast<WS3*>(wbase), lane, b, s, k, rd,
                                           x0, y0, sy, resid_only);
   else
-    strip2_body<n_lo, false, RBN>(A, ws, lane, b, s, k, rd, x0, y0, sy, resid_only);
+    strip2_body<n_lo, false, RBN, false, D64, FW>(A, ws, lane, b, s, k, rd, x0, y0, sy, resid_only);
 }

@@ -1,0 +1,107 @@
+"""Batches of small 2D stages on the strip path (the cluster path's split
+residual, whole rows per warp up to 64 columns) against the same instances on
+the cluster path (strips=2).  Given an iterate, the residual's terms are
+rounded alike, so the norms of one iteration agree to the last bits; the lower
+layer differs by float32 rounding: each path's direction is within 8 units in
+the last place (2^-21 relative) of the exact one at its largest entry, so one
+iteration's changes agree to 2^-20 of the largest.  A solve contracts those
+differences with its iterates: the same count (one more or less where a norm
+lands on the tolerance) and, for equal counts, solutions within 1e-8."""
+import numpy as np
+import pytest
+
+from paper_2004_02484_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    from paper_2004_02484_gb300 import build as b
+    b.build()
+    import torch
+    torch.cuda.set_device(0)
+    from paper_2004_02484_gb300 import nmpc as G
+    return G
+
+
+# (mx, my, horizon, instances): the narrowest grid, 64 columns and the first
+# grids of two strips, heights off the strips' rows, enough stages for strips
+SIZES = [(24, 17, 7, 130), (62, 33, 20, 24), (64, 64, 50, 10), (66, 40, 30, 12), (112, 25, 20, 30),
+         (114, 31, 24, 20)]
+
+
+def _insts(mx, my, n, k, variant=0):
+    k *= 1 + variant  # a red-black launch holds half the stages
+    return [wl.heat2d(mx, my, n, 2, 2, seed=70 + b, ref_amp=0.6 + 0.01 * b) for b in range(k)]
+
+
+def _solver(G, insts, strips, **opts):
+    s = G.Solver(insts, precision=G.NMPC_MIXED, strips=strips, max_iter=4000, **opts)
+    assert G.nmpc_strip_plan(s.h)["instances"] == (len(insts) if strips == 0 else 0)
+    return s
+
+
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("variant,n_lo,n_u_it", [(0, 2, 2), (1, 2, 2), (0, 1, 1)])
+def test_one_iteration_equals_the_cluster_path(G, size, variant, n_lo, n_u_it):
+    import torch
+    insts = _insts(*size, variant)
+    gen = torch.Generator().manual_seed(3)
+    out = []
+    for strips in (0, 2):
+        s = _solver(G, insts, strips, variant=variant, n_lo=n_lo, n_u_it=n_u_it)
+        if not out:
+            x0 = torch.cat([torch.from_numpy(i.x0).repeat(i.horizon) for i in insts])
+            x = x0 + 0.01 * torch.randn(x0.shape, dtype=torch.float64, generator=gen)
+            lam = 1e-4 * torch.randn(x0.shape, dtype=torch.float64, generator=gen)
+            u = torch.randn(s.n_u, dtype=torch.float64, generator=gen)
+            x, lam, u = x.cuda(), lam.cuda(), u.cuda()
+        xo, lo, uo = torch.empty_like(x), torch.empty_like(lam), torch.empty_like(u)
+        r = G.nmpc_iterate(s.h, s.x0, s.ref, x, u, lam, xo, uo, lo, 1, s.n)
+        out.append((r, xo - x, uo - u, lo - lam))
+        s.close()
+    assert np.abs(out[0][0][:, 0] / out[1][0][:, 0] - 1).max() <= 1e-6
+    for a, b in zip(out[0][1:], out[1][1:]):
+        assert float((a - b).abs().max()) <= 2.0 ** -20 * float(b.abs().max())
+
+
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("variant", [0, 1])
+def test_solves_follow_the_cluster_path(G, size, variant):
+    insts = _insts(*size, variant)
+    got = []
+    for strips in (0, 2):
+        s = _solver(G, insts, strips, variant=variant, tol=1e-7)
+        rc, st = s.solve()
+        assert rc == G.NMPC_OK
+        got.append(([e.iters for e in st], [t.cpu().numpy() for t in s.state()]))
+        s.close()
+    it = np.array([g[0] for g in got])
+    assert np.abs(it[0] - it[1]).max() <= 1
+    if (it[0] == it[1]).all():
+        for a, b in zip(*(g[1] for g in got)):
+            assert np.abs(a - b).max() <= 1e-8 * np.abs(b).max()
+
+
+def test_unaligned_iterates_are_accepted(G):
+    """Stages that the cluster path would take at any alignment."""
+    import torch
+    insts = _insts(64, 64, 50, 3)
+    s = _solver(G, insts, 0)
+    n = s.n_s
+    buf = torch.zeros(2 * n + 4, dtype=torch.float64, device="cuda")
+    x, lam = buf[1:n + 1], buf[n + 2:2 * n + 2]
+    assert x.data_ptr() % 16 == 8 or lam.data_ptr() % 16 == 8
+    x.copy_(torch.cat([torch.from_numpy(i.x0).repeat(i.horizon) for i in insts]))
+    u = torch.zeros(s.n_u, dtype=torch.float64, device="cuda")
+    xa, la = x.clone(), lam.clone()
+    assert np.array_equal(G.nmpc_residual(s.h, s.x0, s.ref, x, u, lam, s.n)[:, 0],
+                          G.nmpc_residual(s.h, s.x0, s.ref, xa, u, la, s.n)[:, 0])
+    outs = []
+    for xi, li in ((x, lam), (xa, la)):
+        o = [torch.empty_like(t) for t in (xa, u, la)]
+        G.nmpc_iterate(s.h, s.x0, s.ref, xi, u, li, *o, 3, s.n)
+        outs.append(o)
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+    s.close()
