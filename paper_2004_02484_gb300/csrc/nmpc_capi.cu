@@ -620,19 +620,17 @@ cudaError_t launch_patch(const nmpc_handle* h, const IterArgs& A, cudaStream_t s
   // which records the running-instance count for it
   if (h->n_tail > 0 && mode == nmpc_dev::MODE_SOLVE) count = std::max(count, 1);
   if (count == 0) return cudaSuccess;
-  const int per = h->strip_d64 ? PATCH_D64_ITEMS : PATCH_WARPS;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((count + per - 1) / per));
+  cfg.gridDim = dim3((unsigned)((count + PATCH_WARPS - 1) / PATCH_WARPS));
   cfg.blockDim = dim3(32 * PATCH_WARPS);
-  cfg.dynamicSmemBytes = h->strip_d64 ? 0 : h->patch_smem;
+  cfg.dynamicSmemBytes = h->patch_smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = (mode == nmpc_dev::MODE_SOLVE) ? 1 : 0;
-  return cudaLaunchKernelEx(
-      &cfg, h->strip_d64 ? patch_d64_kernel(h->opts.n_lo) : patch_kernel<T>(h->opts.n_lo), A, mode, j);
+  return cudaLaunchKernelEx(&cfg, patch_kernel<T>(h->opts.n_lo), A, mode, j);
 }
 
 template <typename T>
@@ -747,7 +745,8 @@ cudaError_t launch_iterate(nmpc_handle* h, const IterArgs& A, cudaStream_t st, i
   }
   if (h->n_strips > 0) {
     // the actuators' v3 first (not needed by a residual-only pass)
-    if (!(MODE == nmpc_dev::MODE_ONESHOT && A.resid_only)) {
+    // (D64 strips compute the controls in reach themselves)
+    if (h->n_patches > 0 && !(MODE == nmpc_dev::MODE_ONESHOT && A.resid_only)) {
       h->launches++;
       e = timed(h, KT_PATCH, st, [&]() {
         return h->mixed ? launch_patch<float>(h, A, st, MODE, j)
@@ -920,7 +919,7 @@ int validate(const nmpc_desc* d) {
 // line-list compaction, every path's iteration kernels (twice per iteration
 // for red-black), the counter advance.
 long long chunk_launches(const nmpc_handle* h, int chunk) {
-  const long long per_iter = (h->n_work > 0 ? 1 : 0) + (h->n_strips > 0 ? 2 : 0) +
+  const long long per_iter = (h->n_work > 0 ? 1 : 0) + (h->n_strips > 0 ? 1 : 0) + (h->n_patches > 0 ? 1 : 0) +
                              (h->n_lines > 0 ? 1 : 0);
   return (h->n_lines > 0 ? 1 : 0) + (long long)chunk * per_iter * (h->rb ? 2 : 1) + 1;
 }
@@ -1526,13 +1525,15 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       if ((I.mx & 1) || (I.s_off & 1) || (I.g_off & 1)) two = false;
     }
   }
-  // Batches of smaller stages (no instance needs strips by its size, no
-  // cluster shape asked for): strips as soon as a launch holds more stages
-  // than the device keeps clusters resident.  Up to there an iteration is one
-  // wave of clusters (64x64, N = 50: one instance 24.6 us, strips 30), above it
-  // the waves add up (two instances 46.5 against 31 us, 16: 265 against 67, 128:
-  // 2036 against 406; 32x32, N = 20: 8 instances 20.5 against 31, 16: 50 against
-  // 35; red-black 64x64: two instances 50 against 80, four 96 against 86).
+  // Smaller stages (no instance needs strips by its size, no cluster shape
+  // asked for): strips where a launch holds more stages than the device keeps
+  // clusters resident, or the stages have more than 2048 cells.  Otherwise an
+  // iteration is one wave of clusters, which is as fast (32x32, N = 20, eight
+  // instances: 20.6 against 21.6 us, red-black 41.6 against 47.3).  Larger
+  // stages: 64x64, N = 50, one instance 24.8 against 20.9 us, red-black 50.6
+  // against 44.1; 96x80, N = 30: 24.0 against 18.7.  Beyond one wave the
+  // clusters' waves add up: 64x64 two instances 46.5 against 21.4 us, 16: 265
+  // against 56, 128: 2039 against 346; 32x32 16 instances 50 against 28.
   bool d64 = false, fw = false;
   if (my_max == 0 && o.strips == 0 && two && !o.cluster && !o.threads && !o.cells && !o.u_local &&
       !o.persistent) {
@@ -1544,7 +1545,9 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       fw = fw && I.mx <= 64;
       stages += h->rb ? (I.N + 1) / 2 : I.N;
     }
-    if (d64) {
+    int ng_max = 0;
+    for (const InstDev& I : h->inst_h) ng_max = std::max(ng_max, I.ng);
+    if (d64 && ng_max <= 2048) {
       const LaunchPlan P0 = plan_launch(h->inst_h.data(), n_instances, stages, o, h->mixed,
                                         std::max(1, h->num_sms), max_optin);
       d64 = !P0.smem_mode ||
@@ -1574,7 +1577,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       // region and pipeline: the split of the columns with the fewest
       const long long room = 4LL * STRIP2_MIN_BLOCKS * std::max(1, h->num_sms);
       long long best = 0;
-      for (int segs = 1; segs == 1 || (my_max + segs - 1) / segs >= 8; ++segs) {
+      for (int segs = 1; segs == 1 || (my_max + segs - 1) / segs >= 4; ++segs) {
         const int rows = (my_max + segs - 1) / segs;
         long long warps = 0;
         for (const InstDev& I : h->inst_h)
@@ -1595,7 +1598,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   // the tail plan (two columns per lane, solves): strips of ty_tail own rows
   // where the main plan's are at least four times taller
   int ty_tail = 0;
-  if (my_max > 0 && two && o.tail_rows >= 0) {
+  if (my_max > 0 && two && !d64 && o.tail_rows >= 0) {
     const int want = o.tail_rows > 0 ? o.tail_rows : 64;
     if (o.tail_rows > 0 ? want < ty : ty >= 4 * want) ty_tail = want;
   }
@@ -1616,7 +1619,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
         if (ty_tail > 0)
           for (int y0 = 0; y0 < I.my; y0 += ty_tail)
             for (int x0 = 0; x0 < I.mx; x0 += tx) tail.push_back(make_int4(b, s, x0, y0));
-        for (int a = 0; a < I.nu; ++a) patches.push_back(make_int4(b, s, a, 0));
+        for (int a = 0; a < I.nu && !d64; ++a) patches.push_back(make_int4(b, s, a, 0));
       }
     } else {
       cl_inst.push_back(I);

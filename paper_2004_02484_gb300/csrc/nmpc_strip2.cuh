@@ -142,6 +142,7 @@ struct StripShared2 {
   __align__(16) double ring[RING * 2 * 64];
   __align__(16) double sring[STRIP_SHORT * NF * 64];
   StripAct act[MAX_NU];
+  float v3[MAX_NU];  // D64: their controls' v3
   int n_act;
 };
 
@@ -150,6 +151,157 @@ __device__ __forceinline__ void cp_async16_zfill(void* dst_smem, const void* src
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src),
                "r"(valid ? 16 : 0));
+}
+
+// v3 of an actuator by half a warp (D64 strips): the u fixed-point iteration
+// of Sec. 5.2 (eqs. 22-24) in the full-field form's own order, on the cells
+// within 2 (n_lo - 1) grid steps of the actuator (13 for n_lo = 2), lane q of
+// the half holding cell q.  No other actuator's cell is among them (the host
+// checks), so v3 comes out as the cluster path's, operation by operation.
+// (k_patch, before strips of the other form, computes a square of 49 cells,
+// four of five of which its result does not depend on, and a second
+// right-hand side, in a launch of its own.)
+// Cell q of the diamond: itself, its four neighbours, the eight at two steps;
+// the neighbours (left, right, above, below) of cells 0 .. 4.
+static __constant__ signed char diamond_x[13] = {0, -1, 1, 0, 0, -2, 2, 0, 0, -1, 1, -1, 1};
+static __constant__ signed char diamond_y[13] = {0, 0, 0, -1, 1, 0, 0, -2, 2, -1, -1, 1, 1};
+static __constant__ signed char diamond_n[5][4] = {
+    {1, 2, 3, 4}, {5, 0, 9, 11}, {0, 6, 10, 12}, {9, 10, 7, 0}, {11, 12, 0, 8}};
+
+template <int n_lo, bool FULL>
+__device__ __forceinline__ float half_warp_v3(const IterArgs& A, const InstDev& I, int s, int a,
+                                              int rd, bool rbn, int lane) {
+  const int q = lane & 15, base = lane & 16;
+  const int mx = I.mx, my = I.my;
+  const bool last = (s == I.N - 1);
+  const int ca = A.act[I.act_off + a], ay = ca / mx, ax = ca - ay * mx;
+  const int qc = q < 13 ? q : 0;
+  const int gx = ax + diamond_x[qc], gy = ay + diamond_y[qc];
+  const bool in = gx >= 0 && gx < mx && gy >= 0 && gy < my;
+  const long long so = I.s_off + (long long)s * I.ng;
+  const double* Xg = A.xin[rd] + so;
+  const double* Lg = A.lin[rd] + so;
+  // red-black half 1: x_{i-1}, lambda_{i+1} as updated by half 0
+  const double* XPg = (s == 0) ? A.x0 + I.g_off : (rbn ? A.xout[rd ^ 1] : A.xin[rd]) + so - I.ng;
+  const double* LNg = (rbn ? A.lout[rd ^ 1] : A.lin[rd]) + so + I.ng;
+  const int c = in ? gy * mx + gx : 0;
+  // a field at the cell and its four neighbours (zero outside the grid)
+  struct Star {
+    double m, l, r, u, d;
+  };
+  auto star = [&](const double* f) {
+    Star v;
+    v.m = in ? f[c] : 0.0;
+    v.l = in && gx > 0 ? f[c - 1] : 0.0;
+    v.r = in && gx < mx - 1 ? f[c + 1] : 0.0;
+    v.u = in && gy > 0 ? f[c - mx] : 0.0;
+    v.d = in && gy < my - 1 ? f[c + mx] : 0.0;
+    return v;
+  };
+  const Star x = star(Xg), lm = star(Lg);
+  const double xp = in ? XPg[c] : 0.0, ln = in && !last ? LNg[c] : 0.0;
+  const double rc = in ? A.ref[I.g_off + c] : 0.0;
+  const double ua = A.uin[rd][I.u_off + (long long)s * I.nu + a];
+  const bool centre = q == 0;
+  float K1, K3, dp, axx;
+  if constexpr (FULL) {
+    const double k0 = I.k0, k1 = I.k1, h = I.h;
+    auto phi = [&](double w) { return k0 * (w + 0.5 * k1 * w * w); };
+    const double lphi = I.cx * (phi(x.l) + phi(x.r)) + I.cy * (phi(x.u) + phi(x.d)) - I.dcoef * phi(x.m);
+    const double mu = I.cx * (lm.l + lm.r) + I.cy * (lm.u + lm.d) - I.dcoef * lm.m;
+    const double dphi = k0 * (1.0 + k1 * x.m);
+    const double s1 = lphi + (centre ? I.b0 * ua : 0.0);
+    const double s3 = I.q * (x.m - rc) + dphi * mu;
+    const double lnx = last ? I.hqf * (x.m - rc) : ln;
+    K1 = d2f(__fma_rn(h, s1, xp - x.m));
+    K3 = d2f(__fma_rn(h, s3, lnx - lm.m));
+    dp = d2f(dphi);
+    axx = d2f(h * (I.q + k0 * k1 * mu) + (last ? I.hqf : 0.0));
+  } else {
+    const float fk0 = I.fk0, fk1h = I.fk1h, fcx = I.fcx, fcy = I.fcy, fdc = I.fdc;
+    auto phi = [&](double w) {
+      const float v = d2f(w);
+      return __fmul_rn(fk0, __fmaf_rn(__fmul_rn(fk1h, v), v, v));
+    };
+    auto lap = [&](float m, float l, float r, float u, float d) {
+      return __fmaf_rn(-fdc, m,
+                       __fmaf_rn(fcx, __fadd_rn(l, r), __fmul_rn(fcy, __fadd_rn(u, d))));
+    };
+    const float xv = d2f(x.m), rv = d2f(rc);
+    const float lphi = lap(phi(x.m), phi(x.l), phi(x.r), phi(x.u), phi(x.d));
+    const float mu = lap(d2f(lm.m), d2f(lm.l), d2f(lm.r), d2f(lm.u), d2f(lm.d));
+    dp = __fmul_rn(fk0, __fmaf_rn(I.fk1, xv, 1.0f));
+    const float s1 = __fmaf_rn(I.fb0, centre ? d2f(ua) : 0.0f, lphi);
+    const float dr = __fsub_rn(xv, rv);
+    const float s3 = __fmaf_rn(dp, mu, __fmul_rn(I.fq, dr));
+    const float hqff = last ? I.fhqf : 0.0f;
+    K1 = __fmaf_rn(I.fh, s1, d2f(xp - x.m));
+    K3 = __fmaf_rn(I.fh, s3, d2f(ln - lm.m));
+    if (last) K3 = __fadd_rn(K3, __fmul_rn(hqff, dr));
+    axx = __fmaf_rn(I.fh, __fmaf_rn(I.fk01, mu, I.fq), hqff);
+  }
+  const float th = I.fh, tb0 = I.fb0, tcx = I.fcx, tcy = I.fcy, auu = I.fauu;
+  auto sub_prod = [](float v, float r, float off) { return __fmaf_rn(-r, off, v); };
+  const float rg = in && q < 13 ? __frcp_rn(sub_prod(-1.0f, __fmul_rn(th, I.fdc), dp)) : 0.0f;
+  const float b3 = (float)(I.h * (I.r * ua + I.b0 * lm.m));
+  auto nsum = [&](float v) {  // over the neighbours, at the cells 0 .. 4
+    const int qq = q < 5 ? q : 0;
+    const float l = __shfl_sync(0xffffffffu, v, base + diamond_n[qq][0]);
+    const float r = __shfl_sync(0xffffffffu, v, base + diamond_n[qq][1]);
+    const float u = __shfl_sync(0xffffffffu, v, base + diamond_n[qq][2]);
+    const float d = __shfl_sync(0xffffffffu, v, base + diamond_n[qq][3]);
+    return __fmaf_rn(tcx, __fadd_rn(l, r), __fmul_rn(tcy, __fadd_rn(u, d)));
+  };
+  float v1 = __fmul_rn(-K1, rg), v3 = 0.0f;
+  for (int n = 0; n < A.n_u_it; ++n) {
+    if (n > 0 && centre) v1 = __fmul_rn(__fmaf_rn(__fmul_rn(th, tb0), v3, -K1), rg);
+    float v5 = v1;
+    if constexpr (n_lo > 1) v5 = sub_prod(v1, rg, __fmul_rn(th, nsum(__fmul_rn(dp, v1))));
+    const float w1 = __fmul_rn(sub_prod(-K3, axx, v5), rg);
+    float v4 = w1;
+    if constexpr (n_lo > 1) v4 = sub_prod(w1, rg, __fmul_rn(__fmul_rn(th, dp), nsum(w1)));
+    v3 = __fdiv_rn(__fmaf_rn(__fmul_rn(th, tb0), v4, b3), auu);
+  }
+  return v3;  // the centre's lane (q = 0)
+}
+
+// The actuators within reach of the region at column x0 - P, row gy0 (RH rows),
+// sorted by (row, region column, index), into the warp's list.
+template <int P, typename WS>
+__device__ __forceinline__ void strip2_actuators(const IterArgs& A, const InstDev& I, WS& ws,
+                                             int lane, int x0, int gy0, int RH) {
+  const int nu = I.nu;
+  const float inv_mx = 1.0f / (float)I.mx;
+  long long key[2];
+  int rr[2], rl[2];
+#pragma unroll
+  for (int h2 = 0; h2 < 2; ++h2) {
+    const int a = lane + 32 * h2;
+    key[h2] = 0x7fffffffffffffffLL;
+    rr[h2] = rl[h2] = 0;
+    if (a < nu) {
+      const int c = A.act[I.act_off + a];
+      const int cy = fdiv(c, I.mx, inv_mx), cx = c - cy * I.mx;
+      rl[h2] = cx - (x0 - P);
+      rr[h2] = cy - gy0;
+      if (rl[h2] >= 0 && rl[h2] < 64 && rr[h2] >= 0 && rr[h2] < RH)
+        key[h2] = ((long long)rr[h2] * 64 + rl[h2]) * MAX_NU + a;
+    }
+  }
+  int rank[2] = {0, 0};
+  for (int l = 0; l < 32; ++l) {
+    const long long k0 = __shfl_sync(0xffffffffu, key[0], l);
+    const long long k1 = __shfl_sync(0xffffffffu, key[1], l);
+#pragma unroll
+    for (int h2 = 0; h2 < 2; ++h2) rank[h2] += (k0 < key[h2]) + (k1 < key[h2]);
+  }
+#pragma unroll
+  for (int h2 = 0; h2 < 2; ++h2)
+    if (key[h2] != 0x7fffffffffffffffLL)
+      ws.act[rank[h2]] = StripAct{rr[h2], rl[h2], lane + 32 * h2, 0};
+  const int n = __popc(__ballot_sync(0xffffffffu, key[0] != 0x7fffffffffffffffLL)) +
+                __popc(__ballot_sync(0xffffffffu, key[1] != 0x7fffffffffffffffLL));
+  if (lane == 0) ws.n_act = n;
 }
 
 template <int n_lo, bool FULL, bool RBN, bool GSN = false, bool D64 = false, bool FW = false>
@@ -174,42 +326,20 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
   const bool own_lane = (FW || (lane >= n_lo && lane < 32 - n_lo)) && gx_ok;
   const int gy0 = y0 - E;
 
-  // actuators in reach, sorted by (row, region column, index)
-  {
-    const float inv_mx = 1.0f / (float)I.mx;
-    long long key[2];
-    int rr[2], rl[2];
-#pragma unroll
-    for (int h2 = 0; h2 < 2; ++h2) {
-      const int a = lane + 32 * h2;
-      key[h2] = 0x7fffffffffffffffLL;
-      rr[h2] = rl[h2] = 0;
-      if (a < nu) {
-        const int c = A.act[I.act_off + a];
-        const int cy = fdiv(c, I.mx, inv_mx), cx = c - cy * I.mx;
-        rl[h2] = cx - (x0 - P);
-        rr[h2] = cy - gy0;
-        if (rl[h2] >= 0 && rl[h2] < 64 && rr[h2] >= 0 && rr[h2] < RH)
-          key[h2] = ((long long)rr[h2] * 64 + rl[h2]) * MAX_NU + a;
-      }
-    }
-    int rank[2] = {0, 0};
-    for (int l = 0; l < 32; ++l) {
-      const long long k0 = __shfl_sync(0xffffffffu, key[0], l);
-      const long long k1 = __shfl_sync(0xffffffffu, key[1], l);
-#pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2) rank[h2] += (k0 < key[h2]) + (k1 < key[h2]);
-    }
-#pragma unroll
-    for (int h2 = 0; h2 < 2; ++h2)
-      if (key[h2] != 0x7fffffffffffffffLL)
-        ws.act[rank[h2]] = StripAct{rr[h2], rl[h2], lane + 32 * h2, 0};
-    const int n = __popc(__ballot_sync(0xffffffffu, key[0] != 0x7fffffffffffffffLL)) +
-                  __popc(__ballot_sync(0xffffffffu, key[1] != 0x7fffffffffffffffLL));
-    if (lane == 0) ws.n_act = n;
-  }
+  // (D64: the kernel has sorted them before it waited for the launch before)
+  if constexpr (!D64) strip2_actuators<P>(A, I, ws, lane, x0, gy0, RH);
   __syncwarp();
   const int n_act = ws.n_act;
+  if constexpr (D64) {
+    // the controls in reach, two at a time (another strip whose region holds
+    // the same actuator computes the same value)
+    for (int e0 = 0; e0 < n_act && !resid_only; e0 += 2) {
+      const int e = e0 + (lane >> 4);
+      const float v = half_warp_v3<n_lo, FULL>(A, I, s, ws.act[min(e, n_act - 1)].a, rd, RBN, lane);
+      if ((lane & 15) == 0 && e < n_act) ws.v3[e] = v;
+    }
+    __syncwarp();
+  }
   int na = 0;
   int next_row = n_act > 0 ? ws.act[0].row : 0x7fffffff;
 
@@ -328,7 +458,7 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
           const StripAct e = ws.act[na];
           if ((e.lane >> 1) == lane) {
             const double ua = uin_s[e.a];
-            const float v3a = (float)v3_s[e.a];
+            const float v3a = D64 ? ws.v3[na] : (float)v3_s[e.a];
             if (e.lane & 1) {
               srcd.y += ua;
               srcf.y += d2f(ua);
@@ -549,7 +679,8 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
     }
     if (!resid_only)
       A.uout[rd ^ 1][I.u_off + (long long)s * nu + a.a] =
-          ua - alpha * (double)(float)A.v3g[I.u_off + (long long)s * nu + a.a];
+          ua - alpha * (double)(D64 ? ws.v3[e]
+                                    : (float)A.v3g[I.u_off + (long long)s * nu + a.a]);
   }
   double rmax, rsq;
   float mags[4];
@@ -609,10 +740,22 @@ __global__ void __launch_bounds__(STRIP2_WARPS * 32, STRIP2_MIN_BLOCKS)
   const int k = (MODE == MODE_SOLVE) ? *(volatile int*)A.iter_k + launch_iter(A, j_launch) : 0;
   const int half = launch_half(A, j_launch);
   const int rd = (MODE == MODE_SOLVE) ? (k & 1) : 0;
+  if constexpr (D64) {
+    // what no launch changes (the item, its instance, the actuators in reach)
+    // before the wait: a chain of dependent loads that a short strip, a few
+    // rows of a single instance, would wait for in every iteration
+    const int e = ((A.rb && half) ? A.n_strips_even : 0) + blockIdx.x * STRIP2_WARPS + warp;
+    if (e < (A.rb && !half ? A.n_strips_even : A.n_strips)) {
+      const int4 it = A.strips[e];
+      const InstDev& I = A.inst[it.x];
+      constexpr int E = 2 * n_lo - 1, P = FW ? 0 : strip2_pad(n_lo);
+      strip2_actuators<P>(A, I, ws, lane, it.z, it.w - E, min(A.strip_y, I.my - it.w) + 2 * E);
+    }
+  }
   pdl_wait();
   // the tail plan once few instances run (the count k_patch recorded before
   // this launch: the same value for every warp)
-  const bool tail = MODE == MODE_SOLVE && A.n_tail > 0 && *A.strip_run <= A.tail_below;
+  const bool tail = !D64 && MODE == MODE_SOLVE && A.n_tail > 0 && *A.strip_run <= A.tail_below;
   const int n_all = tail ? A.n_tail : A.n_strips, n_even = tail ? A.n_tail_even : A.n_strips_even;
   const int item = ((A.rb && half) ? n_even : 0) + blockIdx.x * STRIP2_WARPS + warp;
   const int item_end = A.rb ? (half ? n_all : n_even) : n_all;
