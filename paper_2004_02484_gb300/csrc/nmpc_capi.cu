@@ -109,7 +109,8 @@ struct nmpc_handle {
   bool strip2 = false;  // two grid columns per lane (k_strip2)
   // a batch of stages that would also fit a cluster: the strips' split residual
   // is the cluster path's (strip_d64), whole rows per warp (strip_fw)
-  bool strip_d64 = false, strip_fw = false;
+  // (strip_al: 16-byte aligned column pairs)
+  bool strip_d64 = false, strip_fw = false, strip_al = true;
   // the tail plan of k_strip2: strips of tail_y own rows for the launches
   // that run with at most tail_below instances still running
   int4* tail_d = nullptr;
@@ -652,7 +653,7 @@ cudaError_t launch_strip(const nmpc_handle* h, const IterArgs& A, cudaStream_t s
   cfg.attrs = attr;
   cfg.numAttrs = (mode == nmpc_dev::MODE_SOLVE) ? 1 : 0;
   const TileKernel kern = h->strip_d64
-                              ? strip_d64_kernel(h->opts.n_lo, rb_half1(A, j), h->strip_fw)
+                              ? strip_d64_kernel(h->opts.n_lo, rb_half1(A, j), h->strip_fw, h->strip_al)
                               : strip_kernel<T>(h->opts.n_lo, rb_half1(A, j), h->strip2);
   return cudaLaunchKernelEx(&cfg, kern, A, mode, j);
 }
@@ -1540,8 +1541,8 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
     fw = d64 = true;
     int stages = 0;
     for (const InstDev& I : h->inst_h) {
-      d64 = d64 && I.mx >= 24 && strip_eligible(I, act_all.data() + I.act_off, o) && !(I.mx & 1) &&
-            !(I.s_off & 1) && !(I.g_off & 1);
+      d64 = d64 && I.mx >= 24 && strip_eligible(I, act_all.data() + I.act_off, o);
+      if ((I.mx & 1) || (I.s_off & 1) || (I.g_off & 1)) h->strip_al = false;
       fw = fw && I.mx <= 64;
       stages += h->rb ? (I.N + 1) / 2 : I.N;
     }
@@ -1703,7 +1704,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
     if (d64)
       for (int rbn = 0; rbn < 2; ++rbn) {
         const cudaError_t e2 = cudaFuncSetAttribute(
-            strip_d64_kernel(o.n_lo, rbn != 0, fw), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            strip_d64_kernel(o.n_lo, rbn != 0, fw, h->strip_al), cudaFuncAttributeMaxDynamicSharedMemorySize,
             max_optin);
         if (e2 != cudaSuccess) {
           fprintf(stderr, "nmpc: kernel attribute: %s\n", cudaGetErrorString(e2));
@@ -1890,7 +1891,7 @@ int nmpc_solve_host(nmpc_handle* h, const double* x0, const double* ref, int hor
 static int oneshot(nmpc_handle* h, const double* xi, const double* ui, const double* li,
                    double* xo, double* uo, double* lo, int resid_only, double* out_res,
                    cudaStream_t st) {
-  if (h->strip2) {
+  if (h->strip2 && h->strip_al) {
     // k_strip2 moves x, lambda as 16-byte column pairs
     auto misaligned = [](const void* p) { return ((uintptr_t)p & 15u) != 0; };
     const bool in_off = misaligned(xi) || misaligned(li);

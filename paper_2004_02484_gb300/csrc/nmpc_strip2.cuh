@@ -21,7 +21,9 @@
 //        rule and rounding bound are those of its cluster path;
 //   FW   grids of at most 64 columns: a warp holds whole rows, no padding
 //        columns are recomputed and the outer lanes' missing neighbours are
-//        the Dirichlet zeros.
+//        the Dirichlet zeros;
+//   AL = false (with D64)  odd grid widths or offsets: columns are copied and
+//        stored one by one, and a pair's second column may lie outside.
 //
 // Requirements checked by the host: float32 lower layer, n_lo <= 2, every
 // strip instance with an even grid width and even offsets of its state and
@@ -145,6 +147,13 @@ struct StripShared2 {
   float v3[MAX_NU];  // D64: their controls' v3
   int n_act;
 };
+
+// 4-byte asynchronous copy (zeros when !valid; src must still be a valid address)
+__device__ __forceinline__ void cp_async4_zfill(void* dst_smem, const void* src, bool valid) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src),
+               "r"(valid ? 4 : 0));
+}
 
 // 16-byte asynchronous copy (zeros when !valid; src must still be a valid address)
 __device__ __forceinline__ void cp_async16_zfill(void* dst_smem, const void* src, bool valid) {
@@ -304,7 +313,8 @@ __device__ __forceinline__ void strip2_actuators(const IterArgs& A, const InstDe
   if (lane == 0) ws.n_act = n;
 }
 
-template <int n_lo, bool FULL, bool RBN, bool GSN = false, bool D64 = false, bool FW = false>
+template <int n_lo, bool FULL, bool RBN, bool GSN = false, bool D64 = false, bool FW = false,
+          bool AL = true>
 __device__ __forceinline__ void strip2_body(const IterArgs& A,
                                             StripShared2<strip_ring_rows(n_lo), strip_fields(RBN)>& ws,
                                             int lane, int b, int s, int k, int rd, int x0, int y0,
@@ -323,6 +333,7 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
   const int RH = own_rows + 2 * E;
   const int gx = x0 - P + 2 * lane;               // even; the pair is gx, gx + 1
   const bool gx_ok = gx >= 0 && gx < I.mx;        // both columns (even width)
+  const bool gx_ok2 = AL ? gx_ok : gx + 1 >= 0 && gx + 1 < I.mx;  // the second one
   const bool own_lane = (FW || (lane >= n_lo && lane < 32 - n_lo)) && gx_ok;
   const int gy0 = y0 - E;
 
@@ -365,7 +376,17 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
     return ring + RING * 2 * 64 + (((r + STRIP_SHORT) & (STRIP_SHORT - 1)) * NF + f) * 64;
   };
   auto ld2 = [](const double* p) { return *reinterpret_cast<const double2*>(p); };
-  const int gxc = min(max(gx, 0), I.mx - 2);
+  auto store2 = [&](double* p, double vx, double vy) {
+    if constexpr (AL) {
+      *reinterpret_cast<double2*>(p) = make_double2(vx, vy);
+    } else {
+      p[0] = vx;
+      if (gx_ok2) p[1] = vy;
+    }
+  };
+  const int gxc = min(max(gx, 0), I.mx - (AL ? 2 : 1));
+  // the pair's second column in a row of the grid (its address, if inside)
+  const int c2 = AL || gx_ok2 ? 1 : 0;
   const int mx = I.mx, my = I.my;
   auto fetch = [&](int rj, int dj) {
     const int gy = gy0 + rj;
@@ -373,17 +394,30 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
     const int c = min(max(gy, 0), my - 1) * mx + gxc;
     double* d = slot_at(dj, 0);
     double* e = sslot_row(rj, 0);
-    cp_async16_zfill(d + RB_X * 64, Xg + c, ok);
-    cp_async16_zfill(d + RB_L * 64, Lg + c, ok);
-    cp_async16_zfill(e + RS_XP * 64, XPg + c, ok);
-    cp_async16_zfill(e + RS_LN * 64, (last ? Lg : LNg) + c, ok && !last);
-    if constexpr (full)
-      cp_async16_zfill(e + RS_RF * 64, RFg + c, ok);
-    else  // the first 8 bytes of the pair's slot
+    auto pair = [&](double* dst, const double* src, bool ok2) {
+      if constexpr (AL) {
+        cp_async16_zfill(dst, src + c, ok2);
+      } else {
+        cp_async8_zfill(dst, src + c, ok2);
+        cp_async8_zfill(dst + 1, src + c + c2, ok2 && gx_ok2);
+      }
+    };
+    pair(d + RB_X * 64, Xg, ok);
+    pair(d + RB_L * 64, Lg, ok);
+    pair(e + RS_XP * 64, XPg, ok);
+    pair(e + RS_LN * 64, last ? Lg : LNg, ok && !last);
+    if constexpr (full) {
+      pair(e + RS_RF * 64, RFg, ok);
+    } else if constexpr (AL) {  // the first 8 bytes of the pair's slot
       cp_async8_zfill(e + RS_RF * 64, RFf + c, ok);
+    } else {
+      float* f = reinterpret_cast<float*>(e + RS_RF * 64);
+      cp_async4_zfill(f, RFf + c, ok);
+      cp_async4_zfill(f + 1, RFf + c + c2, ok && gx_ok2);
+    }
     if constexpr (RBN) {
-      cp_async16_zfill(e + RS_XPN * 64, XPNg + c, ok);
-      cp_async16_zfill(e + RS_LNN * 64, (last ? Lg : LNNg) + c, ok && !last);
+      pair(e + RS_XPN * 64, XPNg, ok);
+      pair(e + RS_LNN * 64, last ? Lg : LNNg, ok && !last);
     }
     asm volatile("cp.async.commit_group;\n" ::);
   };
@@ -491,9 +525,14 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
         const double K1x = xp.x - x.x + t1x, K1y = xp.y - x.y + t1y;
         const double K3x = lnv.x - lam.x + t3x, K3y = lnv.y - lam.y + t3y;
         if (own) {
-          nm.vmax = fmax(nm.vmax, fmax(fmax(abs_or_inf(K1x), abs_or_inf(K3x)),
-                                       fmax(abs_or_inf(K1y), abs_or_inf(K3y))));
-          nm.vsq += K1x * K1x + K3x * K3x + K1y * K1y + K3y * K3y;
+          if (AL || gx_ok2) {
+            nm.vmax = fmax(nm.vmax, fmax(fmax(abs_or_inf(K1x), abs_or_inf(K3x)),
+                                         fmax(abs_or_inf(K1y), abs_or_inf(K3y))));
+            nm.vsq += K1x * K1x + K3x * K3x + K1y * K1y + K3y * K3y;
+          } else {
+            nm.vmax = fmax(nm.vmax, fmax(abs_or_inf(K1x), abs_or_inf(K3x)));
+            nm.vsq += K1x * K1x + K3x * K3x;
+          }
         }
         if constexpr (RBN) {
           const double2 xpn = ld2(qs + RS_XPN * 64);
@@ -528,8 +567,11 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
         F2 K3f = K3h;
         if (last)  // the product rounded on its own (packed operations would be contracted)
           K3f = F2{__fadd_rn(K3h.x, __fmul_rn(hqff.x, dr.x)), __fadd_rn(K3h.y, __fmul_rn(hqff.y, dr.y))};
-        const float k1m = fmax_nan(fabsf(K1f.x), fabsf(K1f.y)), k3m = fmax_nan(fabsf(K3f.x), fabsf(K3f.y));
-        const F2 sq2 = fma2(K1f, K1f, K3f * K3f);
+        // the norms' terms (an outside second column contributes nothing)
+        const bool two = AL || gx_ok2;
+        const F2 n1 = F2{K1f.x, two ? K1f.y : 0.0f}, n3 = F2{K3f.x, two ? K3f.y : 0.0f};
+        const float k1m = fmax_nan(fabsf(n1.x), fabsf(n1.y)), k3m = fmax_nan(fabsf(n3.x), fabsf(n3.y));
+        const F2 sq2 = fma2(n1, n1, n3 * n3);
         if (own) {
           nm.mg.z = fmaxf(nm.mg.z, fmaxf(fmaxf(fabsf(dx.x), fabsf(dl.x)),
                                          fmaxf(fabsf(dx.y), fabsf(dl.y))));
@@ -590,7 +632,7 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
       }
       // 1/diag F_x, zero outside the grid (every sweep there stays zero)
       const F2 dg = F2{-1.0f, -1.0f} - th * tdc * dp;
-      rg = in_grid ? F2{__frcp_rn(dg.x), __frcp_rn(dg.y)} : F2{0.f, 0.f};
+      rg = in_grid ? F2{__frcp_rn(dg.x), AL || gx_ok2 ? __frcp_rn(dg.y) : 0.f} : F2{0.f, 0.f};
       v1 = (th * tb0 * inj - K1) * rg;  // first F_x sweep of F_x v5 = F_u v3 - K1
     }
     if (!resid_only) {
@@ -602,10 +644,8 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
           const F2 w = (F2{0.f, 0.f} - K3 - ax * v1) * rg;
           const double* rs = slot_at(-1, 0);
           const double2 xo = ld2(rs + RB_X * 64), lo = ld2(rs + RB_L * 64);
-          *reinterpret_cast<double2*>(Xo + c) =
-              make_double2(fma(alpha, f2d_upd(v1.x), xo.x), fma(alpha, f2d_upd(v1.y), xo.y));
-          *reinterpret_cast<double2*>(Lo + c) =
-              make_double2(fma(alpha, f2d_upd(w.x), lo.x), fma(alpha, f2d_upd(w.y), lo.y));
+          store2(Xo + c, fma(alpha, f2d_upd(v1.x), xo.x), fma(alpha, f2d_upd(v1.y), xo.y));
+          store2(Lo + c, fma(alpha, f2d_upd(w.x), lo.x), fma(alpha, f2d_upd(w.y), lo.y));
         }
       } else {
         pw[0].push(dp * v1);
@@ -641,10 +681,8 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
               const F2 v5m = sv5.d[E - n_lo - 1];
               const double* rs = slot_at(-E, 0);  // still in the ring
               const double2 xo = ld2(rs + RB_X * 64), lo = ld2(rs + RB_L * 64);
-              *reinterpret_cast<double2*>(Xo + c) =
-                  make_double2(fma(alpha, f2d_upd(v5m.x), xo.x), fma(alpha, f2d_upd(v5m.y), xo.y));
-              *reinterpret_cast<double2*>(Lo + c) =
-                  make_double2(fma(alpha, f2d_upd(v4.x), lo.x), fma(alpha, f2d_upd(v4.y), lo.y));
+              store2(Xo + c, fma(alpha, f2d_upd(v5m.x), xo.x), fma(alpha, f2d_upd(v5m.y), xo.y));
+              store2(Lo + c, fma(alpha, f2d_upd(v4.x), lo.x), fma(alpha, f2d_upd(v4.y), lo.y));
             }
           }
         }
@@ -727,7 +765,7 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
 // One upper-layer iteration over the strip work list with two columns per
 // lane (the strip list's x0 advance by 64 - 2 strip2_pad(n_lo)); control flow
 // as k_strip.
-template <int n_lo, bool RBN, bool D64 = false, bool FW = false>
+template <int n_lo, bool RBN, bool D64 = false, bool FW = false, bool AL = true>
 __global__ void __launch_bounds__(STRIP2_WARPS * 32, STRIP2_MIN_BLOCKS)
     k_strip2(IterArgs A, int MODE, int j_launch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -784,10 +822,10 @@ __global__ void __launch_bounds__(STRIP2_WARPS * 32, STRIP2_MIN_BLOCKS)
     resid_only = (k == A.max_iter);
   }
   if (full)
-    strip2_body<n_lo, true, RBN, false, D64, FW>(A, ws, lane, b, s, k, rd, x0, y0, sy, resid_only);
+    strip2_body<n_lo, true, RBN, false, D64, FW, AL>(A, ws, lane, b, s, k, rd, x0, y0, sy, resid_only);
   else if (RBN && !D64 && MODE == MODE_SOLVE)
     strip2_body<n_lo, false, false, true>(A, *reinterpret_cast<WS3*>(wbase), lane, b, s, k, rd,
                                           x0, y0, sy, resid_only);
   else
-    strip2_body<n_lo, false, RBN, false, D64, FW>(A, ws, lane, b, s, k, rd, x0, y0, sy, resid_only);
+    strip2_body<n_lo, false, RBN, false, D64, FW, AL>(A, ws, lane, b, s, k, rd, x0, y0, sy, resid_only);
 }

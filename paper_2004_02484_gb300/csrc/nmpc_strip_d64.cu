@@ -8,13 +8,18 @@ namespace nmpc_dev {
 #include "nmpc_patch.cuh"
 }  // namespace nmpc_dev
 
-using nmpc_dev::k_strip2;
+namespace {
+template <int n_lo, bool FW, bool AL>
+StripKernel half_of(bool rbn) {
+  return rbn ? nmpc_dev::k_strip2<n_lo, true, true, FW, AL> : nmpc_dev::k_strip2<n_lo, false, true, FW, AL>;
+}
+template <int n_lo>
+StripKernel shape_of(bool rbn, bool full_width, bool aligned) {
+  if (full_width) return aligned ? half_of<n_lo, true, true>(rbn) : half_of<n_lo, true, false>(rbn);
+  return aligned ? half_of<n_lo, false, true>(rbn) : half_of<n_lo, false, false>(rbn);
+}
+}  // namespace
 
-StripKernel strip_d64_kernel(int n_lo, bool rbn, bool full_width) {
-  if (n_lo <= 1) {
-    if (full_width) return rbn ? k_strip2<1, true, true, true> : k_strip2<1, false, true, true>;
-    return rbn ? k_strip2<1, true, true, false> : k_strip2<1, false, true, false>;
-  }
-  if (full_width) return rbn ? k_strip2<2, true, true, true> : k_strip2<2, false, true, true>;
-  return rbn ? k_strip2<2, true, true, false> : k_strip2<2, false, true, false>;
+StripKernel strip_d64_kernel(int n_lo, bool rbn, bool full_width, bool aligned) {
+  return n_lo <= 1 ? shape_of<1>(rbn, full_width, aligned) : shape_of<2>(rbn, full_width, aligned);
 }

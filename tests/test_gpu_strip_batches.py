@@ -27,7 +27,8 @@ def G():
 
 # (mx, my, horizon, instances): the narrowest grid, 64 columns and the first
 # grids of two strips, heights off the strips' rows, enough stages for strips
-SIZES = [(24, 17, 7, 130), (62, 33, 20, 24), (64, 64, 50, 10), (66, 40, 30, 12), (112, 25, 20, 30),
+# and odd widths (columns copied one by one, a last pair half outside)
+SIZES = [(25, 18, 9, 100), (63, 40, 20, 24), (65, 37, 25, 16), (113, 31, 24, 20), (24, 17, 7, 130), (62, 33, 20, 24), (64, 64, 50, 10), (66, 40, 30, 12), (112, 25, 20, 30),
          (114, 31, 24, 20)]
 
 
