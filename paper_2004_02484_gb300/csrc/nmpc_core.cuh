@@ -66,6 +66,9 @@ struct IterArgs {
   int n_work;
   int n_inst;
   const int* act;
+  // cluster path, n_lo <= 2: per grid cell (packed as x0) the grid steps to the
+  // nearest actuator, 255 beyond 2; null: not used
+  const unsigned char* act_dist;
   const double* x0;
   const double* ref;
   // state buffers: solve mode reads [k & 1] and writes [(k + 1) & 1];

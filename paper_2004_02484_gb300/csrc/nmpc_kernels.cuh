@@ -458,6 +458,23 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
   struct V2 {
     T v, w;
   };
+  // The slots whose cells an application after the first recomputes: F_u v3
+  // changes on the actuator cells only, so v5 and the first F_x^T sweep change
+  // within n_lo - 1 grid steps of one and v4 within 2 (n_lo - 1); every other
+  // cell keeps the bits that it would get again (n_lo <= 2: no field serves two
+  // sweeps).  Three full applications a cell were most of a float64
+  // iteration's arithmetic.
+  unsigned near1 = 0xffffffffu, near2 = 0xffffffffu;
+  if (!MULTI && A.act_dist != nullptr && n_full > 1 && n_lo <= 2) {
+    near1 = near2 = 0u;
+#pragma unroll
+    for (int k2 = 0; k2 < NC; ++k2) {
+      if (!((c0.valid >> k2) & 1u)) continue;
+      const int d = A.act_dist[I.g_off + g.lo + tid + k2 * bd];
+      near1 |= (d <= n_lo - 1 ? 1u : 0u) << k2;
+      near2 |= (d <= 2 * (n_lo - 1) ? 1u : 0u) << k2;
+    }
+  }
   for (int it = 0; it < n_full; ++it) {
     if (it > 0) {
       // c4 = F_u v3 - K1 changes only on actuator cells: refresh v1, p1 there
@@ -492,15 +509,19 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
     if (n_lo == 1) {
       pass<NC, NC, MULTI, T>(g, c0,
           [&](const Slot& sl, const Cells<NC>&) {
+            if (it > 0 && !((near1 >> sl.k) & 1u)) return T(0);
             const int pb = wpos(sl.p);
             return (-WV(pb, F_B2) - WV(pb, F_AX) * WV(pb, F_V1)) * WV(pb, F_RG);
           },
-          [&](const Slot& sl, const Cells<NC>& cs, T w) { put(cs, sl, F_W1, w); });
+          [&](const Slot& sl, const Cells<NC>& cs, T w) {
+            if (it == 0 || ((near1 >> sl.k) & 1u)) put(cs, sl, F_W1, w);
+          });
     } else {
       cur = F_Y5;
       const bool lastsw = (n_lo == 2);
       pass<NC, NC, MULTI, V2>(g, c0,
           [&](const Slot& sl, const Cells<NC>&) {
+            if (it > 0 && !((near1 >> sl.k) & 1u)) return V2{T(0), T(0)};
             const int pb = wpos(sl.p);
             const T off = th * (tcx * (WV(pb - RB, F_P1) + WV(pb + RB, F_P1)) +
                                 tcy * (WV(pb - WRB, F_P1) + WV(pb + WRB, F_P1)));
@@ -508,6 +529,7 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
             return V2{v, (-WV(pb, F_B2) - WV(pb, F_AX) * v) * WV(pb, F_RG)};
           },
           [&](const Slot& sl, const Cells<NC>& cs, V2 o) {
+            if (it > 0 && !((near1 >> sl.k) & 1u)) return;
             if (wide) put(cs, sl, F_Y5, o.v);
             else if (sl.v) WV(wpos(sl.p), F_Y5) = o.v;
             if (lastsw) put(cs, sl, F_W1, o.w);
@@ -541,6 +563,7 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
       cur = F_Y4;
       pass<NC, NC, MULTI, T>(g, c0,
           [&](const Slot& sl, const Cells<NC>&) {
+            if (it > 0 && !((near2 >> sl.k) & 1u)) return T(0);
             const int pb = wpos(sl.p);
             const T off = th * WV(pb, F_DP) *
                           (tcx * (WV(pb - RB, F_W1) + WV(pb + RB, F_W1)) +
@@ -548,6 +571,7 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
             return WV(pb, F_W1) - WV(pb, F_RG) * off;
           },
           [&](const Slot& sl, const Cells<NC>& cs, T v) {
+            if (it > 0 && !((near2 >> sl.k) & 1u)) return;
             if (wide) put(cs, sl, F_Y4, v);
             else if (sl.v) WV(wpos(sl.p), F_Y4) = v;
           });
