@@ -355,6 +355,11 @@ __device__ __forceinline__ double abs_or_inf(double v) {
   return (a <= 1.79e308) ? a : CUDART_INF;  // NaN and Inf count as +Inf
 }
 
+// Bits of |v|: non-negative doubles order as integers, NaN above infinity.
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+
 // max(a, b) that returns NaN when either is NaN (one instruction)
 __device__ __forceinline__ float fmax_nan(float a, float b) {
   float d;

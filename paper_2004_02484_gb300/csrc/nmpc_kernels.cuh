@@ -311,6 +311,9 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
     }
   };
   if (full) {
+    // the maximum on integers: comparisons of doubles go to the two-lane
+    // float64 pipe, six a cell
+    unsigned long long vbits = 0ull;
     pass<NC, 1, MULTI, P2Out>(g, c0,
         [&](const Slot& sl, const Cells<NC>&) {
           P2Out o{T(0), T(0), T(0), T(0), false};
@@ -351,7 +354,7 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
           const double K1 = __fma_rn(h, s1, xp - x);
           const double K3 = __fma_rn(h, s3, ln - lam);
           if (valid) {
-            vmax = fmax(vmax, fmax(abs_or_inf(K1), abs_or_inf(K3)));
+            vbits = max(vbits, max(abs_bits(K1), abs_bits(K3)));
             vsq += K1 * K1 + K3 * K3;
           }
           double K1r = K1, K3r = K3;
@@ -366,6 +369,8 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
           return o;
         },
         p2_store);
+    // (NaN counts as infinite)
+    vmax = __longlong_as_double((long long)min(vbits, 0x7ff0000000000000ull));
   } else {
     const float cxf = I.fcx, cyf = I.fcy, dcf = I.fdc, hf = I.fh;
     const float k0f_ = I.fk0, k1f_ = I.fk1, qf_ = I.fq, b0f = I.fb0;
