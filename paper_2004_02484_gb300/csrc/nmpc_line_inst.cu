@@ -412,13 +412,26 @@ __global__ void __launch_bounds__(32 * li_max_warps(CPL), 1)
       publish((unsigned long long)__double_as_longlong(vmax), RES_FULL_MARK, vsq);
     } else {
       for (int o = 16; o > 0; o >>= 1) fs += __shfl_xor_sync(0xffffffffu, fs, o);
-      publish((unsigned long long)__double_as_longlong(f2d(warp_max_nn(fmx))),
-              (unsigned long long)__double_as_longlong(e_max), f2d(fs));
+      // (as the bits of the floats that the norm and the bound are)
+      publish(__float_as_uint(warp_max_nn(fmx)), __float_as_uint((float)e_max), f2d(fs));
     }
   };
-  // the instance's norms: every warp reduces what all of them published
-  auto collect = [&](unsigned long long& r, unsigned long long& e) {
+  // the instance's norms: every warp reduces what all of them published (a
+  // split pass's are floats widened: their maxima in two warp reductions)
+  auto collect = [&](unsigned long long& r, unsigned long long& e, bool full) {
     r = e = 0ull;
+    if (!full) {
+      unsigned rf = 0u, ef = 0u;
+      for (int w = lane; w < wt; w += 32) {
+        rf = max(rf, (unsigned)red_r[w]);
+        ef = max(ef, (unsigned)red_e[w]);
+      }
+      rf = __reduce_max_sync(0xffffffffu, rf);
+      ef = __reduce_max_sync(0xffffffffu, ef);
+      r = (unsigned long long)__double_as_longlong(f2d(__uint_as_float(rf)));
+      e = (unsigned long long)__double_as_longlong(f2d(__uint_as_float(ef)));
+      return;
+    }
     for (int w = lane; w < wt; w += 32) {
       r = max(r, red_r[w]);
       e = max(e, red_e[w]);
@@ -437,7 +450,7 @@ __global__ void __launch_bounds__(32 * li_max_warps(CPL), 1)
     bool full = (k == A.max_iter) || (k == 0 && f0);
     if (k > 0) {
       unsigned long long rb, eb;
-      collect(rb, eb);
+      collect(rb, eb, prev_full);
       r = __longlong_as_double((long long)rb);
       if (k == 1) r0 = r;
       if (threadIdx.x == 0) {  // read by later iterations' decisions
@@ -462,7 +475,7 @@ __global__ void __launch_bounds__(32 * li_max_warps(CPL), 1)
       stages(std::true_type{}, false, true);
       sync_all();
       unsigned long long rb, eb;
-      collect(rb, eb);
+      collect(rb, eb, true);
       r = __longlong_as_double((long long)rb);
       if (k == 0) r0 = r;
       if (k == A.max_iter)
