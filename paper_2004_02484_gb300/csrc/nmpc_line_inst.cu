@@ -88,10 +88,11 @@ __device__ __forceinline__ void li_nsum(const V (&v)[CPL], V (&out)[CPL], int la
 // What bounds it: the float64 pipe (56% busy on 304 instances of 256 cells:
 // two differences and two updates a cell) and latency (0.45 instructions a
 // cycle a scheduler, 16 warps a SM at 128 registers).  1024 ragged instances
-// (M 32..256, N 10..60): 54.6 -> 41.2 ms a solve; one instance of M = 32,
-// N = 20 on 8 CTAs: 1007 -> 561 us (828 us on one CTA, whose warps share one
-// float64 pipe).
-template <int CPL>
+// (M 32..256, N 10..60): 54.6 -> 41.2 ms a solve, 37.8 with the sweeps a
+// constant; one instance of M = 32, N = 20 on 8 CTAs: 1007 -> 561 us, 506 with
+// the constant (828 us on one CTA, whose warps share one float64 pipe).
+// NLO: the sweeps per solve as a constant (2, the default), or 0 to read them.
+template <int CPL, int NLO>
 __global__ void __launch_bounds__(32 * li_max_warps(CPL), 1)
     k_line_inst(IterArgs A, const int* list, int csize, int rows_max, int nu_max, int* retry) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(32 * li_max_warps(CPL), 1)
 
   const float th = I.fh, tdc = I.fdc, tcx = I.fcx, tb0 = I.fb0;
   const double alpha = A.alpha;
-  const int n_lo = A.n_lo, n_u_it = A.n_u_it;
+  const int n_lo = NLO > 0 ? NLO : A.n_lo, n_u_it = A.n_u_it;
   double xp[CPL];  // x_{i-1} of iterate k, the lane's cells
 
   // x below the warp's first stage into xp; lambda above its last one into NX
@@ -357,10 +358,25 @@ __global__ void __launch_bounds__(32 * li_max_warps(CPL), 1)
 #pragma unroll
         for (int t = 0; t < CPL; ++t) y5[t] = v1[t];
         for (int sw = 1; sw < n_lo; ++sw) {
+          // the neighbours' Phi' sweep, a product inside the lane rounded with
+          // the sum where k_line's were
           float pw[CPL];
 #pragma unroll
-          for (int t = 0; t < CPL; ++t) pw[t] = dp[t] * y5[t];
-          li_nsum<CPL, float>(pw, ns, lane);
+          for (int t = 0; t < CPL; ++t) pw[t] = __fmul_rn(dp[t], y5[t]);
+          float lft = __shfl_up_sync(0xffffffffu, pw[CPL - 1], 1);
+          float rgt = __shfl_down_sync(0xffffffffu, pw[0], 1);
+          lft = (lane == 0) ? 0.0f : lft;
+          rgt = (lane == 31) ? 0.0f : rgt;
+#pragma unroll
+          for (int t = 0; t < CPL; ++t) {
+            const int tl = t > 0 ? t - 1 : 0, tr = t < CPL - 1 ? t + 1 : 0;
+            const float l = t > 0 ? pw[tl] : lft, r = t < CPL - 1 ? pw[tr] : rgt;
+            // (not the lane's first and last, which its neighbours read too)
+            const bool fl = t - 1 >= 1 && t - 1 <= CPL - 2, fr = t + 1 <= CPL - 2;
+            if (fl) ns[t] = __fmaf_rn(dp[tl], y5[tl], r);
+            else if (fr) ns[t] = __fmaf_rn(dp[tr], y5[tr], l);
+            else ns[t] = __fadd_rn(l, r);
+          }
 #pragma unroll
           for (int t = 0; t < CPL; ++t) y5[t] = __fmaf_rn(-rg[t], __fmul_rn(th, __fmul_rn(tcx, ns[t])), v1[t]);
         }
@@ -538,14 +554,16 @@ using nmpc_dev::InstDev;
 using nmpc_dev::IterArgs;
 using Kernel = void (*)(IterArgs, const int*, int, int, int, int*);
 
-Kernel kernel_of(int cpl) {
+template <int NLO>
+Kernel kernel_with(int cpl) {
   switch (cpl) {
-    case 1: return nmpc_dev::k_line_inst<1>;
-    case 2: return nmpc_dev::k_line_inst<2>;
-    case 4: return nmpc_dev::k_line_inst<4>;
-    default: return nmpc_dev::k_line_inst<8>;
+    case 1: return nmpc_dev::k_line_inst<1, NLO>;
+    case 2: return nmpc_dev::k_line_inst<2, NLO>;
+    case 4: return nmpc_dev::k_line_inst<4, NLO>;
+    default: return nmpc_dev::k_line_inst<8, NLO>;
   }
 }
+Kernel kernel_of(int cpl, int n_lo) { return n_lo == 2 ? kernel_with<2>(cpl) : kernel_with<0>(cpl); }
 
 // Cells per lane, as on the line path: the smallest of 1, 2, 4, 8 that covers
 // mx (at most 256) cells.
@@ -612,9 +630,11 @@ std::vector<LineInstLaunch> line_inst_plan(const std::vector<InstDev>& inst,
 // function's, whichever handle launches it).
 cudaError_t line_inst_configure(int max_smem) {
   for (int cpl = 1; cpl <= 8; cpl *= 2) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        kernel_of(cpl), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-    if (e != cudaSuccess) return e;
+    for (int n_lo = 1; n_lo <= 2; ++n_lo) {
+      const cudaError_t e = cudaFuncSetAttribute(
+          kernel_of(cpl, n_lo), cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+      if (e != cudaSuccess) return e;
+    }
   }
   return cudaSuccess;
 }
@@ -642,7 +662,7 @@ cudaError_t line_inst_solve(const std::vector<LineInstLaunch>& plan, const IterA
     }
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel_of(L.cpl), A, list_d + L.first, L.csize,
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel_of(L.cpl, A.n_lo), A, list_d + L.first, L.csize,
                                              L.rows, L.nu, retry);
     if (e != cudaSuccess) return e;
   }
