@@ -76,12 +76,13 @@ __host__ __device__ constexpr size_t stage_bytes(int ng) {
 // divisions, sit in the group's first nu threads, so that one or two warps
 // execute them and not every warp that owns an actuator point; the maximum
 // norm is taken on integers.  1024 plates of 13x13, N = 20, float64: 326 ->
-// 144 ms a solve; one plate: 4.8 -> 2.4 ms.
+// 144 ms a solve, 140 with the sweeps a constant; one plate: 4.8 -> 2.3 ms.
 // F_x = h (L diag(Phi'(w)) - diag(beta + 4 gr x^3)) - I on the state points;
 // v is zero at the actuator points.  The lower layer runs in T (float64, or
 // float32 in mixed precision: the residual, the coefficients and the update
 // stay float64, so the fixed point is the float64 root).
-template <typename T, int PPT, bool NEU, bool D2>
+// NLO: the sweeps per solve as a constant (2, the default), or 0 to read them.
+template <typename T, int PPT, bool NEU, bool D2, int NLO>
 __global__ void __launch_bounds__(PPT == 1 ? 256 : 512, PPT == 1 ? 3 : 2)
     k_plate_dir(PArgs A, Ctl C, Iter S, stage_drv::Range R) {
   extern __shared__ __align__(16) double smem[];
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(PPT == 1 ? 256 : 512, PPT == 1 ? 3 : 2)
   T v5[PPT], v4[PPT];
 #pragma unroll
   for (int j = 0; j < PPT; ++j) v5[j] = v4[j] = T(0);
-  const int n_lo = A.n_lo;
+  const int n_lo = NLO > 0 ? NLO : A.n_lo;
   T *ex = fC, *ex2 = fD;  // the next exchange's field, the other one
   for (int itu = 0; itu <= A.n_u_it; ++itu) {
     if (itu > 0) {
@@ -427,14 +428,20 @@ PArgs make_args(const nmpc_plate* h) {
 
 // k_plate_dir for a group of stages.
 using DirKernel = void (*)(PArgs, stage_drv::Ctl, stage_drv::Iter, stage_drv::Range);
-template <typename T, int PPT>
+template <typename T, int PPT, int NLO>
 DirKernel dir_kernel_of(bool neu, bool d2) {
-  if (neu) return d2 ? plate_dev::k_plate_dir<T, PPT, true, true> : plate_dev::k_plate_dir<T, PPT, true, false>;
-  return d2 ? plate_dev::k_plate_dir<T, PPT, false, true> : plate_dev::k_plate_dir<T, PPT, false, false>;
+  using namespace plate_dev;
+  if (neu) return d2 ? k_plate_dir<T, PPT, true, true, NLO> : k_plate_dir<T, PPT, true, false, NLO>;
+  return d2 ? k_plate_dir<T, PPT, false, true, NLO> : k_plate_dir<T, PPT, false, false, NLO>;
 }
-DirKernel dir_kernel(bool mixed, const stage_drv::Group& g) {
-  if (mixed) return g.ppt == 1 ? dir_kernel_of<float, 1>(g.neu, g.d2) : dir_kernel_of<float, 2>(g.neu, g.d2);
-  return g.ppt == 1 ? dir_kernel_of<double, 1>(g.neu, g.d2) : dir_kernel_of<double, 2>(g.neu, g.d2);
+template <int NLO>
+DirKernel dir_kernel_with(bool mixed, const stage_drv::Group& g) {
+  if (mixed)
+    return g.ppt == 1 ? dir_kernel_of<float, 1, NLO>(g.neu, g.d2) : dir_kernel_of<float, 2, NLO>(g.neu, g.d2);
+  return g.ppt == 1 ? dir_kernel_of<double, 1, NLO>(g.neu, g.d2) : dir_kernel_of<double, 2, NLO>(g.neu, g.d2);
+}
+DirKernel dir_kernel(bool mixed, int n_lo, const stage_drv::Group& g) {
+  return n_lo == 2 ? dir_kernel_with<2>(mixed, g) : dir_kernel_with<0>(mixed, g);
 }
 size_t stage_smem(bool mixed, const stage_drv::Group& g) {
   return mixed ? plate_dev::stage_bytes<float>(g.ng_max) : plate_dev::stage_bytes<double>(g.ng_max);
@@ -452,7 +459,7 @@ struct PlateDir {
       A.half = half;
       for (const stage_drv::Group& g : h->drv.groups) {
         const cudaError_t e =
-            stage_drv::launch_stages(dir_kernel(mixed, g), stage_smem(mixed, g),
+            stage_drv::launch_stages(dir_kernel(mixed, A.n_lo, g), stage_smem(mixed, g),
                                      stage_drv::range_of(g, A.rb != 0, half), A, C, S, st);
         if (e != cudaSuccess) return e;
       }
