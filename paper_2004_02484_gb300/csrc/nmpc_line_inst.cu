@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <map>
+#include <tuple>
 
 namespace nmpc_dev {
 
@@ -584,33 +585,51 @@ std::vector<LineInstLaunch> line_inst_plan(const std::vector<InstDev>& inst,
                                            int max_smem, std::vector<int>* list) {
   std::vector<LineInstLaunch> plan;
   list->clear();
-  // few instances: as many warps as stages, for the shortest iteration; a
-  // batch: CTAs of which two or more share a SM, so that one computes while
-  // the other waits at its barrier
-  const bool few = (int)which.size() * 2 <= num_sms;
-  std::map<std::pair<int, int>, std::vector<int>> classes;  // (cells per lane, CTAs) -> instances
+  // few instances (their CTAs have a SM each): as many warps as stages, for
+  // the shortest iteration; a batch: CTAs of which two or more share a SM, so
+  // that one computes while the other waits at its barrier
+  const int n = (int)which.size();
+  // CTAs an instance may take for speed (256 cells, N = 60, us an iteration:
+  // 20 instances on clusters of four 12.7, of two 21.6; 64 cells, N = 20, 76
+  // instances 5.9 against 10.6 in the batch form).  Clusters of four fill 144
+  // of 152 SMs; a 37th would wait for a place (24.7).
+  int spread = 1;
+  while (spread < 8 && n * spread * 2 <= num_sms - (spread > 1 ? num_sms / 19 : 0)) spread *= 2;
+  auto most_warps = [](bool few, int cpl) {
+    return few ? nmpc_dev::li_max_warps(cpl) : std::min(8, nmpc_dev::li_max_warps(cpl) / 2);
+  };
+  auto ctas_of = [&](bool few, int cpl, const InstDev& I) {  // 0: does not fit
+    const size_t room = few ? (size_t)max_smem : std::min<size_t>(max_smem, 110 * 1024);
+    for (int c = 1; c <= 8; c *= 2) {
+      const int w = std::min(most_warps(few, cpl), (I.N + c - 1) / c);
+      if (c * w > nmpc_dev::LI_MAX_WARPS) return 0;
+      // few: at most four stages a SM, whose warps share its float64 pipe
+      if (few && c < spread && c * 4 < I.N) continue;
+      if (nmpc_dev::li_layout(cpl, rows_of(I.N, c, w), w, I.nu).bytes <= room) return c;
+    }
+    return 0;
+  };
+  // (cells per lane, CTAs, few) -> instances
+  std::map<std::tuple<int, int, bool>, std::vector<int>> classes;
   for (int b : which) {
     const InstDev& I = inst[b];
     const int cpl = li_cells_per_lane(I.mx);
-    const int wmax = few ? nmpc_dev::li_max_warps(cpl) : std::min(8, nmpc_dev::li_max_warps(cpl) / 2);
-    const size_t room = few ? (size_t)max_smem : std::min<size_t>(max_smem, 110 * 1024);
-    int c = 1;
-    for (;; c *= 2) {
-      const int w = std::min(wmax, (I.N + c - 1) / c);
-      if (c > 8 || c * w > nmpc_dev::LI_MAX_WARPS) return {};
-      // few: at most four stages a SM, whose warps share its float64 pipe
-      if (few && c < 8 && c * 4 < I.N) continue;
-      if (nmpc_dev::li_layout(cpl, rows_of(I.N, c, w), w, I.nu).bytes <= room) break;
-    }
-    classes[{cpl, c}].push_back(b);
+    int c = ctas_of(true, cpl, I);
+    // (eight cells a lane and more stages than warps: 38 .. 72 instances of 256
+    // cells, N = 60, 21.7 us, in the batch form 19.5 .. 20.3; with fewer cells a
+    // lane more warps fit: 128 cells 15.0 against 17.7)
+    const bool few = c > 0 && n * c <= num_sms &&
+                     !(cpl == 8 && c > 1 && I.N > c * most_warps(true, cpl));
+    if (!few) c = ctas_of(false, cpl, I);
+    if (!c) return {};
+    classes[{cpl, c, few}].push_back(b);
   }
   for (auto it = classes.rbegin(); it != classes.rend(); ++it) {
-    const int cpl = it->first.first, c = it->first.second;
+    const int cpl = std::get<0>(it->first), c = std::get<1>(it->first);
     std::vector<int>& v = it->second;
     std::stable_sort(v.begin(), v.end(), [&](int a, int b) { return inst[a].N > inst[b].N; });
     LineInstLaunch L{cpl, c, 0, (int)list->size(), (int)v.size(), 0, 0, 0};
-    const int wmax = few ? nmpc_dev::li_max_warps(cpl) : std::min(8, nmpc_dev::li_max_warps(cpl) / 2);
-    L.warps = std::min(wmax, (inst[v[0]].N + c - 1) / c);
+    L.warps = std::min(most_warps(std::get<2>(it->first), cpl), (inst[v[0]].N + c - 1) / c);
     int rows = 0, nu = 0;
     for (int b : v) {
       rows = std::max(rows, rows_of(inst[b].N, c, L.warps));
