@@ -1574,18 +1574,24 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       }
     if (o.strip_rows) {
       ty = std::min(o.strip_rows, my_max);
-    } else if (d64) {
+    } else if (two) {
       // a row step takes about 1.5 us whatever the number of resident warps
       // (12 a SM), so a launch takes its waves times the rows of a strip's
-      // region and pipeline: the split of the columns with the fewest
+      // region and pipeline: the split of the columns with the fewest (three
+      // 156x110, N = 96, red-black: 28 rows and one wave a half, 112 us an
+      // iteration, where 16 rows, two waves, took 141)
       const long long room = 4LL * STRIP2_MIN_BLOCKS * std::max(1, h->num_sms);
       long long best = 0;
-      for (int segs = 1; segs == 1 || (my_max + segs - 1) / segs >= 4; ++segs) {
+      const int least = d64 ? 4 : 16;
+      for (int segs = 1; segs == 1 || (my_max + segs - 1) / segs >= least; ++segs) {
         const int rows = (my_max + segs - 1) / segs;
         long long warps = 0;
-        for (const InstDev& I : h->inst_h)
+        for (int b = 0; b < n_instances; ++b) {
+          if (!on_strips[b]) continue;
+          const InstDev& I = h->inst_h[b];
           warps += (long long)(h->rb ? (I.N + 1) / 2 : I.N) * ((I.mx + tx - 1) / tx) *
                    ((I.my + rows - 1) / rows);
+        }
         const long long cost = ((warps + room - 1) / room) * (rows + 3 * E);
         if (segs == 1 || cost < best) {
           best = cost;
