@@ -123,7 +123,8 @@ typedef struct {
                       residual stays.  Convergence is only ever declared on
                       a float64 residual.  Handles with strip-path instances
                       use max(split_min, 1e-6): their split residual takes
-                      the stage differences from float32 values        */
+                      the stage differences from float32 values (not so
+                      where strips = 0 took stages that fit a cluster)  */
   int u_local;     /* 1: the u-iteration uses the actuators' local responses
                       (P^{-1} is a fixed linear map, so Y(v3) = Y(0) + sum_b
                       v3_b Z(e_b) with Z(e_b) zero outside 2(n_lo-1) cells of
@@ -152,13 +153,21 @@ typedef struct {
                       (redundant border work instead of cluster exchanges);
                       actuator controls v3 from patches around the
                       actuators.  0 = auto (stages too large for a cluster of
-                      <= 8 CTAs with staged inputs), 1 = every eligible 2D
+                      <= 8 CTAs with staged inputs; and NMPC_MIXED handles of
+                      eligible smaller 2D stages, n_lo <= 2, at least 24
+                      columns, no cluster / threads / cells / persistent
+                      asked for, of which a launch holds more than stay
+                      resident or which have more than 2048 cells: these keep
+                      the cluster path's residual and iterates bit for bit),
+                      1 = every eligible 2D
                       instance, 2 = never.  Eligible: n_lo <= 4, and for
                       n_u_it > 1 no two actuators on one cell or within
                       2 (n_lo - 1) cells (Manhattan) of each other          */
-  int strip_rows;   /* own rows per strip (0..65535); 0 = auto (whole columns
-                      when the batch gives enough strips, else shorter
-                      strips, at least 16 rows)                             */
+  int strip_rows;   /* own rows per strip (0..65535); 0 = auto (two columns
+                      per lane: the rows that minimise waves of resident
+                      warps x row steps, at least 16, smaller stages 4;
+                      one column per lane: whole columns when the batch
+                      gives enough strips, else at least 16 rows)           */
   int lines;        /* NMPC_MIXED 1D instances of at most 256 cells on the
                       line path: one warp per stage, the stage's cells in
                       registers (8 per lane at most), every pass of the
@@ -192,7 +201,8 @@ typedef struct {
                       where NMPC_MIXED, n_lo <= 2 and every strip instance
                       has an even grid width and even array offsets: 64-column
                       regions with 64 - 4 n_lo own columns, packed float32
-                      pairs; else one), 1 = one (32-column regions)         */
+                      pairs; also at odd widths for the smaller stages of
+                      strips = 0; else one), 1 = one (32-column regions)    */
   int tail_rows;    /* two-column strip path, solves: own rows of a second,
                       finer strip plan taken by the launches of a batch's
                       tail, when at most tail_below instances still run
@@ -263,7 +273,8 @@ int nmpc_solve_host(nmpc_handle* h, const double* x0, const double* ref, int hor
    [n_instances][2] = (||K_b||_inf, ||K_b||_2).  Synchronizes on stream.
    When the handle runs its strip path with two columns per lane
    (nmpc_opts.strip_cols), x and lam must be 16-byte aligned (BAD_ARG
-   otherwise); the same holds for nmpc_iterate's x and lam arrays. */
+   otherwise); the same holds for nmpc_iterate's x and lam arrays.  Stages
+   that fit a cluster are taken at any alignment. */
 int nmpc_residual(nmpc_handle* h, const double* x0, const double* ref, const double* x,
                   const double* u, const double* lam, double* out, void* stream);
 

@@ -84,7 +84,7 @@ void nmpc_plate_default_opts(nmpc_plate_opts* o);
 
 /* Validate the descriptors (BAD_ARG: dims, bounds, tau > 0 with u_lo >= u_hi,
    actuator indices out of the grid or repeated; UNSUPPORTED: more than
-   NMPC_PLATE_MAX_POINTS points or NMPC_MAX_NU inputs), build the stencil
+   NMPC_PLATE_MAX_POINTS points or NMPC_MAX_NU inputs), build the index
    tables and allocate the workspace on the current device.  Synchronous. */
 int nmpc_plate_setup(const nmpc_plate_desc* descs, int n_instances, const nmpc_plate_opts* opts,
                      nmpc_plate** out);

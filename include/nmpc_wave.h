@@ -82,7 +82,7 @@ void nmpc_wave_default_opts(nmpc_wave_opts* o);
 
 /* Validate the descriptors (BAD_ARG: dims, a <= 0, negative weights, r <= 0,
    actuator indices out of the grid or repeated; UNSUPPORTED: more than
-   NMPC_WAVE_MAX_POINTS points or NMPC_MAX_NU inputs), build the stencil
+   NMPC_WAVE_MAX_POINTS points or NMPC_MAX_NU inputs), build the index
    tables and allocate the workspace on the current device.  Synchronous. */
 int nmpc_wave_setup(const nmpc_wave_desc* descs, int n_instances, const nmpc_wave_opts* opts,
                     nmpc_wave** out);

@@ -1,10 +1,11 @@
 """Build the sm_103a shared library ``_lib/libnmpc_gb300.so`` with nvcc.
 
 Six translation units (the solver's C ABI with its kernels, the whole-instance
-solves of 1D problems, the strips of batches of small 2D stages, the learned warm start's network, the pinned-actuator solver of the paper's plate and
-the second-order-in-time solver), compiled in parallel in-tree and linked
-into one library; the outputs are git-ignored.  ``build()`` rebuilds only when a
-source is newer than the library.
+solves of 1D problems, the strips of batches of small 2D stages, the learned
+warm start's network, the pinned-actuator solver of the paper's plate and the
+second-order-in-time solver), compiled in parallel in-tree and linked into one
+library; the outputs are git-ignored.  ``build()`` rebuilds only when a source
+is newer than the library.
 """
 from __future__ import annotations
 
