@@ -469,8 +469,12 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
   // cell keeps the bits that it would get again (n_lo <= 2: no field serves two
   // sweeps).  Three full applications a cell were most of a float64
   // iteration's arithmetic.
+  // (Float64 lower layer only: the float32 kernel is latency-bound, and the
+  // tests cost it more than the cells: 64x64, N = 50, n_lo = 1, n_u_it = 1,
+  // 2.35 against 2.47 ms a solve.)
+  constexpr bool NEAR = sizeof(T) == 8;
   unsigned near1 = 0xffffffffu, near2 = 0xffffffffu;
-  if (!MULTI && A.act_dist != nullptr && n_full > 1 && n_lo <= 2) {
+  if (NEAR && !MULTI && A.act_dist != nullptr && n_full > 1 && n_lo <= 2) {
     near1 = near2 = 0u;
 #pragma unroll
     for (int k2 = 0; k2 < NC; ++k2) {
@@ -514,19 +518,19 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
     if (n_lo == 1) {
       pass<NC, NC, MULTI, T>(g, c0,
           [&](const Slot& sl, const Cells<NC>&) {
-            if (it > 0 && !((near1 >> sl.k) & 1u)) return T(0);
+            if (NEAR && it > 0 && !((near1 >> sl.k) & 1u)) return T(0);
             const int pb = wpos(sl.p);
             return (-WV(pb, F_B2) - WV(pb, F_AX) * WV(pb, F_V1)) * WV(pb, F_RG);
           },
           [&](const Slot& sl, const Cells<NC>& cs, T w) {
-            if (it == 0 || ((near1 >> sl.k) & 1u)) put(cs, sl, F_W1, w);
+            if (!NEAR || it == 0 || ((near1 >> sl.k) & 1u)) put(cs, sl, F_W1, w);
           });
     } else {
       cur = F_Y5;
       const bool lastsw = (n_lo == 2);
       pass<NC, NC, MULTI, V2>(g, c0,
           [&](const Slot& sl, const Cells<NC>&) {
-            if (it > 0 && !((near1 >> sl.k) & 1u)) return V2{T(0), T(0)};
+            if (NEAR && it > 0 && !((near1 >> sl.k) & 1u)) return V2{T(0), T(0)};
             const int pb = wpos(sl.p);
             const T off = th * (tcx * (WV(pb - RB, F_P1) + WV(pb + RB, F_P1)) +
                                 tcy * (WV(pb - WRB, F_P1) + WV(pb + WRB, F_P1)));
@@ -534,7 +538,7 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
             return V2{v, (-WV(pb, F_B2) - WV(pb, F_AX) * v) * WV(pb, F_RG)};
           },
           [&](const Slot& sl, const Cells<NC>& cs, V2 o) {
-            if (it > 0 && !((near1 >> sl.k) & 1u)) return;
+            if (NEAR && it > 0 && !((near1 >> sl.k) & 1u)) return;
             if (wide) put(cs, sl, F_Y5, o.v);
             else if (sl.v) WV(wpos(sl.p), F_Y5) = o.v;
             if (lastsw) put(cs, sl, F_W1, o.w);
@@ -568,7 +572,7 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
       cur = F_Y4;
       pass<NC, NC, MULTI, T>(g, c0,
           [&](const Slot& sl, const Cells<NC>&) {
-            if (it > 0 && !((near2 >> sl.k) & 1u)) return T(0);
+            if (NEAR && it > 0 && !((near2 >> sl.k) & 1u)) return T(0);
             const int pb = wpos(sl.p);
             const T off = th * WV(pb, F_DP) *
                           (tcx * (WV(pb - RB, F_W1) + WV(pb + RB, F_W1)) +
@@ -576,7 +580,7 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
             return WV(pb, F_W1) - WV(pb, F_RG) * off;
           },
           [&](const Slot& sl, const Cells<NC>& cs, T v) {
-            if (it > 0 && !((near2 >> sl.k) & 1u)) return;
+            if (NEAR && it > 0 && !((near2 >> sl.k) & 1u)) return;
             if (wide) put(cs, sl, F_Y4, v);
             else if (sl.v) WV(wpos(sl.p), F_Y4) = v;
           });
