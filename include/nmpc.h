@@ -161,8 +161,9 @@ typedef struct {
                       the cluster path's residual and iterates bit for bit),
                       1 = every eligible 2D
                       instance, 2 = never.  Eligible: n_lo <= 4, and for
-                      n_u_it > 1 no two actuators on one cell or within
-                      2 (n_lo - 1) cells (Manhattan) of each other          */
+                      n_u_it > 1 (auto, smaller stages: for any n_u_it) no
+                      two actuators on one cell or within 2 (n_lo - 1) cells
+                      (Manhattan) of each other                             */
   int strip_rows;   /* own rows per strip (0..65535); 0 = auto (two columns
                       per lane: the rows that minimise waves of resident
                       warps x row steps, at least 16, smaller stages 4;

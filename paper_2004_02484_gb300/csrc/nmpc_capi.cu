@@ -841,22 +841,24 @@ cudaError_t configure_kernels(size_t smem) {
                               (int)(smem - fa.sharedSizeBytes));
 }
 
-// Whether instance I may run on the strip path: 2D, n_lo <= 4, and for
-// n_u_it > 1 actuators on distinct cells more than 2 (n_lo - 1) cells apart
-// (Manhattan), so that each actuator's u-iteration sees only its own
-// response.
-bool strip_eligible(const InstDev& I, const int* act, const nmpc_opts& o) {
-  if (I.dim != 2 || o.n_lo > 4) return false;
-  if (o.n_u_it > 1) {
-    const int reach = 2 * (o.n_lo - 1);
-    for (int a = 0; a < I.nu; ++a)
-      for (int b = a + 1; b < I.nu; ++b) {
-        const int dx = std::abs(act[a] % I.mx - act[b] % I.mx);
-        const int dy = std::abs(act[a] / I.mx - act[b] / I.mx);
-        if (dx + dy <= reach) return false;
-      }
-  }
+// Whether instance I's actuators sit on distinct cells more than 2 (n_lo - 1)
+// cells apart (Manhattan), the reach of an actuator's own response.
+bool actuators_apart(const InstDev& I, const int* act, const nmpc_opts& o) {
+  const int reach = 2 * (o.n_lo - 1);
+  for (int a = 0; a < I.nu; ++a)
+    for (int b = a + 1; b < I.nu; ++b) {
+      const int dx = std::abs(act[a] % I.mx - act[b] % I.mx);
+      const int dy = std::abs(act[a] / I.mx - act[b] / I.mx);
+      if (dx + dy <= reach) return false;
+    }
   return true;
+}
+
+// Whether instance I may run on the strip path: 2D, n_lo <= 4, and for
+// n_u_it > 1 actuators out of each other's reach, so that each actuator's
+// u-iteration sees only its own response.
+bool strip_eligible(const InstDev& I, const int* act, const nmpc_opts& o) {
+  return I.dim == 2 && o.n_lo <= 4 && (o.n_u_it <= 1 || actuators_apart(I, act, o));
 }
 
 // Whether instance I runs on the line path: 1D, at most 32 x LINE_MAX_CPL
@@ -1537,13 +1539,17 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   // against 44.1; 96x80, N = 30: 24.0 against 18.7.  Beyond one wave the
   // clusters' waves add up: 64x64 two instances 46.5 against 21.4 us, 16: 265
   // against 56, 128: 2039 against 346; 32x32 16 instances 50 against 28.
+  // Actuators within each other's reach stay on clusters for every n_u_it:
+  // these strips evaluate K_1 around an actuator (half_warp_v3) with that
+  // actuator's heat alone, where k_patch adds all of them.
   bool d64 = false, fw = false;
   if (my_max == 0 && o.strips == 0 && two && !o.cluster && !o.threads && !o.cells && !o.u_local &&
       !o.persistent) {
     fw = d64 = true;
     int stages = 0;
     for (const InstDev& I : h->inst_h) {
-      d64 = d64 && I.mx >= 24 && strip_eligible(I, act_all.data() + I.act_off, o);
+      const int* act = act_all.data() + I.act_off;
+      d64 = d64 && I.mx >= 24 && strip_eligible(I, act, o) && actuators_apart(I, act, o);
       if ((I.mx & 1) || (I.s_off & 1) || (I.g_off & 1)) h->strip_al = false;
       fw = fw && I.mx <= 64;
       stages += h->rb ? (I.N + 1) / 2 : I.N;

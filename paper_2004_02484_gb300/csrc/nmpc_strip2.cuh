@@ -166,7 +166,8 @@ __device__ __forceinline__ void cp_async16_zfill(void* dst_smem, const void* src
 // of Sec. 5.2 (eqs. 22-24) in the full-field form's own order, on the cells
 // within 2 (n_lo - 1) grid steps of the actuator (13 for n_lo = 2), lane q of
 // the half holding cell q.  No other actuator's cell is among them (the host
-// checks), so v3 comes out as the cluster path's, operation by operation.
+// takes these strips only then, whatever n_u_it), so v3 comes out as the
+// cluster path's, operation by operation.
 // (k_patch, before strips of the other form, computes a square of 49 cells,
 // four of five of which its result does not depend on, and a second
 // right-hand side, in a launch of its own.)

@@ -106,3 +106,42 @@ def test_unaligned_iterates_are_accepted(G):
         outs.append(o)
     assert all(torch.equal(a, b) for a, b in zip(*outs))
     s.close()
+
+
+# actuators on one cell, on neighbouring cells, two cells apart
+NEAR_ACTUATORS = {"one_cell": [(20, 15), (20, 15), (40, 33)],
+                  "adjacent": [(20, 15), (21, 15), (40, 33), (40, 34)],
+                  "two_cells": [(20, 15), (21, 16), (40, 33), (42, 33)]}
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n_lo", [1, 2])
+@pytest.mark.parametrize("kind", list(NEAR_ACTUATORS))
+def test_one_u_iteration_with_actuators_in_each_others_reach(G, kind, n_lo, variant):
+    """n_u_it = 1: every actuator's heat counts in the rows that another one's
+    control is computed from.  One iteration as on the cluster path, and solves
+    that converge as its do."""
+    import torch
+    mx, my, n, k = 64, 50, 20, 24
+    insts = _insts(mx, my, n, k, variant)
+    for i in insts:
+        i.act = np.asarray([y * mx + x for x, y in NEAR_ACTUATORS[kind]], dtype=np.int32)
+    gen = torch.Generator().manual_seed(4)
+    x0 = torch.cat([torch.from_numpy(i.x0).repeat(i.horizon) for i in insts])
+    x = (x0 + 0.01 * torch.randn(x0.shape, dtype=torch.float64, generator=gen)).cuda()
+    lam = (1e-4 * torch.randn(x0.shape, dtype=torch.float64, generator=gen)).cuda()
+    u = torch.randn(sum(i.horizon * len(i.act) for i in insts), dtype=torch.float64, generator=gen).cuda()
+    step, iters, status = [], [], []
+    for strips in (0, 2):
+        s = G.Solver(insts, precision=G.NMPC_MIXED, strips=strips, max_iter=1000, tol=1e-6,
+                     variant=variant, n_lo=n_lo, n_u_it=1)
+        out = [torch.empty_like(t) for t in (x, u, lam)]
+        G.nmpc_iterate(s.h, s.x0, s.ref, x, u, lam, *out, 1, s.n)
+        step.append([b - a for a, b in zip((x, u, lam), out)])
+        st = s.solve()[1]
+        iters.append(np.array([e.iters for e in st]))
+        status.append([e.status for e in st])
+        s.close()
+    for a, b in zip(*step):
+        assert float((a - b).abs().max()) <= 2.0 ** -20 * float(b.abs().max())
+    assert status[0] == status[1] and np.abs(iters[0] - iters[1]).max() <= 1
