@@ -405,6 +405,9 @@ __global__ void __launch_bounds__(32 * li_max_warps(CPL), 1)
           }
         }
       }
+      // every lane has read the stage's controls (usum) before their owners
+      // overwrite them
+      __syncwarp();
       // ---- S_i <- S_i - alpha Delta s_i (float64) ----
 #pragma unroll
       for (int t = 0; t < CPL; ++t) {
