@@ -1185,11 +1185,12 @@ int solve_core(nmpc_handle* h, int horizon, const double* weights, int init, dou
       h->iter_launches += runs * chunk;
     }
     if (!by_instance || h->h_active[11] == 0) break;
-    // an instance diverged on its split residual: iterate from S^0 (nothing
-    // of the state before the solve has been overwritten)
+    // instances that diverged on their split residual iterate from S^0: it is
+    // still in buffer 0, and their control words are as start() left them
+    // (k_line_inst writes neither, and counts them as running); the others are
+    // finished and keep their solutions
     by_instance = done = false;
-    rc0 = start();
-    if (rc0 != NMPC_OK) return rc0;
+    CK(cudaMemsetAsync(h->ictl + 11, 0, sizeof(int), st));
   }
   h->has_state = true;
   int rc = NMPC_OK;

@@ -85,7 +85,8 @@ __device__ __forceinline__ void li_nsum(const V (&v)[CPL], V (&out)[CPL], int la
 // first and updates only if the solve goes on, since the returned iterate is
 // the one whose residual passed.  A split residual that diverges is known only
 // after the update, so that instance asks for a solve by iterations (*retry),
-// which returns the iterate before it.
+// which returns the iterate before it; it stores nothing, so S^0 and its control
+// words are there for that (the other instances of the launch are done).
 // What bounds it: the float64 pipe (56% busy on 304 instances of 256 cells:
 // two differences and two updates a cell) and latency (0.45 instructions a
 // cycle a scheduler, 16 warps a SM at 128 registers).  1024 ragged instances

@@ -102,3 +102,34 @@ def test_a_diverging_instance_returns_what_the_iterations_return(G):
         assert np.array_equal(np.isnan(x), np.isnan(y))
         ok = ~np.isnan(y)
         assert np.abs(x[ok] - y[ok]).max() <= 1e-9 * np.abs(y[ok]).max()
+
+
+@pytest.mark.parametrize("init", ["cold", "shift"])
+def test_only_the_diverging_instance_is_iterated(G, init):
+    """One start state with a NaN among 24: that instance alone goes through the
+    iterations (it stops in their first chunk), the others keep the solutions
+    of the whole-instance launches, bit for bit those of a batch without it."""
+    import torch
+    insts = wl.heat1d_ragged_batch(n=24, base_seed=8500)
+    bad, out = 7, []
+    for with_nan in (False, True):
+        s = G.Solver(insts, precision=G.NMPC_MIXED, tol=1e-6, max_iter=2000)
+        if init == "shift":
+            assert s.solve()[0] == G.NMPC_OK
+        if with_nan:
+            s.x0[sum(i.mx for i in insts[:bad]) + 3] = float("nan")
+        before = G.nmpc_launch_plan(s.h)["iteration_launches"]
+        rc, st = s.solve(init=G.NMPC_INIT_COLD if init == "cold" else G.NMPC_INIT_SHIFT)
+        launches = G.nmpc_launch_plan(s.h)["iteration_launches"] - before
+        assert launches == (1 + 16 if with_nan else 1)  # the default check_every
+        assert [e.status for e in st] == [G.NMPC_STATUS_DIVERGED if with_nan and b == bad
+                                          else G.NMPC_STATUS_CONVERGED for b in range(s.n)]
+        x, u, lam = s.state()
+        out.append((torch.split(x, [i.horizon * i.mx for i in insts]),
+                    torch.split(u, [i.horizon * len(i.act) for i in insts]),
+                    torch.split(lam, [i.horizon * i.mx for i in insts]), [e.iters for e in st]))
+        s.close()
+    for b in range(len(insts)):
+        if b != bad:
+            assert all(torch.equal(out[0][q][b], out[1][q][b]) for q in range(3))
+            assert out[0][3][b] == out[1][3][b]
