@@ -173,10 +173,13 @@ __device__ __forceinline__ void cp_async16_zfill(void* dst_smem, const void* src
 // right-hand side, in a launch of its own.)
 // Cell q of the diamond: itself, its four neighbours, the eight at two steps;
 // the neighbours (left, right, above, below) of cells 0 .. 4.
-static __constant__ signed char diamond_x[13] = {0, -1, 1, 0, 0, -2, 2, 0, 0, -1, 1, -1, 1};
-static __constant__ signed char diamond_y[13] = {0, 0, 0, -1, 1, 0, 0, -2, 2, -1, -1, 1, 1};
-static __constant__ signed char diamond_n[5][4] = {
-    {1, 2, 3, 4}, {5, 0, 9, 11}, {0, 6, 10, 12}, {9, 10, 7, 0}, {11, 12, 0, 8}};
+// (Four bits each in immediate words: tables in constant memory were read with
+// a different index in every lane, and a module that has any makes each of its
+// launches bind them, 0.1 to 0.3 us apiece, the other paths' too: a 256-cell
+// line, N = 240, 200 iterations, 2.59 -> 2.63 ms.)
+constexpr unsigned long long DIAMOND_X = 0x3131224022312ull, DIAMOND_Y = 0x3311402231222ull;  // + 2
+constexpr unsigned DIAMOND_L = 0xb9051u, DIAMOND_R = 0xca602u, DIAMOND_U = 0x7a93u,
+                   DIAMOND_D = 0x80cb4u;
 
 template <int n_lo, bool FULL>
 __device__ __forceinline__ float half_warp_v3(const IterArgs& A, const InstDev& I, int s, int a,
@@ -186,7 +189,8 @@ __device__ __forceinline__ float half_warp_v3(const IterArgs& A, const InstDev& 
   const bool last = (s == I.N - 1);
   const int ca = A.act[I.act_off + a], ay = ca / mx, ax = ca - ay * mx;
   const int qc = q < 13 ? q : 0;
-  const int gx = ax + diamond_x[qc], gy = ay + diamond_y[qc];
+  const int gx = ax + (int)((DIAMOND_X >> (4 * qc)) & 15) - 2;
+  const int gy = ay + (int)((DIAMOND_Y >> (4 * qc)) & 15) - 2;
   const bool in = gx >= 0 && gx < mx && gy >= 0 && gy < my;
   const long long so = I.s_off + (long long)s * I.ng;
   const double* Xg = A.xin[rd] + so;
@@ -256,10 +260,10 @@ __device__ __forceinline__ float half_warp_v3(const IterArgs& A, const InstDev& 
   const float b3 = (float)(I.h * (I.r * ua + I.b0 * lm.m));
   auto nsum = [&](float v) {  // over the neighbours, at the cells 0 .. 4
     const int qq = q < 5 ? q : 0;
-    const float l = __shfl_sync(0xffffffffu, v, base + diamond_n[qq][0]);
-    const float r = __shfl_sync(0xffffffffu, v, base + diamond_n[qq][1]);
-    const float u = __shfl_sync(0xffffffffu, v, base + diamond_n[qq][2]);
-    const float d = __shfl_sync(0xffffffffu, v, base + diamond_n[qq][3]);
+    const float l = __shfl_sync(0xffffffffu, v, base + (int)((DIAMOND_L >> (4 * qq)) & 15));
+    const float r = __shfl_sync(0xffffffffu, v, base + (int)((DIAMOND_R >> (4 * qq)) & 15));
+    const float u = __shfl_sync(0xffffffffu, v, base + (int)((DIAMOND_U >> (4 * qq)) & 15));
+    const float d = __shfl_sync(0xffffffffu, v, base + (int)((DIAMOND_D >> (4 * qq)) & 15));
     return __fmaf_rn(tcx, __fadd_rn(l, r), __fmul_rn(tcy, __fadd_rn(u, d)));
   };
   float v1 = __fmul_rn(-K1, rg), v3 = 0.0f;
