@@ -44,7 +44,6 @@ struct nmpc_handle {
   InstDev* inst_d = nullptr;
   int2* work_d = nullptr;
   int* act_d = nullptr;
-  unsigned char* act_dist_d = nullptr;  // cluster path, n_lo <= 2 (IterArgs::act_dist)
   double* x0_d = nullptr;
   double* ref_d = nullptr;
   float* ref_f_d = nullptr;  // ref truncated to float32 (two-column strip path)
@@ -192,7 +191,7 @@ void free_all(nmpc_handle* h) {
   if (!h) return;
   if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
   if (h->loop_exec) cudaGraphExecDestroy(h->loop_exec);
-  void* ptrs[] = {h->inst_d, h->work_d, h->act_d, h->act_dist_d, h->x0_d, h->ref_d, h->ref_f_d, h->uo_d, h->w_d,
+  void* ptrs[] = {h->inst_d, h->work_d, h->act_d, h->x0_d, h->ref_d, h->ref_f_d, h->uo_d, h->w_d,
                   h->xb[0], h->xb[1], h->xb[2], h->ub[0], h->ub[1], h->ub[2],
                   h->lb[0], h->lb[1], h->lb[2], h->ictl, h->res_inf, h->res_err, h->res_sq,
                   h->res_first, h->status, h->iters, h->final_buf, h->fin_inf,
@@ -212,7 +211,6 @@ IterArgs make_args(nmpc_handle* h) {
   A.n_work = h->n_work;
   A.n_inst = h->n_inst;
   A.act = h->act_d;
-  A.act_dist = h->act_dist_d;
   A.x0 = h->x0_d;
   A.ref = h->ref_d;
   A.ref_f = h->ref_f_d;
@@ -1808,23 +1806,25 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   A(dev_alloc(&h->line_inst_d, line_list.size()));
   if (!h->line_inst.empty()) A(line_inst_configure(max_optin));
   A(dev_alloc(&h->v3_d, h->n_strips > 0 ? h->n_u : 0));
-  A(dev_alloc(&h->act_d, act_all.size()));
-  std::vector<unsigned char> act_dist;
-  if (h->n_work > 0 && h->smem_mode && o.n_lo <= 2) {
-    act_dist.assign(h->n_g, 255);
-    for (const InstDev& I : h->inst_h)
+  // float64 cluster kernels, n_lo = 2: the cells' distances to the actuators
+  // (InstDev::dist_off), behind the actuators' cells
+  if (h->n_work > 0 && h->smem_mode && !h->mixed && o.n_lo == 2)
+    for (InstDev& I : h->inst_h) {
+      I.dist_off = (int)act_all.size();
+      act_all.resize(act_all.size() + (I.ng + 3) / 4, -1);
+      unsigned char* dist = reinterpret_cast<unsigned char*>(&act_all[I.dist_off]);
       for (int a = 0; a < I.nu; ++a) {
         const int c = act_all[I.act_off + a], cy = c / I.mx, cx = c % I.mx;
         for (int dy = -2; dy <= 2; ++dy)
           for (int dx = -2; dx <= 2; ++dx) {
             const int d = std::abs(dx) + std::abs(dy), x = cx + dx, y = cy + dy;
             if (d > 2 || x < 0 || x >= I.mx || y < 0 || y >= I.my) continue;
-            unsigned char& v = act_dist[I.g_off + (long long)y * I.mx + x];
+            unsigned char& v = dist[y * I.mx + x];
             v = std::min<unsigned char>(v, (unsigned char)d);
           }
       }
-    A(dev_alloc(&h->act_dist_d, act_dist.size()));
-  }
+    }
+  A(dev_alloc(&h->act_d, act_all.size()));
   A(dev_alloc(&h->x0_d, h->n_g));
   A(dev_alloc(&h->ref_d, h->n_g));
   if (h->strip2) A(dev_alloc(&h->ref_f_d, h->n_g));
@@ -1874,8 +1874,6 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
     if (!line_list.empty())
       A(cudaMemcpy(h->line_inst_d, line_list.data(), line_list.size() * sizeof(int),
                    cudaMemcpyHostToDevice));
-    if (!act_dist.empty())
-      A(cudaMemcpy(h->act_dist_d, act_dist.data(), act_dist.size(), cudaMemcpyHostToDevice));
     A(cudaMemcpy(h->act_d, act_all.data(), act_all.size() * sizeof(int), cudaMemcpyHostToDevice));
     A(cudaMemset(h->ictl, 0, 12 * sizeof(int)));
     A(cudaDeviceSynchronize());

@@ -28,7 +28,9 @@ constexpr int MAX_NU = 64;
 
 struct InstDev {
   int dim, mx, my, ng;
-  int N, nu, act_off, pad;
+  int N, nu, act_off;
+  int dist_off;  // where in act (in ints) a byte per cell says how many grid
+                 // steps the nearest actuator is away, 255 beyond 2; 0: nowhere
   long long s_off;  // offset of stage 1 in packed x / lam
   long long u_off;  // offset in packed u
   long long g_off;  // offset in packed x0 / ref
@@ -66,9 +68,6 @@ struct IterArgs {
   int n_work;
   int n_inst;
   const int* act;
-  // cluster path, n_lo <= 2: per grid cell (packed as x0) the grid steps to the
-  // nearest actuator, 255 beyond 2; null: not used
-  const unsigned char* act_dist;
   const double* x0;
   const double* ref;
   // state buffers: solve mode reads [k & 1] and writes [(k + 1) & 1];

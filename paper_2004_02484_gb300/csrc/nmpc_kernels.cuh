@@ -464,24 +464,27 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
     T v, w;
   };
   // The slots whose cells an application after the first recomputes: F_u v3
-  // changes on the actuator cells only, so v5 and the first F_x^T sweep change
-  // within n_lo - 1 grid steps of one and v4 within 2 (n_lo - 1); every other
-  // cell keeps the bits that it would get again (n_lo <= 2: no field serves two
-  // sweeps).  Three full applications a cell were most of a float64
-  // iteration's arithmetic.
-  // (Float64 lower layer only: the float32 kernel is latency-bound, and the
-  // tests cost it more than the cells: 64x64, N = 50, n_lo = 1, n_u_it = 1,
-  // 2.35 against 2.47 ms a solve.)
+  // changes on the actuator cells only, so with n_lo = 2 v5 and the first F_x^T
+  // sweep change within one grid step of one and v4 within two; every other
+  // cell keeps the bits that it would get again (no field serves two sweeps).
+  // Three full applications a cell were most of a float64 iteration's
+  // arithmetic.
+  // (Float64 lower layer with n_lo = 2 only: the float32 kernel is
+  // latency-bound, and the tests cost it more than the cells, 64x64, N = 50,
+  // n_lo = 1, n_u_it = 1, 2.35 against 2.47 ms a solve; so with n_lo = 1 in
+  // float64, whose applications are one pass each: four 64x64, N = 20, 3.74
+  // against 3.82 ms.)
   constexpr bool NEAR = sizeof(T) == 8;
   unsigned near1 = 0xffffffffu, near2 = 0xffffffffu;
-  if (NEAR && !MULTI && A.act_dist != nullptr && n_full > 1 && n_lo <= 2) {
+  if (NEAR && !MULTI && I.dist_off > 0 && n_full > 1) {
     near1 = near2 = 0u;
+    const unsigned char* dist = reinterpret_cast<const unsigned char*>(A.act + I.dist_off) + g.lo;
 #pragma unroll
     for (int k2 = 0; k2 < NC; ++k2) {
       if (!((c0.valid >> k2) & 1u)) continue;
-      const int d = A.act_dist[I.g_off + g.lo + tid + k2 * bd];
-      near1 |= (d <= n_lo - 1 ? 1u : 0u) << k2;
-      near2 |= (d <= 2 * (n_lo - 1) ? 1u : 0u) << k2;
+      const int d = dist[tid + k2 * bd];
+      near1 |= (d <= 1 ? 1u : 0u) << k2;
+      near2 |= (d <= 2 ? 1u : 0u) << k2;
     }
   }
   for (int it = 0; it < n_full; ++it) {
@@ -518,13 +521,10 @@ __device__ void process_item(const IterArgs& A, int b, int s, int k, int rd, boo
     if (n_lo == 1) {
       pass<NC, NC, MULTI, T>(g, c0,
           [&](const Slot& sl, const Cells<NC>&) {
-            if (NEAR && it > 0 && !((near1 >> sl.k) & 1u)) return T(0);
             const int pb = wpos(sl.p);
             return (-WV(pb, F_B2) - WV(pb, F_AX) * WV(pb, F_V1)) * WV(pb, F_RG);
           },
-          [&](const Slot& sl, const Cells<NC>& cs, T w) {
-            if (!NEAR || it == 0 || ((near1 >> sl.k) & 1u)) put(cs, sl, F_W1, w);
-          });
+          [&](const Slot& sl, const Cells<NC>& cs, T w) { put(cs, sl, F_W1, w); });
     } else {
       cur = F_Y5;
       const bool lastsw = (n_lo == 2);
