@@ -9,6 +9,7 @@
 #include "nmpc_line_inst.h"
 
 #include <algorithm>
+#include <cmath>
 #include <map>
 #include <tuple>
 
@@ -628,6 +629,16 @@ std::vector<LineInstLaunch> line_inst_plan(const std::vector<InstDev>& inst,
     if (!c) return {};
     classes[{cpl, c, few}].push_back(b);
   }
+  // Batch-form CTAs against one launch per iteration (us an iteration): a warp
+  // here takes t_stage for each of its stages, k_line t_wave for 16 stages a
+  // SM.  Few long instances leave SMs without a CTA and their warps with many
+  // stages: N = 66, one instance of 64 cells 28.9 against 10.1, N = 160, twelve
+  // of 32 cells 47 against 10.9; or the last wave of CTAs is nearly empty: 76 of
+  // 256 cells, N = 66, 46.6 against 43 (72: 26.7 against 34).
+  static const double t_stage[9] = {0, 2.3, 3.1, 0, 4.3, 0, 0, 0, 8.0};
+  static const double t_wave[9] = {0, 8.5, 10, 0, 12, 0, 0, 0, 15.5};
+  bool batch = false;
+  double longest = 0, work = 0, stages = 0, by_launches = 0;
   for (auto it = classes.rbegin(); it != classes.rend(); ++it) {
     const int cpl = std::get<0>(it->first), c = std::get<1>(it->first);
     std::vector<int>& v = it->second;
@@ -645,6 +656,25 @@ std::vector<LineInstLaunch> line_inst_plan(const std::vector<InstDev>& inst,
     L.smem = nmpc_dev::li_layout(cpl, rows, L.warps, nu).bytes;
     if (L.smem > (size_t)max_smem) return {};
     plan.push_back(L);
+    const bool few = std::get<2>(it->first);
+    batch = batch || !few;
+    const int sms = num_sms - (c > 2 ? num_sms / 19 : 0);
+    const double t = (rows + L.warps - 1) / L.warps * t_stage[cpl];
+    double waves = (double)L.n * c / (few ? sms : 2 * sms);
+    if (classes.size() == 1) waves = std::ceil(waves);
+    longest = std::max(longest, t);
+    work += waves * t;
+    for (int b : v) {
+      stages += inst[b].N;
+      by_launches += inst[b].N * t_wave[cpl];
+    }
+  }
+  if (batch) {
+    by_launches *= std::ceil(stages / (16.0 * num_sms)) / stages;
+    if (std::max(longest, work) > by_launches) {
+      list->clear();
+      return {};
+    }
   }
   return plan;
 }

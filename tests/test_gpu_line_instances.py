@@ -133,3 +133,27 @@ def test_only_the_diverging_instance_is_iterated(G, init):
         if b != bad:
             assert all(torch.equal(out[0][q][b], out[1][q][b]) for q in range(3))
             assert out[0][3][b] == out[1][3][b]
+
+
+# (cells, N, instances, whole-instance launches): every cells-per-lane form as
+# clusters of eight, four and two CTAs or one, with as many warps as stages or
+# batch form; long horizons and batches whose CTAs would leave SMs idle stay on
+# launches by iteration
+ROUTES = [(32, 60, 1, True), (64, 64, 1, True), (128, 33, 4, True), (256, 60, 4, True), (256, 60, 20, True),
+          (128, 40, 36, True), (32, 110, 44, True), (256, 60, 44, True), (64, 20, 100, True),
+          (128, 110, 28, True), (256, 60, 100, True), (32, 66, 1, False), (64, 80, 4, False),
+          (128, 110, 12, False), (32, 160, 20, False), (256, 160, 4, False), (256, 40, 44, False),
+          (256, 66, 76, False)]
+
+
+@pytest.mark.parametrize("m,n,k,whole", ROUTES)
+def test_route(G, m, n, k, whole):
+    insts = [wl.heat1d(m, n, 2, 0.01, seed=40 + b) for b in range(k)]
+    kw = dict(tol=1e-5, max_iter=2000)
+    s = G.Solver(insts, precision=G.NMPC_MIXED, **kw)
+    before = G.nmpc_launch_plan(s.h)["iteration_launches"]
+    assert s.solve()[0] == G.NMPC_OK
+    launches = G.nmpc_launch_plan(s.h)["iteration_launches"] - before
+    s.close()
+    assert (launches == 1) == whole
+    _same(_solve(G, insts, 1, **kw), _solve(G, insts, 0, **kw))
