@@ -156,9 +156,10 @@ typedef struct {
                       <= 8 CTAs with staged inputs; and NMPC_MIXED handles of
                       eligible smaller 2D stages, n_lo <= 2, at least 24
                       columns, no cluster / threads / cells / persistent
-                      asked for, of which a launch holds more than stay
-                      resident or which have more than 2048 cells: these keep
-                      the cluster path's residual and iterates bit for bit),
+                      asked for, of which a launch holds several times what
+                      stays resident, or which have more than 2048 cells and
+                      are few: these keep the cluster path's residual and
+                      iterates bit for bit),
                       1 = every eligible 2D
                       instance, 2 = never.  Eligible: n_lo <= 4, and for
                       n_u_it > 1 (auto, smaller stages: for any n_u_it) no

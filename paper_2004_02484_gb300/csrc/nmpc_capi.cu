@@ -1530,14 +1530,26 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
     }
   }
   // Smaller stages (no instance needs strips by its size, no cluster shape
-  // asked for): strips where a launch holds more stages than the device keeps
-  // clusters resident, or the stages have more than 2048 cells.  Otherwise an
-  // iteration is one wave of clusters, which is as fast (32x32, N = 20, eight
-  // instances: 20.6 against 21.6 us, red-black 41.6 against 47.3).  Larger
-  // stages: 64x64, N = 50, one instance 24.8 against 20.9 us, red-black 50.6
-  // against 44.1; 96x80, N = 30: 24.0 against 18.7.  Beyond one wave the
-  // clusters' waves add up: 64x64 two instances 46.5 against 21.4 us, 16: 265
-  // against 56, 128: 2039 against 346; 32x32 16 instances 50 against 28.
+  // asked for): strips where the clusters' waves add up, us an iteration: 64x64,
+  // N = 50, two instances 46.5 on clusters against 21.4, 16: 265 against 56, 128:
+  // 2039 against 346; 32x32, N = 20, 16 instances: 45 against 30.
+  // The waves that it takes: two where a SM holds one cluster's CTA or the grids
+  // fill the strips' 64 columns; more where several stages share a SM (24x24,
+  // three a SM, N = 20: 64 instances, three waves, 43 against 54; 128, six
+  // waves, 78 against 77; 30x30, two a SM, from the third wave on), in red-black
+  // order with n_lo = 2, whose second half reads two fields more (24x30, N = 20,
+  // four waves 0.8 of the clusters' speed, seven 0.96, twelve 1.2; 33x50, odd,
+  // five waves 0.98), and with n_u_it = 1, which saves clusters a third of
+  // their passes.  Horizons below ten are not asked for more than two waves
+  // (their solves are 16 to 25 iterations; 25x18, N = 9, 100 instances 0.91 of
+  // the clusters' speed, red-black 0.63).
+  // In one wave an iteration of these strips is shorter than of clusters for
+  // stages of more than 2048 cells (64x64, N = 50, one instance: 24.8 against
+  // 19.3; not with n_lo = 2 and n_u_it = 1: 48x48, N = 20, red-black 38.5 against
+  // 39.2), but one with a float64 residual is longer, and the instances of a
+  // batch take theirs at different iterations: one instance, or stages enough
+  // that a solve has many iterations (four 96x80, N = 3: 344 against 406 us a
+  // solve; two 64x64, N = 20: 1085 against 1019).
   // Actuators within each other's reach stay on clusters for every n_u_it:
   // these strips evaluate K_1 around an actuator (half_warp_v3) with that
   // actuator's heat alone, where k_patch adds all of them.
@@ -1545,21 +1557,41 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   if (my_max == 0 && o.strips == 0 && two && !o.cluster && !o.threads && !o.cells && !o.u_local &&
       !o.persistent) {
     fw = d64 = true;
-    int stages = 0;
+    int stages = 0, ng_max = 0, least_n = h->inst_h[0].N;
     for (const InstDev& I : h->inst_h) {
       const int* act = act_all.data() + I.act_off;
       d64 = d64 && I.mx >= 24 && strip_eligible(I, act, o) && actuators_apart(I, act, o);
       if ((I.mx & 1) || (I.s_off & 1) || (I.g_off & 1)) h->strip_al = false;
       fw = fw && I.mx <= 64;
       stages += h->rb ? (I.N + 1) / 2 : I.N;
+      ng_max = std::max(ng_max, I.ng);
+      least_n = std::min(least_n, I.N);
     }
-    int ng_max = 0;
-    for (const InstDev& I : h->inst_h) ng_max = std::max(ng_max, I.ng);
-    if (d64 && ng_max <= 2048) {
+    if (d64) {
+      const int own = fw ? 64 : 64 - 2 * nmpc_dev::strip2_pad(o.n_lo);
+      double fill = 1.0;  // of the strips' columns, the least
+      for (const InstDev& I : h->inst_h)
+        fill = std::min(fill, (double)I.mx / ((I.mx + own - 1) / own * own));
       const LaunchPlan P0 = plan_launch(h->inst_h.data(), n_instances, stages, o, h->mixed,
                                         std::max(1, h->num_sms), max_optin);
-      d64 = !P0.smem_mode ||
-            stages > clusters_resident(P0.csize, P0.threads, P0.cpt, P0.smem, h->mixed);
+      const int room =
+          std::max(1, clusters_resident(P0.csize, P0.threads, P0.cpt, P0.smem, h->mixed));
+      const int waves = (stages + room - 1) / room;
+      const int per_sm = P0.csize > 1 ? 1 : room / std::max(1, h->num_sms);
+      const bool rb2 = h->rb && o.n_lo == 2, one_pass = o.n_lo == 2 && o.n_u_it == 1;
+      int need = 2;
+      if (least_n >= 10) {
+        if (rb2)
+          need = per_sm > 2 ? 12 : (per_sm == 2 ? 8 : (fill < 0.5 || !h->strip_al ? 6 : 3));
+        else if (fill < 0.75)
+          need = per_sm > 2 ? 6 : (per_sm == 2 ? 3 : 2);
+        if (one_pass && need > 2) need *= 2;
+      }
+      if (P0.smem_mode && waves == 1)
+        d64 = ng_max > 2048 && fill >= 0.5 && !one_pass &&
+              (n_instances == 1 ? least_n >= (h->rb ? 5 : 2) : least_n >= 20 && !rb2);
+      else if (P0.smem_mode)
+        d64 = waves >= need;
     }
     fw = fw && d64;
     if (d64) {

@@ -145,3 +145,16 @@ def test_one_u_iteration_with_actuators_in_each_others_reach(G, kind, n_lo, vari
     for a, b in zip(*step):
         assert float((a - b).abs().max()) <= 2.0 ** -20 * float(b.abs().max())
     assert status[0] == status[1] and np.abs(iters[0] - iters[1]).max() <= 1
+
+
+@pytest.mark.parametrize("mx,my,n,k,opts,strips", [
+    (64, 64, 50, 1, {}, True), (64, 64, 20, 2, {}, True), (96, 80, 5, 1, dict(variant=1), True),
+    (32, 32, 20, 16, {}, True), (24, 24, 20, 192, {}, True), (64, 8, 20, 50, {}, True),
+    (64, 64, 1, 1, {}, False), (96, 80, 3, 4, {}, False), (48, 48, 20, 4, dict(variant=1), False),
+    (48, 48, 20, 4, dict(n_u_it=1), False), (64, 64, 10, 1, dict(variant=1, n_u_it=1), False),
+    (24, 24, 20, 64, {}, False), (24, 30, 20, 90, dict(variant=1), False),
+    (32, 32, 20, 24, dict(variant=1), False)])
+def test_stages_that_clusters_take_faster_stay_there(G, mx, my, n, k, opts, strips):
+    s = G.Solver([wl.heat2d(mx, my, n, 2, 2, seed=b) for b in range(k)], precision=G.NMPC_MIXED, **opts)
+    assert G.nmpc_strip_plan(s.h)["instances"] == (k if strips else 0)
+    s.close()
