@@ -77,7 +77,8 @@ struct Iter {
 };
 
 // The work items that one launch shape covers: the stages of the instances of
-// one grid kind (dimension, boundary condition), even stages first.  A stage
+// one grid kind (dimension, boundary condition; see driver_alloc), even stages
+// first.  A stage
 // is a group of tps threads (a multiple of 32) with ppt points each, spc
 // groups to a CTA: a 64-point string on a 256-thread CTA of its own left six
 // of eight warps idle, four of them share one now.  More than 256 points take
@@ -398,16 +399,16 @@ struct GridKind {
 };
 
 // The thread groups' shape for stages of ng points, n of them in all.
-inline void shape_group(Group& g) {
+inline void shape_group(Group& g, int sms) {
   g.ppt = g.ng_max > 256 ? 2 : 1;
   g.tps = 32 * ((g.ng_max + 32 * g.ppt - 1) / (32 * g.ppt));
   // at most 256 threads a CTA (8 named barriers); two CTAs' worth of stages
-  // for each of the 152 SMs before stages share a CTA
-  g.spc = std::max(1, std::min(256 / g.tps, g.n / 304));
+  // for each SM before stages share a CTA
+  g.spc = std::max(1, std::min(256 / g.tps, g.n / (2 * sms)));
 }
 
-// Offsets from lay_h[b].{N, nx, nu}; the work items (instance, stage) by grid
-// kind, even stages first.
+// Offsets from lay_h[b].{N, nx, nu}; the work items (instance, stage) by
+// group, even stages first.
 inline cudaError_t driver_alloc(Driver& d, const std::vector<GridKind>& grid, bool directions) {
   d.n = (int)d.lay_h.size();
   d.n_g = d.n_x = d.n_u = 0;
@@ -421,23 +422,42 @@ inline cudaError_t driver_alloc(Driver& d, const std::vector<GridKind>& grid, bo
     d.n_u += (long long)L.N * L.nu;
     d.n_g += L.nx;
   }
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  sms = std::max(1, sms);
+  // One group per grid kind; where a kind has stages of up to 256 points beside
+  // larger ones and more of both than run at once with the larger ones' threads
+  // (two CTAs a SM), the smaller ones are a group of their own: a launch more
+  // per iteration, but they need not have two points a thread and 288 to 512
+  // threads a stage (one 24x24 plate and 511 of 5x5, N = 20, float64: 118 ms a
+  // solve in one group, 49 in two).
   for (int kind = 0; kind < 4; ++kind) {
-    Group g{};
-    g.neu = kind & 1;
-    g.d2 = kind & 2;
-    g.first = (int)work.size();
-    for (int par = 0; par < 2; ++par) {
-      for (int b = 0; b < d.n; ++b) {
-        if (grid[b].neu != g.neu || (grid[b].dim == 2) != g.d2) continue;
-        g.ng_max = std::max(g.ng_max, grid[b].ng);
-        for (int s = par; s < d.lay_h[b].N; s += 2) work.push_back(make_int2(b, s));
+    long long n[2] = {0, 0};  // stages of up to 256 points, of more
+    auto of_kind = [&](int b) {
+      return grid[b].neu == ((kind & 1) != 0) && (grid[b].dim == 2) == ((kind & 2) != 0);
+    };
+    for (int b = 0; b < d.n; ++b)
+      if (of_kind(b)) n[grid[b].ng > 256] += d.lay_h[b].N;
+    const bool split = n[0] > 0 && n[1] > 0 && n[0] + n[1] > 2 * sms;
+    for (int large = 0; large < (split ? 2 : 1); ++large) {
+      Group g{};
+      g.neu = kind & 1;
+      g.d2 = kind & 2;
+      g.first = (int)work.size();
+      for (int par = 0; par < 2; ++par) {
+        for (int b = 0; b < d.n; ++b) {
+          if (!of_kind(b) || (split && (grid[b].ng > 256) != (large == 1))) continue;
+          g.ng_max = std::max(g.ng_max, grid[b].ng);
+          for (int s = par; s < d.lay_h[b].N; s += 2) work.push_back(make_int2(b, s));
+        }
+        if (par == 0) g.n_even = (int)work.size() - g.first;
       }
-      if (par == 0) g.n_even = (int)work.size() - g.first;
+      g.n = (int)work.size() - g.first;
+      if (g.n == 0) continue;
+      shape_group(g, sms);
+      d.groups.push_back(g);
     }
-    g.n = (int)work.size() - g.first;
-    if (g.n == 0) continue;
-    shape_group(g);
-    d.groups.push_back(g);
   }
   d.n_work = (int)work.size();
   cudaError_t e = cudaSuccess;

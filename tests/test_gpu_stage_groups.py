@@ -91,3 +91,34 @@ def test_plate_iteration(case, variant, name, n_lo, n_u_it):
     _check(GP.PlateSolver(insts, variant=variant, n_lo=n_lo, n_u_it=n_u_it), probs, states,
            lambda p, X, U, L: P.iteration(p, X, U, L, name, n_lo, n_u_it)[:3],
            {0, len(insts) // 2, len(insts) - 1})
+
+
+# one stage kind with grids of both thread shapes, more of them than run at once
+MIXED_WAVES = lambda: ([wl.wave_instance(dim=2, m=5, horizon=5, T=0.015, seed=b) for b in range(70)] +
+                       [wl.wave_instance(dim=2, m=17, horizon=3, T=0.009)])
+MIXED_PLATES = lambda: wl.plate_batch(45, m=5, horizon=7, act_idx=(1, 3)) + [wl.plate_instance(m=17, horizon=3, T=15.0)]
+
+
+@pytest.mark.parametrize("variant,name", [(0, "jacobi"), (1, "redblack")])
+def test_grids_of_both_thread_shapes(variant, name):
+    from paper_2004_02484_gb300 import plate as GP
+    from paper_2004_02484_gb300 import wave as GW
+    rng = np.random.default_rng(7)
+    insts = MIXED_WAVES()
+    probs = [Wv.WaveProblem(i) for i in insts]
+    states = []
+    for p in probs:
+        X, U, L = p.cold_start()
+        states.append((X + 0.05 * rng.standard_normal(X.shape), U + 0.5 * rng.standard_normal(U.shape),
+                       L + 0.01 * rng.standard_normal(L.shape)))
+    _check(GW.WaveSolver(insts, variant=variant), probs, states,
+           lambda p, X, U, L: Wv.iteration(p, X, U, L, name, 2, 2)[:3], {0, 40, 69, 70})
+    insts = MIXED_PLATES()
+    probs = [P.PinnedProblem(i) for i in insts]
+    states = []
+    for p in probs:
+        X, U, L = p.cold_start()
+        states.append((X + 15.0 * rng.standard_normal(X.shape), rng.uniform(p.u_lo + 20, p.u_hi - 20, U.shape),
+                       L + 1e-3 * rng.standard_normal(L.shape)))
+    _check(GP.PlateSolver(insts, variant=variant), probs, states,
+           lambda p, X, U, L: P.iteration(p, X, U, L, name, 2, 2)[:3], {0, 22, 44, 45})
