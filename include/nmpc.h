@@ -211,7 +211,9 @@ typedef struct {
                       (more warps per instance: a few running instances'
                       strips no longer leave the GPU latency-bound).  0 =
                       auto (64 where the main plan's rows are >= 256, else
-                      none), -1 = none, else 8..65535                      */
+                      none; by itself the plan takes such rows only where
+                      the batch has six waves of them), -1 = none, else
+                      8..65535                                             */
   int tail_below;   /* running instances at or below which a launch takes the
                       tail plan: 0 = auto (those whose main-plan strips fill
                       fewer than six waves of resident warps), else >= 1   */

@@ -154,6 +154,7 @@ namespace {
 // Lower limit of the residual level at which handles with strip-path
 // instances switch to the float64 residual (see make_args).
 constexpr double STRIP_SPLIT_FLOOR = 1e-6;
+constexpr int TAIL_ROWS = 64;  // of the automatic tail plan (nmpc_opts::tail_rows)
 
 template <typename T>
 size_t small_shared_bytes() {
@@ -1616,7 +1617,11 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       // (12 a SM), so a launch takes its waves times the rows of a strip's
       // region and pipeline: the split of the columns with the fewest (three
       // 156x110, N = 96, red-black: 28 rows and one wave a half, 112 us an
-      // iteration, where 16 rows, two waves, took 141)
+      // iteration, where 16 rows, two waves, took 141).  Where k_patch has
+      // computed the controls, four more for a strip's start (twelve 256x256, N =
+      // 100: 128 rows, seven waves, 943 us, 86 rows, ten waves, 981); with the
+      // controls computed inside, short strips are worth more than that (96 of
+      // 32x32, N = 20, red-black: 6.2 ms a solve without the four, 8.0 with).
       const long long room = 4LL * STRIP2_MIN_BLOCKS * std::max(1, h->num_sms);
       long long best = 0;
       const int least = d64 ? 4 : 16;
@@ -1629,8 +1634,14 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
           warps += (long long)(h->rb ? (I.N + 1) / 2 : I.N) * ((I.mx + tx - 1) / tx) *
                    ((I.my + rows - 1) / rows);
         }
-        const long long cost = ((warps + room - 1) / room) * (rows + 3 * E);
-        if (segs == 1 || cost < best) {
+        const long long cost = ((warps + room - 1) / room) * (rows + 3 * E + (d64 ? 0 : 4));
+        // (rows that come with a tail plan, below, need the six waves above
+        // which that is not taken from the first iteration on: 30 instances of
+        // 256x256, N = 60: 209 ms on whole columns, all of it tail plan, 197 on
+        // half columns)
+        if (!d64 && !o.tail_rows && !o.tail_below && rows >= 4 * TAIL_ROWS && warps <= 6 * room)
+          continue;
+        if (best == 0 || cost < best) {
           best = cost;
           ty = rows;
         }
@@ -1645,7 +1656,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   // where the main plan's are at least four times taller
   int ty_tail = 0;
   if (my_max > 0 && two && !d64 && o.tail_rows >= 0) {
-    const int want = o.tail_rows > 0 ? o.tail_rows : 64;
+    const int want = o.tail_rows > 0 ? o.tail_rows : TAIL_ROWS;
     if (o.tail_rows > 0 ? want < ty : ty >= 4 * want) ty_tail = want;
   }
   std::vector<int2> work;

@@ -383,3 +383,14 @@ def test_tail_plan_solve_is_bit_identical_to_the_main_plan(G, variant):
     s = G.Solver(big, precision=G.NMPC_MIXED, strips=1, strip_rows=128)
     assert G.nmpc_strip_plan(s.h)["tail_rows"] == 0
     s.close()
+
+
+@pytest.mark.parametrize("n,horizon,opts,rows,tail", [
+    (30, 60, {}, 128, 0), (30, 60, dict(variant=1), 128, 0), (24, 100, {}, 256, 64),
+    (30, 60, dict(tail_rows=64), 256, 64), (30, 60, dict(tail_rows=-1), 256, 0),
+    (30, 60, dict(strip_rows=256), 256, 64)])
+def test_no_rows_whose_tail_plan_would_run_the_whole_batch(G, n, horizon, opts, rows, tail):
+    s = G.Solver(wl.heat2d_large_batch(n=n, horizon=horizon), precision=G.NMPC_MIXED, **opts)
+    plan = G.nmpc_strip_plan(s.h)
+    s.close()
+    assert plan["strip_y"] == rows and plan["tail_rows"] == tail
