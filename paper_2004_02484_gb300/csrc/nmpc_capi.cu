@@ -1540,7 +1540,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   // waves, 78 against 77; 30x30, two a SM, from the third wave on), in red-black
   // order with n_lo = 2, whose second half reads two fields more (24x30, N = 20,
   // four waves 0.8 of the clusters' speed, seven 0.96, twelve 1.2; 33x50, odd,
-  // five waves 0.98), and with n_u_it = 1, which saves clusters a third of
+  // five waves 0.98; 130x100, two waves, 1.9), and with n_u_it = 1, which saves clusters a third of
   // their passes.  Horizons below ten are not asked for more than two waves
   // (their solves are 16 to 25 iterations; 25x18, N = 9, 100 instances 0.91 of
   // the clusters' speed, red-black 0.63).
@@ -1558,7 +1558,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   if (my_max == 0 && o.strips == 0 && two && !o.cluster && !o.threads && !o.cells && !o.u_local &&
       !o.persistent) {
     fw = d64 = true;
-    int stages = 0, ng_max = 0, least_n = h->inst_h[0].N;
+    int stages = 0, ng_max = 0, least_g = h->inst_h[0].ng, least_n = h->inst_h[0].N;
     for (const InstDev& I : h->inst_h) {
       const int* act = act_all.data() + I.act_off;
       d64 = d64 && I.mx >= 24 && strip_eligible(I, act, o) && actuators_apart(I, act, o);
@@ -1566,6 +1566,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       fw = fw && I.mx <= 64;
       stages += h->rb ? (I.N + 1) / 2 : I.N;
       ng_max = std::max(ng_max, I.ng);
+      least_g = std::min(least_g, I.ng);
       least_n = std::min(least_n, I.N);
     }
     if (d64) {
@@ -1583,14 +1584,19 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       int need = 2;
       if (least_n >= 10) {
         if (rb2)
-          need = per_sm > 2 ? 12 : (per_sm == 2 ? 8 : (fill < 0.5 || !h->strip_al ? 6 : 3));
+          need = per_sm > 2    ? 12
+                 : per_sm == 2 ? 8
+                 : least_g >= 4096 ? 2
+                 : fill < 0.5 || !h->strip_al ? 6 : 3;
         else if (fill < 0.75)
           need = per_sm > 2 ? 6 : (per_sm == 2 ? 3 : 2);
         if (one_pass && need > 2) need *= 2;
       }
       if (P0.smem_mode && waves == 1)
-        d64 = ng_max > 2048 && fill >= 0.5 && !one_pass &&
-              (n_instances == 1 ? least_n >= (h->rb ? 5 : 2) : least_n >= 20 && !rb2);
+        d64 = ng_max > 2048 && (fill >= 0.5 || h->strip_al) && !one_pass &&
+              (n_instances == 1 ? least_n >= (h->rb ? 5 : 2)
+                                : least_n >= 20 && (!rb2 || (o.n_u_it > 3 && fill >= 0.75 &&
+                                                             h->strip_al)));
       else if (P0.smem_mode)
         d64 = waves >= need;
     }

@@ -150,6 +150,8 @@ def test_one_u_iteration_with_actuators_in_each_others_reach(G, kind, n_lo, vari
 @pytest.mark.parametrize("mx,my,n,k,opts,strips", [
     (64, 64, 50, 1, {}, True), (64, 64, 20, 2, {}, True), (96, 80, 5, 1, dict(variant=1), True),
     (32, 32, 20, 16, {}, True), (24, 24, 20, 192, {}, True), (64, 8, 20, 50, {}, True),
+    (130, 100, 20, 2, dict(variant=1), True), (24, 90, 10, 1, {}, True),
+    (64, 64, 20, 2, dict(variant=1, n_u_it=5), True),
     (64, 64, 1, 1, {}, False), (96, 80, 3, 4, {}, False), (48, 48, 20, 4, dict(variant=1), False),
     (48, 48, 20, 4, dict(n_u_it=1), False), (64, 64, 10, 1, dict(variant=1, n_u_it=1), False),
     (24, 24, 20, 64, {}, False), (24, 30, 20, 90, dict(variant=1), False),
