@@ -160,3 +160,24 @@ def test_stages_that_clusters_take_faster_stay_there(G, mx, my, n, k, opts, stri
     s = G.Solver([wl.heat2d(mx, my, n, 2, 2, seed=b) for b in range(k)], precision=G.NMPC_MIXED, **opts)
     assert G.nmpc_strip_plan(s.h)["instances"] == (k if strips else 0)
     s.close()
+
+
+@pytest.mark.parametrize("size", SIZES + [(64, 64, 50, 1), (90, 70, 20, 1)])
+@pytest.mark.parametrize("n_lo", [1, 2])
+def test_residual_equals_the_cluster_path(G, size, n_lo):
+    """The float64 norms of one state: the same sums in another order (a few
+    hundred thousand terms: 1e-12 relative)."""
+    import torch
+    insts = _insts(*size)
+    gen = torch.Generator().manual_seed(9)
+    out = []
+    for strips in (0, 2):
+        s = _solver(G, insts, strips, n_lo=n_lo)
+        if not out:
+            x0 = torch.cat([torch.from_numpy(i.x0).repeat(i.horizon) for i in insts])
+            x = (x0 + 0.01 * torch.randn(x0.shape, dtype=torch.float64, generator=gen)).cuda()
+            lam = (1e-4 * torch.randn(x0.shape, dtype=torch.float64, generator=gen)).cuda()
+            u = torch.randn(s.n_u, dtype=torch.float64, generator=gen).cuda()
+        out.append(G.nmpc_residual(s.h, s.x0, s.ref, x, u, lam, s.n))
+        s.close()
+    assert np.abs(out[0] / out[1] - 1).max() <= 1e-12
