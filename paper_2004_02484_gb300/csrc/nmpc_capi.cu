@@ -1548,9 +1548,10 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
   // stages of more than 2048 cells (64x64, N = 50, one instance: 24.8 against
   // 19.3; not with n_lo = 2 and n_u_it = 1: 48x48, N = 20, red-black 38.5 against
   // 39.2), but one with a float64 residual is longer, and the instances of a
-  // batch take theirs at different iterations: one instance, or stages enough
+  // batch take theirs at different iterations: one instance, stages enough
   // that a solve has many iterations (four 96x80, N = 3: 344 against 406 us a
-  // solve; two 64x64, N = 20: 1085 against 1019).
+  // solve; two 64x64, N = 20: 1085 against 1019), or larger stages (two 130x100,
+  // N = 3: 428 against 380).
   // Actuators within each other's reach stay on clusters for every n_u_it:
   // these strips evaluate K_1 around an actuator (half_warp_v3) with that
   // actuator's heat alone, where k_patch adds all of them.
@@ -1586,7 +1587,7 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
         if (rb2)
           need = per_sm > 2    ? 12
                  : per_sm == 2 ? 8
-                 : least_g >= 4096 ? 2
+                 : least_g >= 3000 ? 2
                  : fill < 0.5 || !h->strip_al ? 6 : 3;
         else if (fill < 0.75)
           need = per_sm > 2 ? 6 : (per_sm == 2 ? 3 : 2);
@@ -1594,9 +1595,10 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       }
       if (P0.smem_mode && waves == 1)
         d64 = ng_max > 2048 && (fill >= 0.5 || h->strip_al) && !one_pass &&
-              (n_instances == 1 ? least_n >= (h->rb ? 5 : 2)
-                                : least_n >= 20 && (!rb2 || (o.n_u_it > 3 && fill >= 0.75 &&
-                                                             h->strip_al)));
+              (n_instances == 1   ? least_n >= (h->rb ? 5 : 2)
+               : least_g >= 10000 ? true
+                                  : least_n >= 20 && (!rb2 || (o.n_u_it > 3 && fill >= 0.75 &&
+                                                               h->strip_al)));
       else if (P0.smem_mode)
         d64 = waves >= need;
     }
