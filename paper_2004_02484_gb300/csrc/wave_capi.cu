@@ -58,7 +58,6 @@ inline void derive(WInst& I) {
 struct WArgs {
   const WInst* inst;
   const int* act_of;  // [sum ng]: actuator index at the point, or -(grid steps to the nearest one)
-  const int* act_pt;  // [sum nu]: grid point of actuator a
   const double* x0;
   const double* wref;
   const double* uref;
@@ -370,7 +369,7 @@ struct nmpc_wave {
   long long n_a = 0, n_w = 0;  // sum n_u, sum n_g
   int ng_max = 0;
   WInst* inst_d = nullptr;
-  int *act_of = nullptr, *act_pt = nullptr;
+  int* act_of = nullptr;
   double *wref = nullptr, *uref = nullptr;
 };
 
@@ -378,7 +377,7 @@ namespace {
 
 void free_wave(nmpc_wave* h) {
   stage_drv::driver_free(h->drv);
-  void* ptrs[] = {h->inst_d, h->act_of, h->act_pt, h->wref, h->uref};
+  void* ptrs[] = {h->inst_d, h->act_of, h->wref, h->uref};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -405,7 +404,6 @@ WArgs make_args(const nmpc_wave* h) {
   WArgs A{};
   A.inst = h->inst_d;
   A.act_of = h->act_of;
-  A.act_pt = h->act_pt;
   A.x0 = h->drv.x0;
   A.wref = h->wref;
   A.uref = h->uref;
@@ -491,7 +489,7 @@ int nmpc_wave_setup(const nmpc_wave_desc* descs, int n, const nmpc_wave_opts* op
   nmpc_wave* h = new (std::nothrow) nmpc_wave();
   if (!h) return NMPC_ERR_CUDA;
   h->opts = o;
-  std::vector<int> act_of, act_pt;
+  std::vector<int> act_of;
   std::vector<stage_drv::GridKind> grid;
   long long n_pts = 0;
   for (int b = 0; b < n; ++b) {
@@ -521,7 +519,6 @@ int nmpc_wave_setup(const nmpc_wave_desc* descs, int n, const nmpc_wave_opts* op
     wave_dev::derive(I);
     const std::vector<int> ao = stage_drv::actuator_map(d.dim, d.m, d.n_u, d.act_cell);
     act_of.insert(act_of.end(), ao.begin(), ao.end());
-    for (int a = 0; a < d.n_u; ++a) act_pt.push_back(d.act_cell[a]);
     grid.push_back(stage_drv::GridKind{d.dim, d.m, I.ng, d.bc == 0});
     stage_drv::Layout L{};
     L.N = I.N;
@@ -539,12 +536,10 @@ int nmpc_wave_setup(const nmpc_wave_desc* descs, int n, const nmpc_wave_opts* op
   auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   A(stage_drv::dalloc(&h->inst_d, n));
   A(stage_drv::dalloc(&h->act_of, act_of.size()));
-  A(stage_drv::dalloc(&h->act_pt, act_pt.size()));
   A(stage_drv::dalloc(&h->wref, h->n_w));
   A(stage_drv::dalloc(&h->uref, h->n_a));
   A(stage_drv::upload(h->inst_d, h->inst_h));
   A(stage_drv::upload(h->act_of, act_of));
-  A(stage_drv::upload(h->act_pt, act_pt));
   if (e != cudaSuccess) {
     fprintf(stderr, "nmpc_wave_setup: %s\n", cudaGetErrorString(e));
     free_wave(h);
