@@ -169,6 +169,14 @@ struct Nbr {
 __device__ __forceinline__ float rcp(float v) { return __frcp_rn(v); }
 __device__ __forceinline__ double rcp(double v) { return __drcp_rn(v); }
 
+// b / d from r = 1 / d rounded: the product and its correction, one rounding as
+// in a division.
+template <typename T>
+__device__ __forceinline__ T quot(T b, T d, T r) {
+  const T q = b * r;
+  return fma(fma(-q, d, b), r, q);
+}
+
 // Bits of |v|: non-negative doubles order as integers, NaN above infinity, so
 // that a maximum costs the integer pipe and not the two-lane float64 one and
 // keeps a NaN.
