@@ -181,3 +181,37 @@ def test_residual_equals_the_cluster_path(G, size, n_lo):
         out.append(G.nmpc_residual(s.h, s.x0, s.ref, x, u, lam, s.n))
         s.close()
     assert np.abs(out[0] / out[1] - 1).max() <= 1e-12
+
+
+def _per_instance(insts, tensors):
+    cells = [i.horizon * i.mx * i.my for i in insts]
+    return list(zip(*(np.split(t.cpu().numpy(), np.cumsum(n)[:-1]) for t, n in
+                      zip(tensors, (cells, [i.horizon * len(i.act) for i in insts], cells)))))
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("rows", [0, 9])
+def test_every_instance_of_a_mixed_batch_follows_the_cluster_path(G, rows, variant):
+    """Odd and even widths, one and several strips a row, in one handle, cold and
+    then shifted by a stage, also with the strips' rows given: each instance's
+    count within one of the cluster path's and most of them equal, solutions
+    with equal counts within 1e-8, with others within a step at the tolerance
+    (1e-4 of the largest entry: the last step of a solve to 1e-7)."""
+    insts = [wl.heat2d(mx, my, 20, 2, 2, seed=300 + 10 * b + q, ref_amp=0.6 + 0.01 * b)
+             for b in range(10 * (1 + variant)) for q, (mx, my) in
+             enumerate([(63, 65), (64, 64), (130, 40), (77, 50)])]
+    sol, iters = [], []
+    for strips in (0, 2):
+        s = _solver(G, insts, strips, variant=variant, tol=1e-7, strip_rows=rows)
+        for init in (G.NMPC_INIT_COLD, G.NMPC_INIT_SHIFT):
+            rc, st = s.solve(init)
+            assert rc == G.NMPC_OK
+            iters.append(np.array([e.iters for e in st]))
+            sol.append(_per_instance(insts, s.state()))
+        s.close()
+    for q in (0, 1):
+        same = iters[q] == iters[q + 2]
+        assert np.abs(iters[q] - iters[q + 2]).max() <= 1 and same.mean() >= 0.75
+        for b in range(len(insts)):
+            for x, y in zip(sol[q][b], sol[q + 2][b]):
+                assert np.abs(x - y).max() <= (1e-8 if same[b] else 1e-4) * np.abs(y).max(), (q, b)
