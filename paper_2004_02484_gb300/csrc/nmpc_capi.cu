@@ -654,7 +654,8 @@ cudaError_t launch_strip(const nmpc_handle* h, const IterArgs& A, cudaStream_t s
   cfg.attrs = attr;
   cfg.numAttrs = (mode == nmpc_dev::MODE_SOLVE) ? 1 : 0;
   const TileKernel kern = h->strip_d64
-                              ? strip_d64_kernel(h->opts.n_lo, rb_half1(A, j), h->strip_fw, h->strip_al)
+                              ? strip_d64_kernel(h->opts.n_lo, rb_half1(A, j), h->strip_fw, h->strip_al,
+                                                 mode == nmpc_dev::MODE_ONESHOT && A.resid_only)
                               : strip_kernel<T>(h->opts.n_lo, rb_half1(A, j), h->strip2);
   return cudaLaunchKernelEx(&cfg, kern, A, mode, j);
 }
@@ -1766,10 +1767,10 @@ int nmpc_setup(const nmpc_desc* descs, int n_instances, const nmpc_opts* opts,
       h->n_tail_even = 0;
     }
     if (d64)
-      for (int rbn = 0; rbn < 2; ++rbn) {
+      for (int q = 0; q < 3; ++q) {
         const cudaError_t e2 = cudaFuncSetAttribute(
-            strip_d64_kernel(o.n_lo, rbn != 0, fw, h->strip_al), cudaFuncAttributeMaxDynamicSharedMemorySize,
-            max_optin);
+            strip_d64_kernel(o.n_lo, q == 1, fw, h->strip_al, q == 2),
+            cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
         if (e2 != cudaSuccess) {
           fprintf(stderr, "nmpc: kernel attribute: %s\n", cudaGetErrorString(e2));
           delete h;

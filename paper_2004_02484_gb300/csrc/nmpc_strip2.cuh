@@ -319,7 +319,7 @@ __device__ __forceinline__ void strip2_actuators(const IterArgs& A, const InstDe
 }
 
 template <int n_lo, bool FULL, bool RBN, bool GSN = false, bool D64 = false, bool FW = false,
-          bool AL = true>
+          bool AL = true, bool RO = false>
 __device__ __forceinline__ void strip2_body(const IterArgs& A,
                                             StripShared2<strip_ring_rows(n_lo), strip_fields(RBN)>& ws,
                                             int lane, int b, int s, int k, int rd, int x0, int y0,
@@ -455,18 +455,17 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
   Shift<F2, n_lo - 1> sk3, sax, sv1;
   Shift<F2, n_lo - 1> sv5, sw1;
 
-  // D64: a residual alone needs the own rows only, and no row after them (a
-  // strip of four own rows walks thirteen, ten of them with the float64 terms:
-  // 64x64, N = 50, one nmpc_residual 101 us, clusters 71, now 71 us)
-  const bool own_rows_only = D64 && full && resid_only;
-  const int steps = own_rows_only ? RH - E + 1 : RH + E;
+  // RO (a residual alone, FULL) needs the own rows only, and no row after them
+  // (a strip of four own rows walks thirteen, ten of them with the float64
+  // terms: 64x64, N = 50, one nmpc_residual 101 us, clusters 71, now 71 us)
+  const int steps = RO ? RH - E + 1 : RH + E;
   for (int j = 0; j < steps; ++j) {
     fetch(j + STRIP_AHEAD, STRIP_AHEAD);
     asm volatile("cp.async.wait_group %0;\n" ::"n"(STRIP_AHEAD));
     // ---- pass 0: row j ----
     {
       const double2 x = ld2(slot_at(0, RB_X)), l = ld2(slot_at(0, RB_L));
-      if (own_rows_only && j < E - 1) {
+      if (RO && j < E - 1) {
         // above the own rows' neighbours
       } else if constexpr (full) {
         phd.push(D2{k0d * (x.x + 0.5 * k1d * x.x * x.x), k0d * (x.y + 0.5 * k1d * x.y * x.y)});
@@ -523,7 +522,7 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
       const double2 x = ld2(rs + RB_X * 64), lam = ld2(rs + RB_L * 64);
       const double2 xp = ld2(qs + RS_XP * 64);
       F2 K1;
-      if (own_rows_only && rj < E) {
+      if (RO && rj < E) {
         K1 = F2{0.f, 0.f};
       } else if constexpr (full) {
         const double2 rc = ld2(qs + RS_RF * 64);
@@ -778,7 +777,9 @@ __device__ __forceinline__ void strip2_body(const IterArgs& A,
 // One upper-layer iteration over the strip work list with two columns per
 // lane (the strip list's x0 advance by 64 - 2 strip2_pad(n_lo)); control flow
 // as k_strip.
-template <int n_lo, bool RBN, bool D64 = false, bool FW = false, bool AL = true>
+// (RO: one-shot launches of nmpc_residual, a kernel of its own because the rows
+// it skips cost the solves' kernel registers)
+template <int n_lo, bool RBN, bool D64 = false, bool FW = false, bool AL = true, bool RO = false>
 __global__ void __launch_bounds__(STRIP2_WARPS * 32, STRIP2_MIN_BLOCKS)
     k_strip2(IterArgs A, int MODE, int j_launch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -816,6 +817,10 @@ __global__ void __launch_bounds__(STRIP2_WARPS * 32, STRIP2_MIN_BLOCKS)
   const int b = it.x, s = it.y, x0 = it.z, y0 = it.w;
   if (!stage_in_half(A, s, half)) return;
 
+  if constexpr (RO) {
+    strip2_body<n_lo, true, false, false, D64, FW, AL, true>(A, ws, lane, b, s, k, rd, x0, y0, sy, true);
+    return;
+  }
   bool resid_only, full;
   if (MODE == MODE_ONESHOT) {
     resid_only = (A.resid_only != 0);

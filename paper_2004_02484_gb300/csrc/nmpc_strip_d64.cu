@@ -10,16 +10,19 @@ namespace nmpc_dev {
 
 namespace {
 template <int n_lo, bool FW, bool AL>
-StripKernel half_of(bool rbn) {
+StripKernel pass_of(bool rbn, bool resid) {
+  if (resid) return nmpc_dev::k_strip2<n_lo, false, true, FW, AL, true>;
   return rbn ? nmpc_dev::k_strip2<n_lo, true, true, FW, AL> : nmpc_dev::k_strip2<n_lo, false, true, FW, AL>;
 }
 template <int n_lo>
-StripKernel shape_of(bool rbn, bool full_width, bool aligned) {
-  if (full_width) return aligned ? half_of<n_lo, true, true>(rbn) : half_of<n_lo, true, false>(rbn);
-  return aligned ? half_of<n_lo, false, true>(rbn) : half_of<n_lo, false, false>(rbn);
+StripKernel shape_of(bool rbn, bool full_width, bool aligned, bool resid) {
+  if (full_width)
+    return aligned ? pass_of<n_lo, true, true>(rbn, resid) : pass_of<n_lo, true, false>(rbn, resid);
+  return aligned ? pass_of<n_lo, false, true>(rbn, resid) : pass_of<n_lo, false, false>(rbn, resid);
 }
 }  // namespace
 
-StripKernel strip_d64_kernel(int n_lo, bool rbn, bool full_width, bool aligned) {
-  return n_lo <= 1 ? shape_of<1>(rbn, full_width, aligned) : shape_of<2>(rbn, full_width, aligned);
+StripKernel strip_d64_kernel(int n_lo, bool rbn, bool full_width, bool aligned, bool resid) {
+  return n_lo <= 1 ? shape_of<1>(rbn, full_width, aligned, resid)
+                   : shape_of<2>(rbn, full_width, aligned, resid);
 }
