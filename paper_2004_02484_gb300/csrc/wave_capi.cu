@@ -38,6 +38,7 @@ struct WInst {
   // b / a; gain / a; h^2 c lw / a; E's diagonal at W = 0 and its 3 h^2;
   // h gain / a; h r + gamma and 1 / that
   double ia, cl, kia, bia, gia, se, ed0, hh3, fu, auu, rauu;
+  float fauu, frauu;  // the last two in float32 (a conversion runs on the float64 pipe)
 };
 
 // The derived fields.
@@ -54,6 +55,8 @@ inline void derive(WInst& I) {
   I.fu = I.h * I.gia;
   I.auu = I.h * I.r + I.gamma;
   I.rauu = 1.0 / I.auu;
+  I.fauu = (float)I.auu;
+  I.frauu = 1.0f / I.fauu;
 }
 
 struct WArgs {
@@ -84,8 +87,10 @@ __host__ __device__ constexpr size_t stage_bytes(int ng) {
 // is taken on integers.  With n_lo = 2 the u-iterations after the first
 // recompute only the points that a control can reach (2 grid steps for v9):
 // all others keep the bits that they would get again.  256 membranes of
-// 32x32, N = 10, float64: 81.2 -> 25.9 ms a solve; 256 strings of 64 points,
-// N = 20, mixed, red-black: 21.3 -> 4.6 ms (with four stages a CTA).
+// 32x32, N = 10, float64: 81.0 -> 25.9 ms a solve (float64 pipe 85% busy; two
+// points a thread in 64 registers, 512 threads and two CTAs a SM, with 344 bytes
+// of spills); 256 strings of 64 points, N = 20, mixed, red-black: 21.2 -> 4.6 ms
+// (one point a thread, no spills, four stages a CTA, 76%).
 // The lower layer runs in T: float64, or float32 in mixed precision (the
 // residual, the coefficients and the update stay float64, so the fixed point
 // is the float64 root).
@@ -215,7 +220,8 @@ __global__ void __launch_bounds__(PPT == 1 ? 256 : 512, PPT == 1 ? 3 : 2)
   // v3, K_3): v3 = (K_2 - F_u^T y_lambda) / A_uu from v3 = 0, then the last y.
   // F_u = [0; h B / a]; A_uu = h r + gamma.
   const T hT = (T)h, clT = (T)cl, sT = (T)I.se, d2T = (T)d2, axv = (T)(h * I.qv);
-  const T fu = (T)I.fu, auu = (T)I.auu, rauu = (T)I.rauu;
+  const T fu = (T)I.fu;
+  const T auu = sizeof(T) == 4 ? I.fauu : I.auu, rauu = sizeof(T) == 4 ? I.frauu : I.rauu;
 #pragma unroll
   for (int j = 0; j < PPT; ++j)  // K1V + h grad_W g K1W
     r7[j] += hT * (clT * (nb[j].sum(fD) - d2T * k1w[j]) - kw3[j] * k1w[j]);
@@ -272,12 +278,14 @@ __global__ void __launch_bounds__(PPT == 1 ? 256 : 512, PPT == 1 ? 3 : 2)
 #pragma unroll
     for (int j = 0; j < PPT; ++j) {
       if (-ap[j] <= near2) v9[j] = c[j];
-      // (a corrected quotient: with the product alone the controls' rms error of
-      // an iteration was 1.1 to 1.25 times that of divisions; the diagonal's
-      // keeps the product, whose errors are those of a division)
-      if (itu < A.n_u_it && ap[j] >= 0)
-        sV3[g * MAX_NU + ap[j]] =
-            stage_drv::quot(sK2[g * MAX_NU + ap[j]] - fu * v9[j], auu, rauu);
+      // (the controls that are stored: a corrected quotient; with the product
+      // alone their rms error of an iteration was 1.1 to 1.25 times that of
+      // divisions.  The diagonal's keeps the product, whose errors are those of a
+      // division.)
+      if (itu < A.n_u_it && ap[j] >= 0) {
+        const T b = sK2[g * MAX_NU + ap[j]] - fu * v9[j];
+        sV3[g * MAX_NU + ap[j]] = itu == A.n_u_it - 1 ? stage_drv::quot(b, auu, rauu) : b * rauu;
+      }
     }
   }
   // v8 = h grad_W g^T v9 - b8, and S^{k+1} = S^k - (v5, v3, v4)
