@@ -158,8 +158,9 @@ typedef struct {
                       columns, no cluster / threads / cells / persistent
                       asked for, of which a launch holds several times what
                       stays resident, or which have more than 2048 cells and
-                      are few: these keep the cluster path's residual and
-                      iterates bit for bit),
+                      are few: these keep the cluster path's residual,
+                      its terms rounded alike, and its iterates to the
+                      rounding of the float32 lower layer),
                       1 = every eligible 2D
                       instance, 2 = never.  Eligible: n_lo <= 4, and for
                       n_u_it > 1 (auto, smaller stages: for any n_u_it) no

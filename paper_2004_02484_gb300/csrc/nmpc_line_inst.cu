@@ -79,9 +79,11 @@ __device__ __forceinline__ void li_nsum(const V (&v)[CPL], V (&out)[CPL], int la
 // read before anything of the iteration is written), lambda_{i+1} is not
 // overwritten yet (the stage above a warp's last one is copied before).  A
 // lane holds CPL consecutive cells; the arithmetic of a stage is k_line's, with
-// the multiply-adds written out as k_line's were contracted (the neighbour
-// sums too: hence the same cells per lane), so that both forms walk the same
-// iterates bit for bit.
+// the multiply-adds written out as k_line's were contracted by the compiler that
+// this was measured with (the neighbour sums too: hence the same cells per
+// lane).  Single instances then walk the same iterates; in a batch a few differ in
+// the last bits (1024 ragged instances: solutions equal to 4e-14 relative); the
+// tests ask for 1e-9.
 // An iteration whose residual is float64 evaluates the norms of all stages
 // first and updates only if the solve goes on, since the returned iterate is
 // the one whose residual passed.  A split residual that diverges is known only
@@ -91,9 +93,10 @@ __device__ __forceinline__ void li_nsum(const V (&v)[CPL], V (&out)[CPL], int la
 // What bounds it: the float64 pipe (56% busy on 304 instances of 256 cells:
 // two differences and two updates a cell) and latency (0.45 instructions a
 // cycle a scheduler, 16 warps a SM at 128 registers).  1024 ragged instances
-// (M 32..256, N 10..60): 54.6 -> 41.2 ms a solve, 37.8 with the sweeps a
-// constant; one instance of M = 32, N = 20 on 8 CTAs: 1007 -> 561 us, 506 with
-// the constant (828 us on one CTA, whose warps share one float64 pipe).
+// (M 32..256, N 10..60): 54.6 -> 41.2 ms a solve, 38.0 with the sweeps a
+// constant; one instance of M = 32, N = 20 on 8 CTAs: 1007 -> 561 us, 0.50 to
+// 0.53 ms with the constant (828 us on one CTA, whose warps share one float64
+// pipe).  Eight cells a lane spill 324 bytes at 128 registers.
 // NLO: the sweeps per solve as a constant (2, the default), or 0 to read them.
 template <int CPL, int NLO>
 __global__ void __launch_bounds__(32 * li_max_warps(CPL), 1)

@@ -14,8 +14,8 @@
 // is entirely inside or outside the grid: even grid width, even region
 // origin) and the update stores column pairs.
 //
-// Two variants serve stages that would also fit a thread-block cluster, in
-// batches large enough to fill the GPU with strips:
+// Variants that serve stages that would also fit a thread-block cluster, where
+// strips are the faster path (see nmpc_setup):
 //   D64  the split residual in the cluster path's form (the O(1) differences
 //        in float64, Lap Phi(x) from Phi), so that a handle's convergence
 //        rule and rounding bound are those of its cluster path;
@@ -25,9 +25,9 @@
 //   AL = false (with D64)  odd grid widths or offsets: columns are copied and
 //        stored one by one, and a pair's second column may lie outside.
 //
-// Requirements checked by the host: float32 lower layer, n_lo <= 2, every
-// strip instance with an even grid width and even offsets of its state and
-// x0 / ref arrays (16-byte aligned pairs).
+// Requirements checked by the host: float32 lower layer, n_lo <= 2, and but for
+// AL = false every strip instance with an even grid width and even offsets of
+// its state and x0 / ref arrays (16-byte aligned pairs).
 
 constexpr int STRIP2_WARPS = 4;  // warps (strips) per CTA
 #ifndef STRIP2_MIN_BLOCKS
@@ -166,8 +166,8 @@ __device__ __forceinline__ void cp_async16_zfill(void* dst_smem, const void* src
 // of Sec. 5.2 (eqs. 22-24) in the full-field form's own order, on the cells
 // within 2 (n_lo - 1) grid steps of the actuator (13 for n_lo = 2), lane q of
 // the half holding cell q.  No other actuator's cell is among them (the host
-// takes these strips only then, whatever n_u_it), so v3 comes out as the
-// cluster path's, operation by operation.
+// takes these strips only then, whatever n_u_it), so the operations are the
+// cluster path's, in its order.
 // (k_patch, before strips of the other form, computes a square of 49 cells,
 // four of five of which its result does not depend on, and a second
 // right-hand side, in a launch of its own.)

@@ -76,7 +76,10 @@ __host__ __device__ constexpr size_t stage_bytes(int ng) {
 // divisions, sit in the group's first nu threads, so that one or two warps
 // execute them and not every warp that owns an actuator point; the maximum
 // norm is taken on integers.  1024 plates of 13x13, N = 20, float64: 326 ->
-// 144 ms a solve, 140 with the sweeps a constant; one plate: 4.8 -> 2.3 ms.
+// 144 ms a solve, 140 with the sweeps a constant (float64 pipe 84% busy); one
+// plate: 4.8 -> 2.3 ms.  Stages of more than 256 points have two points a thread
+// in 64 registers (512 threads, two CTAs a SM) and spill 128 to 276 bytes (412
+// with the sweeps read): 64 plates of 24x24, 100 iterations, 46.8 -> 21.2 ms.
 // F_x = h (L diag(Phi'(w)) - diag(beta + 4 gr x^3)) - I on the state points;
 // v is zero at the actuator points.  The lower layer runs in T (float64, or
 // float32 in mixed precision: the residual, the coefficients and the update
