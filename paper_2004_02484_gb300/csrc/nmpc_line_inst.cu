@@ -633,11 +633,13 @@ std::vector<LineInstLaunch> line_inst_plan(const std::vector<InstDev>& inst,
     classes[{cpl, c, few}].push_back(b);
   }
   // Batch-form CTAs against one launch per iteration (us an iteration): a warp
-  // here takes t_stage for each of its stages, k_line t_wave for 16 stages a
-  // SM.  Few long instances leave SMs without a CTA and their warps with many
-  // stages: N = 66, one instance of 64 cells 28.9 against 10.1, N = 160, twelve
-  // of 32 cells 47 against 10.9; or the last wave of CTAs is nearly empty: 76 of
-  // 256 cells, N = 66, 46.6 against 43 (72: 26.7 against 34).
+  // here takes t_stage for each of its stages, k_line t_wave for 16 stages a SM.
+  // The slowest instance's float64 iterations, which walk the stages twice, come
+  // on top (a third with eight cells a lane and clusters, measured).  Few long
+  // instances leave SMs without a CTA and their warps with many stages: N = 66, one
+  // instance of 64 cells 28.9 against 10.1, N = 160, twelve of 32 cells 47 against
+  // 10.9, N = 65, 40 of 256 cells 34 against 29; or the last wave of CTAs is nearly
+  // empty: 76 of 256 cells, N = 66, 46.6 against 43 (72: 26.7 against 34).
   static const double t_stage[9] = {0, 2.3, 3.1, 0, 4.3, 0, 0, 0, 8.0};
   static const double t_wave[9] = {0, 8.5, 10, 0, 12, 0, 0, 0, 15.5};
   bool batch = false;
@@ -664,9 +666,11 @@ std::vector<LineInstLaunch> line_inst_plan(const std::vector<InstDev>& inst,
     const int sms = num_sms - (c > 2 ? num_sms / 19 : 0);
     const double t = (rows + L.warps - 1) / L.warps * t_stage[cpl];
     double waves = (double)L.n * c / (few ? sms : 2 * sms);
-    if (classes.size() == 1) waves = std::ceil(waves);
-    longest = std::max(longest, t);
-    work += waves * t;
+    // (CTAs of one length: 1.06, 1.4, 2.1 and 4.2 waves of them take 1.7, 1.8, 2.7
+    // and 4.7 times one; a slow instance prolongs a second wave that has begun)
+    if (classes.size() == 1) waves = waves > 1.0 ? waves + 0.55 : 1.0;
+    longest = std::max(longest, t * (cpl == 8 && c > 1 ? 1.35 : 1.1));
+    work += waves * t * (classes.size() == 1 && waves > 1.0 && waves < 2.0 ? 1.25 : 1.05);
     for (int b : v) {
       stages += inst[b].N;
       by_launches += inst[b].N * t_wave[cpl];

@@ -143,7 +143,7 @@ ROUTES = [(32, 60, 1, True), (64, 64, 1, True), (128, 33, 4, True), (256, 60, 4,
           (128, 40, 36, True), (32, 110, 44, True), (256, 60, 44, True), (64, 20, 100, True),
           (128, 110, 28, True), (256, 60, 100, True), (32, 66, 1, False), (64, 80, 4, False),
           (128, 110, 12, False), (32, 160, 20, False), (256, 160, 4, False), (256, 40, 44, False),
-          (256, 66, 76, False)]
+          (256, 66, 76, False), (256, 65, 40, False), (256, 40, 76, False)]
 
 
 @pytest.mark.parametrize("m,n,k,whole", ROUTES)
